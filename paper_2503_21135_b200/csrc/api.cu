@@ -35,7 +35,7 @@ bool front_fits(int T, int k);
 cudaError_t launch_front(const LayerDev* L, const WsDev& ws, const void* x, const float* logits, int E, int Es, int k,
                          int renorm, cudaStream_t st);
 cudaError_t launch_combine(const WsDev& ws, int d, int k, int Es, void* y, int y_f32, long long split_stride,
-                           cudaStream_t st);
+                           int n_experts, cudaStream_t st);
 cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
                               long long split_stride, int max_rows, int n_sms, int G, cudaStream_t st);
 cudaError_t setup_ffn_tc2(int n_sms, int* clusters_out);
@@ -76,15 +76,22 @@ struct ArenaLayout {
 
 struct WsLayout {
     size_t status, counts, offsets, off_pad, topk_idx, topk_w, perm, pos, row_token, row_expert, xperm, xsig,
-        hbuf, ypart,
+        hbuf, ypart, ysmall,
         stage_x, stage_logits, stage_y, stage_switch, total;
     std::vector<size_t> guards;  // offsets of the guard blocks
 };
 
 inline int s_pad_of(const dynamo_layer_desc& D) { return (D.max_sig + 15) / 16 * 16; }
+// Forwards whose partial results fit ypart for every K split; larger ones keep the splits of their small experts apart.
+inline bool decode_sized(const dynamo_layer_desc& D, int T) {
+    return (long long)T * (D.top_k + D.n_shared) <= DECODE_ROWS;
+}
+// K splits of the down GEMM on the streaming path.  One 256-row block of a Mixtral-shaped expert is a chain of 112
+// stages: a handful of small experts beside a 1000-token prompt took 107 us in 16 such chains per expert, 29 us in eight
+// times as many.  A split keeps four stages at least (a fine-grained expert has 11): an item pays about as much again
+// to start and to be added up.
 inline int ksplit_for(const dynamo_layer_desc& D, int T) {
-    const long long R = (long long)T * (D.top_k + D.n_shared);
-    return R <= DECODE_ROWS ? std::min(MAX_KSPLIT, D.d_ff / KC) : 1;
+    return std::max(1, std::min(MAX_KSPLIT, D.d_ff / KC / (decode_sized(D, T) ? 1 : 4)));
 }
 inline int switch_ints_per_layer(const dynamo_layer_desc& D) { return D.n_experts * (2 * s_pad_of(D) + 1); }
 
@@ -225,6 +232,7 @@ void ws_layout(const dynamo_layer_desc& D, WsLayout& W) {
     const size_t ks = std::min<size_t>(MAX_KSPLIT, f / KC);
     const size_t small_rows = std::min<size_t>(R, DECODE_ROWS);
     W.ypart = take(std::max(Rp, ks * (small_rows + 8 * n)) * d * 4);   // fp32 rows of the down GEMM, per K split
+    W.ysmall = R > DECODE_ROWS ? take((ks - 1) * n * TC_MIN_ROWS * d * 4) : W.ypart;   // (unused below that size)
     W.stage_x = take(T * d * 2);
     W.stage_logits = take(T * (size_t)D.n_experts * 4);
     W.stage_y = take(T * d * 4);
@@ -296,6 +304,7 @@ WsDev make_ws(const dynamo_ctx* c, int T) {
     w.xsig = (__half*)(b + c->W.xsig);
     w.hbuf = b + c->W.hbuf;
     w.ypart = (float*)(b + c->W.ypart);
+    w.ysmall = decode_sized(D, T) ? nullptr : (float*)(b + c->W.ysmall);
     w.status = (int32_t*)(b + c->W.status);
     w.T = T;
     w.R = T * (D.top_k + D.n_shared);
@@ -306,6 +315,11 @@ WsDev make_ws(const dynamo_ctx* c, int T) {
     // No expert can exceed T rows.  Up to twice the threshold the streaming kernel takes a large expert as
     // chunks of 24 tokens (the later passes over its blocks hit L2), which costs less than two more launches.
     w.tc_min = (c->tc_min_rows != 0x7fffffff && T > 2 * c->tc_min_rows) ? c->tc_min_rows : 0x7fffffff;
+    // The streaming path alone (no row limit per expert): its splits need whole copies of ypart.
+    if (w.tc_min == 0x7fffffff && w.ysmall) {
+        w.ysmall = nullptr;
+        w.ksplit = 1;
+    }
     w.h_bf16 = c->operand_dtype == DYNAMO_OPERAND_BF16;
     return w;
 }
@@ -788,7 +802,7 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         CUDA_TRY(launch_down_fix(L, (const DownDev*)ctx->down_arena, ws, D.d_model, st));
         ctx->launches += 1;
     }
-    CUDA_TRY(launch_combine(ws, D.d_model, D.top_k, D.n_shared, y, y_dtype == DYNAMO_F32, split_stride, st));
+    CUDA_TRY(launch_combine(ws, D.d_model, D.top_k, D.n_shared, y, y_dtype == DYNAMO_F32, split_stride, n, st));
     ctx->launches += (use_tc ? 8 : 6) - (fused_front ? 2 : 0);
     return forward_debug_copies(ctx, ws, T, dbg, st);
 }

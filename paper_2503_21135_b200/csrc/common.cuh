@@ -82,6 +82,8 @@ struct WsDev {
     __half* xsig;         // [R + pad][S_pad]
     uint8_t* hbuf;        // [R + pad][f/128][XROW]
     float* ypart;         // [ksplit][Rpad][d] fp32 rows of the down GEMM, one copy per K split
+    float* ysmall;        // forwards of many rows: K splits 1.. of the experts of the streaming path (their split 0 is in
+                          // ypart), [ksplit - 1][expert][32][d]; NULL in forwards whose ypart holds every split
     int32_t* status;      // device status word
     int32_t T, R, ksplit;
     // Physical rows: every expert's segment starts at a multiple of 8 rows (off_pad), so that the
@@ -102,6 +104,13 @@ struct WsDev {
 constexpr int TC_TILE_BYTES = 2048;
 constexpr int TC_RG_STRIDE = 8 * XROW;
 constexpr int TC_MIN_ROWS = 32;
+
+// Partial result of K split `split` for row `row` of expert e (first row off_e).
+__device__ __forceinline__ float* ypart_row(const WsDev& ws, int split, long long split_stride, int e, int n_experts,
+                                            int row, int off_e, int d) {
+    if (ws.ysmall == nullptr || split == 0) return ws.ypart + split * split_stride + (long long)row * d;
+    return ws.ysmall + (((long long)(split - 1) * n_experts + e) * TC_MIN_ROWS + row - off_e) * d;
+}
 
 // Activation buffers are CHUNK-MAJOR: the 128-k chunk kc of row r sits at (kc * Rcap + r) * XROW, so the
 // slice "rows r0 .. r0+n of chunk kc" that one pipeline stage needs is ONE contiguous bulk copy (many small

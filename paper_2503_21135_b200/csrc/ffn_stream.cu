@@ -329,8 +329,8 @@ __device__ __forceinline__ bool consume_item(const FfnParams& p, FfnSmem* S, uin
             if ((lane & 15) == 0) *reinterpret_cast<float*>(dst + XROW_SUM_OFF + (lane >> 4) * 4) = sum;
         }
     } else {
-        float* yb = p.ws.ypart + (size_t)im.split * p.split_stride;
         const int d = L->d;
+        float* yb = ypart_row(p.ws, im.split, p.split_stride, im.e, p.n_experts, im.row0, p.ws.off_pad[im.e], d);
 #pragma unroll
         for (int a = 0; a < APW; ++a)
 #pragma unroll
@@ -339,7 +339,7 @@ __device__ __forceinline__ bool consume_item(const FfnParams& p, FfnSmem* S, uin
                 for (int c = 0; c < 4; ++c) {
                     const int tok = 8 * j + 2 * tid4 + (c & 1);
                     const int n = im.rb * RB + (atom0 + a) * 16 + gid + ((c >> 1) ? 8 : 0);
-                    if (tok < im.nvalid) yb[(size_t)(im.row0 + tok) * d + n] = total[a][j][c];
+                    if (tok < im.nvalid) yb[(size_t)tok * d + n] = total[a][j][c];
                 }
     }
     return true;

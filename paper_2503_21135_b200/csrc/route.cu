@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(256) front_kernel(const LayerDev* __restrict__
 
 // grid (T, ceil(d / 1024)): each thread owns four output columns of one token.
 __global__ void __launch_bounds__(256) combine_kernel(WsDev ws, int d, int k, int Es, void* __restrict__ y,
-                                                      int y_f32, long long split_stride) {
+                                                      int y_f32, long long split_stride, int n_experts) {
     pdl_prologue();
     if (*ws.status & STATUS_TIMEOUT) return;  // the FFN kernels started nothing: leave y alone
     const int t = blockIdx.x;
@@ -506,9 +506,11 @@ __global__ void __launch_bounds__(256) combine_kernel(WsDev ws, int d, int k, in
         const int r = ws.pos[t * kk + j];
         const float w = (j < k) ? ws.topk_w[t * k + j] : 1.0f;
         float s[4] = {0.f, 0.f, 0.f, 0.f};
-        const int ns = (ws.counts[ws.row_expert[r]] > ws.tc_min) ? 1 : ws.ksplit;  // the tensor-core path does not split K
+        const int e = ws.row_expert[r];
+        const int ns = (ws.counts[e] > ws.tc_min) ? 1 : ws.ksplit;  // the tensor-core path does not split K
         for (int sp = 0; sp < ns; ++sp) {
-            const float4 v = *reinterpret_cast<const float4*>(ws.ypart + sp * split_stride + (long long)r * d + c);
+            const float4 v =
+                *reinterpret_cast<const float4*>(ypart_row(ws, sp, split_stride, e, n_experts, r, ws.off_pad[e], d) + c);
             s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
         }
 #pragma unroll
@@ -549,9 +551,9 @@ cudaError_t launch_front(const LayerDev* L, const WsDev& ws, const void* x, cons
                       Es, k, renorm);
 }
 cudaError_t launch_combine(const WsDev& ws, int d, int k, int Es, void* y, int y_f32, long long split_stride,
-                           cudaStream_t st) {
+                           int n_experts, cudaStream_t st) {
     return launch_pdl(combine_kernel, dim3((unsigned)ws.T, (unsigned)((d + 1023) / 1024)), dim3(256), 0, st, ws, d, k, Es,
-                      y, y_f32, split_stride);
+                      y, y_f32, split_stride, n_experts);
 }
 
 }  // namespace dyn

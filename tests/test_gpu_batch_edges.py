@@ -1,0 +1,52 @@
+"""GPU parity where the forward changes its path with the number of rows: every case against the oracle on a subset of
+its tokens, with the output tolerance of the other parity tests (max |gpu - oracle| / RMS <= 1e-2)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from helpers import make_gpu_layer, make_oracle_layer, rel_err
+from paper_2503_21135_b200 import binding
+from paper_2503_21135_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-2
+
+
+def _layer(max_tokens, **kw):
+    cfg = wl.scaled(wl.CONFIGS["tiny"], zipf=None, tokens=(max_tokens,), **kw)
+    wg, wu, wd = wl.layer_weights(cfg)
+    bits = np.array([[2, 3, 4, 8, 6][e % 5] for e in range(cfg.n_experts)] + [8] * cfg.n_shared, np.int32)
+    pool = wl.cache_pool(cfg)
+    gpu = make_gpu_layer(cfg, wg, wu, wd, bits, pool, max_tokens=max_tokens)
+    ora = make_oracle_layer(cfg, wg, wu, wd, bits)
+    sets = wl.initial_sig_sets(cfg, pool)
+    gpu.set_channel_switch(sets)
+    ora.set_channel_switch(sets)
+    return cfg, gpu, ora
+
+
+def _check(cfg, gpu, ora, x, lg, toks):
+    y = gpu.forward(x.cuda(), lg.cuda(), binding.F32)
+    torch.cuda.synchronize()
+    assert gpu.poll_status() == 0 and gpu.debug_check_guards() == 0
+    ref = ora.forward(oracle.as_u16(x), lg.numpy(), tokens=np.asarray(toks, np.int32))["y"][toks]
+    err = rel_err(y.cpu().numpy()[toks], ref)
+    assert err <= TOL, err
+    assert torch.equal(gpu.forward(x.cuda(), lg.cuda(), binding.F32), y)
+
+
+@pytest.mark.parametrize("group_size", [64, 128])
+def test_small_experts_beside_large_ones(group_size):
+    """More than 1024 rows: the K splits of small experts (at most 32 rows) leave the common buffer.  Row counts on
+    both sides of that limit and of the 8-row tiles, an empty expert, the rest on one large expert."""
+    counts = [32, 31, 33, 1, 0, 24, 9]
+    T = 1030 + sum(counts)
+    cfg, gpu, ora = _layer(T, n_experts=8, top_k=1, group_size=group_size)
+    e = np.concatenate([np.full(c, i) for i, c in enumerate(counts)] + [np.full(1030, 7)])
+    e = e[np.random.default_rng(3).permutation(T)]
+    lg = torch.zeros((T, 8))
+    lg[torch.arange(T), torch.from_numpy(e)] = 4.0
+    x = wl.activations(cfg, T, step=31)
+    toks = np.flatnonzero(e != 7)
+    _check(cfg, gpu, ora, x, lg, np.concatenate([toks, np.flatnonzero(e == 7)[:8]]))
