@@ -96,13 +96,13 @@ struct WsDev {
     int32_t h_bf16;       // 1: hidden activations are rounded to bf16 before they become the down GEMM's operand
 };
 
-// Activation layouts.  Both give a row group of 8 rows the same footprint (8 * XROW bytes per 128-k
-// chunk), so the two FFN paths can share one buffer:
-//   streaming path : row r, chunk c at (r * n_kc + c) * XROW: 128 fp16, then two fp32 sums.
-//   tcgen05 path   : row group rg, chunk c at (rg * n_kc + c) * 8 * XROW: the canonical K-major
-//                    no-swizzle MMA operand tile [k-octet 16][row 8][k 8] fp16 (2048 B).
+// Activation layouts, per expert segment (its rows start at a multiple of 8, off_pad) and 128-k chunk:
+//   streaming path : row r at act_off(chunk, r): 128 fp16, then two fp32 sums (288 bytes a row).
+//   tcgen05 path   : 8-row group g of the segment at tile_off(chunk, segment, g): the canonical K-major no-swizzle MMA
+//                    operand tile [k-octet 16][row 8][k 8] fp16.  The tiles of a segment follow one another without
+//                    the streaming rows' padding: the operand tiles are most of what the pair kernel reads, 7 TB/s of
+//                    L2 reads at 256 tokens a tile, and the pad was a ninth of it.
 constexpr int TC_TILE_BYTES = 2048;
-constexpr int TC_RG_STRIDE = 8 * XROW;
 constexpr int TC_MIN_ROWS = 32;
 
 // Partial result of K split `split` for row `row` of expert e (first row off_e).
@@ -117,6 +117,9 @@ __device__ __forceinline__ float* ypart_row(const WsDev& ws, int split, long lon
 // copies cost the copy engine about as much each as a large one).  Rcap = allocated rows.
 __host__ __device__ __forceinline__ size_t act_off(int kc, int row, int Rcap) {
     return ((size_t)kc * Rcap + row) * XROW;
+}
+__host__ __device__ __forceinline__ size_t tile_off(int kc, int seg_row0, int group, int Rcap) {
+    return act_off(kc, seg_row0, Rcap) + (size_t)group * TC_TILE_BYTES;
 }
 // Gathered activations of the cached ("pool") channels, 32 columns per group pq: (pq * Rcap + r) * 64 bytes.
 constexpr int POOL_GROUP = 32;               // cached channels per significant-channel pipeline stage

@@ -13,7 +13,7 @@
 //   warp 16 weights  : bulk copies of the CTA's half block (codes of atoms 8r..8r+7, params of rows 128r..) into a
 //                      ring of four small slots; a slot goes back as soon as the stage's warps hold its codes.
 //   warp 18 operands : bulk copy of ITS half of the token tile (N/2 tokens: the B operand is split across the
-//                      pair) into a ring of four 36 KB slots, freed by the MMAs' commit.  The operand copy is the long
+//                      pair) into a ring of four 32 KB slots, freed by the MMAs' commit.  The operand copy is the long
 //                      pole of a stage (2000-2800 cycles under load), so it gets the depth; the weights land on
 //                      their own barrier and are dequantized while the tile is still in flight.
 //   warps 0-15 dequant: a whole atom (16 rows x 128 k) of every OTHER stage each (eight warps per stage): packed
@@ -42,11 +42,11 @@ constexpr int T2_W_PROD = 16, T2_W_MMA = 17, T2_W_PRODX = 18;
 constexpr int T2_THREADS = 19 * 32;
 constexpr int T2_N = 256;                              // tokens per work item (128 per CTA)
 constexpr int T2_WHALF_MAX = 17408;                    // half of the largest packed block (8-bit, G = 64)
-constexpr int T2_XTILE = 16 * TC_RG_STRIDE;            // 128 tokens x 128 k: 16 row-group tiles at their buffer pitch
+constexpr int T2_XTILE = 16 * TC_TILE_BYTES;           // 128 tokens x 128 k: 16 row-group tiles
 constexpr int T2_POOL_TILES = POOL_GROUP * POOL_TILE_PITCH;       // cached-channel stage: 32 column tiles in a weight slot ...
 constexpr int T2_POOL_XG = 16 * 512;                              // ... and their operand tile of 16 row groups in an operand slot
 static_assert(T2_POOL_TILES <= T2_WHALF_MAX && T2_POOL_XG <= T2_XTILE, "cached-channel stage does not fit its slots");
-// Two rings of four slots.  The operand tiles (36 KB, read by the MMAs; their copy is the long pole of a stage at
+// Two rings of four slots.  The operand tiles (32 KB, read by the MMAs; their copy is the long pole of a stage at
 // 2000-2800 cycles under load) are freed by the MMAs' commit; the packed weights (read only by the dequant warps, at
 // the start of their visit) have small slots that are handed back as soon as the codes are in registers, so the
 // weights of a warp's next visit are already there when it comes back.  (Five operand + two weight slots measured
@@ -89,7 +89,8 @@ struct T2Item {
     const ExpertDev* ex;
     const uint8_t* wbase;  // first packed block of the item's row block
     int rb, n_valid, n_mma, row0, bits, blk_bytes, n_it;
-    int rg_mine0, n_rg_mine;  // this CTA's half of the token tile: first 8-row group and how many hold rows
+    int seg0;                 // first row of the expert's segment
+    int rg_mine0, n_rg_mine;  // this CTA's half of the token tile: first 8-row group of the segment, how many hold rows
 };
 
 template <bool GATEUP>
@@ -105,12 +106,13 @@ __device__ __forceinline__ T2Item t2_decode_item(const T2Params& p, const int* p
     T2Item it;
     it.rb = local / n_tt;
     it.n_valid = min(T2_N, cnt - tt * T2_N);
-    it.n_mma = (it.n_valid + 31) & ~31;  // N of the pair's MMA; each CTA holds N/2 token rows of B
     it.row0 = p.ws.off_pad[e] + tt * T2_N;
+    it.n_mma = (it.n_valid + 31) & ~31;  // N of the pair's MMA; each CTA holds N/2 token rows of B
     const int half = it.n_mma >> 1;
     const int nv_mine = max(0, min(half, it.n_valid - rank * half));
     it.n_rg_mine = (nv_mine + 7) >> 3;
-    it.rg_mine0 = (it.row0 + rank * half) >> 3;
+    it.seg0 = p.ws.off_pad[e];
+    it.rg_mine0 = (tt * T2_N + rank * half) >> 3;
     it.ex = &L->ex[e];
     it.bits = it.ex->bits;
     it.blk_bytes = it.ex->blk_bytes;
@@ -313,15 +315,15 @@ __global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p
                 if (!ok) break;
                 if (lane == 0) {
                     if (it < n_kc) {
-                        mbar_arrive_expect_tx(&B->fullx[s], (uint32_t)(w.n_rg_mine * TC_RG_STRIDE));
+                        mbar_arrive_expect_tx(&B->fullx[s], (uint32_t)(w.n_rg_mine * TC_TILE_BYTES));
                         if (w.n_rg_mine > 0)
-                            bulk_g2s(st, xbase + act_off(it, 8 * w.rg_mine0, p.ws.Rcap),
-                                     (uint32_t)(w.n_rg_mine * TC_RG_STRIDE), &B->fullx[s]);
+                            bulk_g2s(st, xbase + tile_off(it, w.seg0, w.rg_mine0, p.ws.Rcap),
+                                     (uint32_t)(w.n_rg_mine * TC_TILE_BYTES), &B->fullx[s]);
                     } else {
                         mbar_arrive_expect_tx(&B->fullx[s], (uint32_t)(w.n_rg_mine * 512));
                         if (w.n_rg_mine > 0)
                             bulk_g2s(st, reinterpret_cast<const uint8_t*>(p.ws.xsig) +
-                                             xpool_off(it - n_kc, 8 * w.rg_mine0, p.ws.Rcap),
+                                             xpool_off(it - n_kc, w.seg0 + 8 * w.rg_mine0, p.ws.Rcap),
                                      (uint32_t)(w.n_rg_mine * 512), &B->fullx[s]);
                     }
                 }
@@ -359,7 +361,7 @@ __global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p
                     const uint8_t* st = xring + (size_t)s * T2_XTILE;
                     const uint32_t a0 = tbase + T2_COL_A + 64 * b;
                     if (it < n_kc) {
-                        const uint64_t desc0 = tc_desc(smem_u32(st), 128, TC_RG_STRIDE);
+                        const uint64_t desc0 = tc_desc(smem_u32(st), 128, TC_TILE_BYTES);
 #pragma unroll
                         for (int k8 = 0; k8 < 8; ++k8)
                             tc2_mma_ts_elect(tbase, a0 + 8 * k8, desc0 + (uint64_t)(16 * k8), idesc, (it | k8) ? 1u : 0u);
@@ -488,8 +490,8 @@ __global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p
                             const int n = n0 + odd;                               // even gid stores token n0, odd gid n0 + 1
                             const __half2 pr = odd ? __floats2half2_rn(got, hs[1]) : __floats2half2_rn(hs[0], got);
                             if (n < w.n_valid) {
-                                uint8_t* dst = p.ws.hbuf + act_off(w.rb, (w.row0 + n) & ~7, p.ws.Rcap) + atom_g * 128 +
-                                               (n & 7) * 16 + (gid & ~1) * 2;
+                                uint8_t* dst = p.ws.hbuf + tile_off(w.rb, w.seg0, (w.row0 - w.seg0 + n) >> 3, p.ws.Rcap) +
+                                               atom_g * 128 + (n & 7) * 16 + (gid & ~1) * 2;
                                 *reinterpret_cast<__half2*>(dst) = pr;
                             }
                         } else {

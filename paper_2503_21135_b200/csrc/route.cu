@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(1024) scan_kernel(WsDev ws, int E, int Es, int
 // multiplied by 2^x_scale_exp(bits of the row's expert, k) so that the FFN kernels can use packed codes
 // in place; the per-group sums are of the unscaled fp16 values.
 __device__ __forceinline__ void gather_row(const LayerDev* __restrict__ L, const WsDev& ws,
-                                           const __nv_bfloat16* __restrict__ x, int row, int t, int e, bool tc) {
+                                           const __nv_bfloat16* __restrict__ x, int row, int t, int e, int seg0, bool tc) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (t < 0 && !tc) return;  // padding rows matter only as zero rows of an MMA operand tile
     const int d = L->d;
@@ -321,10 +321,8 @@ __device__ __forceinline__ void gather_row(const LayerDev* __restrict__ L, const
             *reinterpret_cast<uint2*>(out + lane * 8) = packed;
             if ((lane & 15) == 0) *reinterpret_cast<float*>(out + XROW_SUM_OFF + (lane >> 4) * 4) = sum;
         } else {
-            uint8_t* out = ws.xperm + act_off(c, 8 * rg, ws.Rcap);
+            uint8_t* out = ws.xperm + tile_off(c, seg0, (row - seg0) >> 3, ws.Rcap);
             *reinterpret_cast<uint2*>(out + (lane >> 1) * 128 + rr * 16 + (lane & 1) * 8) = packed;
-            // sums of the unscaled values per half chunk, beside the tile: [half 2][row 8] fp32
-            if ((lane & 15) == 0) *reinterpret_cast<float*>(out + TC_TILE_BYTES + ((lane >> 4) * 8 + rr) * 4) = sum;
         }
     }
     if (clamped && ws.status) atomicOr(ws.status, STATUS_RANGE);
@@ -367,7 +365,7 @@ __global__ void __launch_bounds__(256) gather_kernel(const LayerDev* __restrict_
     const int row = blockIdx.x;
     if (row >= ws.off_pad[L->E + L->Es]) return;
     const int e = ws.row_expert[row];
-    gather_row(L, ws, x, row, ws.row_token[row], e, ws.counts[e] > ws.tc_min);
+    gather_row(L, ws, x, row, ws.row_token[row], e, ws.off_pad[e], ws.counts[e] > ws.tc_min);
 }
 
 // Small batches: routing, permutation and gather in ONE launch (three launches cost more than their work when the
@@ -489,7 +487,7 @@ __global__ void __launch_bounds__(256) front_kernel(const LayerDev* __restrict__
     }
     __syncthreads();
     if (my_e < 0) return;
-    gather_row(L, ws, x, row, s_row_t, my_e, s_count[my_e] > ws.tc_min);
+    gather_row(L, ws, x, row, s_row_t, my_e, s_pad[my_e], s_count[my_e] > ws.tc_min);
 }
 
 // grid (T, ceil(d / 1024)): each thread owns four output columns of one token.
