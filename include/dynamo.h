@@ -221,9 +221,10 @@ dynamo_status dynamo_debug_check_guards(dynamo_ctx* ctx, int64_t* n_bad_bytes, v
 enum { DYNAMO_OPERAND_FP16 = 0, DYNAMO_OPERAND_BF16 = 1 };
 dynamo_status dynamo_set_operand_dtype(dynamo_ctx* ctx, int32_t operand_dtype);
 
-/* Path selection: experts that receive more than `rows` tokens in a forward run on the tcgen05
- * (tensor-memory) kernel, the others on the streaming kernel.  Default 32 (also the maximum);
- * 0 switches the tcgen05 path off.  Both paths implement the same arithmetic definition. */
+/* Path selection: experts that receive more than `rows` tokens in a forward run on the paired tcgen05 kernel, the
+ * others on the streaming kernel.  32 (the default and the maximum) also lets the library take one kernel for all
+ * experts of a middle-sized batch; 0 switches the tcgen05 kernels off.  All paths implement the same arithmetic
+ * definition. */
 dynamo_status dynamo_set_tc_min_rows(dynamo_ctx* ctx, int32_t rows);
 
 /* Precision the significant channels are served at (Section IV-B: once the original channels are back in place

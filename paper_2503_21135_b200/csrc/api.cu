@@ -38,6 +38,8 @@ cudaError_t launch_combine(const WsDev& ws, int d, int k, int Es, void* y, int y
                            int n_experts, cudaStream_t st);
 cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
                               long long split_stride, int max_rows, int n_sms, int G, cudaStream_t st);
+cudaError_t launch_ffn_fold(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
+                            long long split_stride, int n_sms, int G, cudaStream_t st);
 cudaError_t setup_ffn_tc2(int n_sms, int* clusters_out);
 cudaError_t launch_ffn_tc2(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int n_experts, int n_clusters,
                            cudaStream_t st);
@@ -92,6 +94,14 @@ inline bool decode_sized(const dynamo_layer_desc& D, int T) {
 // to start and to be added up.
 inline int ksplit_for(const dynamo_layer_desc& D, int T) {
     return std::max(1, std::min(MAX_KSPLIT, D.d_ff / KC / (decode_sized(D, T) ? 1 : 4)));
+}
+// Batches that take the fold kernel: more tokens than the streaming kernel serves alone, and few enough that most
+// experts have one 64-row tile (the codes are expanded once per tile).  Layer of eight experts, top-2, 4096 x 14336:
+// 65 tokens 249 us (streaming kernel 255), 100 tokens 269 (streaming and pair kernel 357), 139: 311 (523),
+// 200: 344 (465), 256 (64 rows an expert): 462 (468), 500: 671 (541).  Not with shared experts, whose rows are all the
+// tokens: the fine-grained layer at 128 tokens 240 us (176), at 300 260 (212).
+inline bool fold_sized(const dynamo_layer_desc& D, int T) {
+    return T > 2 * TC_MIN_ROWS && D.n_shared == 0 && (long long)T * D.top_k <= 62ll * D.n_experts;
 }
 inline int switch_ints_per_layer(const dynamo_layer_desc& D) { return D.n_experts * (2 * s_pad_of(D) + 1); }
 
@@ -315,6 +325,9 @@ WsDev make_ws(const dynamo_ctx* c, int T) {
     // No expert can exceed T rows.  Up to twice the threshold the streaming kernel takes a large expert as
     // chunks of 24 tokens (the later passes over its blocks hit L2), which costs less than two more launches.
     w.tc_min = (c->tc_min_rows != 0x7fffffff && T > 2 * c->tc_min_rows) ? c->tc_min_rows : 0x7fffffff;
+    // Middle-sized batches: one kernel for all experts (see fold_sized).
+    w.fold = c->tc_min_rows == TC_MIN_ROWS && fold_sized(D, T);
+    if (w.fold) w.tc_min = 0x7fffffff;
     // The streaming path alone (no row limit per expert): its splits need whole copies of ypart.
     if (w.tc_min == 0x7fffffff && w.ysmall) {
         w.ysmall = nullptr;
@@ -789,14 +802,20 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
     const bool use_tc = ws.tc_min != 0x7fffffff;                  // experts above 32 rows take the tcgen05 path
     const long long split_stride = (long long)ws.Rpad * D.d_model;  // partials of one K split: [Rpad][d]
     if (ctx->prof_ev[0]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[0], st));
-    const int max_rows = use_tc ? std::min(T, ctx->tc_min_rows) : T;  // rows one expert can have on the streaming path
-    CUDA_TRY(launch_ffn_stream(L, ws, 1, ctx->host_layer.n_rb13, 1, n, split_stride, max_rows, ctx->n_sms,
-                               D.group_size, st));
-    if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, ctx->host_layer.n_rb13, n, ctx->tc2_clusters[1], st));
-    if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
-    CUDA_TRY(launch_ffn_stream(L, ws, 0, ctx->host_layer.n_rb2, ws.ksplit, n, split_stride, max_rows, ctx->n_sms,
-                               D.group_size, st));
-    if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, ctx->host_layer.n_rb2, n, ctx->tc2_clusters[0], st));
+    if (ws.fold) {
+        CUDA_TRY(launch_ffn_fold(L, ws, 1, ctx->host_layer.n_rb13, 1, n, split_stride, ctx->n_sms, D.group_size, st));
+        if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
+        CUDA_TRY(launch_ffn_fold(L, ws, 0, ctx->host_layer.n_rb2, ws.ksplit, n, split_stride, ctx->n_sms, D.group_size, st));
+    } else {
+        const int max_rows = use_tc ? std::min(T, ctx->tc_min_rows) : T;  // rows one expert can have on the streaming path
+        CUDA_TRY(launch_ffn_stream(L, ws, 1, ctx->host_layer.n_rb13, 1, n, split_stride, max_rows, ctx->n_sms,
+                                   D.group_size, st));
+        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, ctx->host_layer.n_rb13, n, ctx->tc2_clusters[1], st));
+        if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
+        CUDA_TRY(launch_ffn_stream(L, ws, 0, ctx->host_layer.n_rb2, ws.ksplit, n, split_stride, max_rows, ctx->n_sms,
+                                   D.group_size, st));
+        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, ctx->host_layer.n_rb2, n, ctx->tc2_clusters[0], st));
+    }
     if (ctx->prof_ev[2]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[2], st));
     if (ctx->down_active) {  // significant hidden units: add what their 8-bit columns of W_down change
         CUDA_TRY(launch_down_fix(L, (const DownDev*)ctx->down_arena, ws, D.d_model, st));

@@ -92,6 +92,7 @@ struct WsDev {
     int32_t* off_pad;     // [E_tot + 1]
     int32_t Rpad;
     int32_t Rcap;         // rows allocated in the activation buffers (their chunk pitch)
+    int32_t fold;         // 1: every expert takes the fold kernel (operand tiles with their group sums)
     int32_t tc_min;       // experts with more rows than this take the tcgen05 path (INT_MAX: none)
     int32_t h_bf16;       // 1: hidden activations are rounded to bf16 before they become the down GEMM's operand
 };
@@ -102,6 +103,8 @@ struct WsDev {
 //                    operand tile [k-octet 16][row 8][k 8] fp16.  The tiles of a segment follow one another without
 //                    the streaming rows' padding: the operand tiles are most of what the pair kernel reads, 7 TB/s of
 //                    L2 reads at 256 tokens a tile, and the pad was a ninth of it.
+//   fold kernel    : 8-row group g at act_off(chunk, 8 g): such a tile, then [group][row 8] fp32 sums of its rows per
+//                    quantization group.
 constexpr int TC_TILE_BYTES = 2048;
 constexpr int TC_MIN_ROWS = 32;
 

@@ -271,10 +271,12 @@ __global__ void __launch_bounds__(1024) scan_kernel(WsDev ws, int E, int Es, int
 // combine kernel measured no gain either.)  The fp16 activations are stored
 // multiplied by 2^x_scale_exp(bits of the row's expert, k) so that the FFN kernels can use packed codes
 // in place; the per-group sums are of the unscaled fp16 values.
+enum : int { LAY_ROWS, LAY_TILES, LAY_FOLD };   // which kernel reads the row: streaming, pair, fold
 __device__ __forceinline__ void gather_row(const LayerDev* __restrict__ L, const WsDev& ws,
-                                           const __nv_bfloat16* __restrict__ x, int row, int t, int e, int seg0, bool tc) {
+                                           const __nv_bfloat16* __restrict__ x, int row, int t, int e, int seg0, int lay) {
+    const bool tc = lay != LAY_ROWS;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (t < 0 && !tc) return;  // padding rows matter only as zero rows of an MMA operand tile
+    if (t < 0 && lay != LAY_TILES) return;  // padding rows matter only as zero rows of an MMA operand tile
     const int d = L->d;
     const int n_kc = d / KC;
     const int bits = L->ex[e].bits;
@@ -321,8 +323,13 @@ __device__ __forceinline__ void gather_row(const LayerDev* __restrict__ L, const
             *reinterpret_cast<uint2*>(out + lane * 8) = packed;
             if ((lane & 15) == 0) *reinterpret_cast<float*>(out + XROW_SUM_OFF + (lane >> 4) * 4) = sum;
         } else {
-            uint8_t* out = ws.xperm + tile_off(c, seg0, (row - seg0) >> 3, ws.Rcap);
+            uint8_t* out = ws.xperm + (lay == LAY_FOLD ? act_off(c, 8 * rg, ws.Rcap)
+                                                       : tile_off(c, seg0, (row - seg0) >> 3, ws.Rcap));
             *reinterpret_cast<uint2*>(out + (lane >> 1) * 128 + rr * 16 + (lane & 1) * 8) = packed;
+            if (lay == LAY_FOLD) {   // sums of the unscaled values per quantization group: [group][row 8] fp32
+                if (L->G == 128) sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+                if ((lane & 15) == 0) *reinterpret_cast<float*>(out + TC_TILE_BYTES + ((lane >> 4) * 8 + rr) * 4) = sum;
+            }
         }
     }
     if (clamped && ws.status) atomicOr(ws.status, STATUS_RANGE);
@@ -365,7 +372,7 @@ __global__ void __launch_bounds__(256) gather_kernel(const LayerDev* __restrict_
     const int row = blockIdx.x;
     if (row >= ws.off_pad[L->E + L->Es]) return;
     const int e = ws.row_expert[row];
-    gather_row(L, ws, x, row, ws.row_token[row], e, ws.off_pad[e], ws.counts[e] > ws.tc_min);
+    gather_row(L, ws, x, row, ws.row_token[row], e, ws.off_pad[e], ws.fold ? LAY_FOLD : (ws.counts[e] > ws.tc_min ? LAY_TILES : LAY_ROWS));
 }
 
 // Small batches: routing, permutation and gather in ONE launch (three launches cost more than their work when the
@@ -487,7 +494,8 @@ __global__ void __launch_bounds__(256) front_kernel(const LayerDev* __restrict__
     }
     __syncthreads();
     if (my_e < 0) return;
-    gather_row(L, ws, x, row, s_row_t, my_e, s_pad[my_e], s_count[my_e] > ws.tc_min);
+    gather_row(L, ws, x, row, s_row_t, my_e, s_pad[my_e],
+               ws.fold ? LAY_FOLD : (s_count[my_e] > ws.tc_min ? LAY_TILES : LAY_ROWS));
 }
 
 // grid (T, ceil(d / 1024)): each thread owns four output columns of one token.

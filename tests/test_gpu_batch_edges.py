@@ -50,3 +50,31 @@ def test_small_experts_beside_large_ones(group_size):
     x = wl.activations(cfg, T, step=31)
     toks = np.flatnonzero(e != 7)
     _check(cfg, gpu, ora, x, lg, np.concatenate([toks, np.flatnonzero(e == 7)[:8]]))
+
+
+@pytest.mark.parametrize("group_size", [64, 128])
+@pytest.mark.parametrize("down", [False, True])
+def test_middle_sized_batches(group_size, down):
+    """One kernel for all experts: row counts around its tiles (16 columns an MMA, 64 rows a pass), every bit-width, an
+    empty expert; with and without significant hidden units (they read h in this kernel's layout)."""
+    counts = [64, 65, 16, 17, 1, 0, 48, 129]
+    T = sum(counts)
+    cfg, gpu, ora = _layer(T, n_experts=8, top_k=1, group_size=group_size)
+    if down:
+        wd = wl.layer_weights(cfg)[2]
+        pool_d = wl.cache_pool_down(cfg, 32)
+        sets_d = wl.sig_sets_down(cfg, pool_d, 16)
+        gpu.pack_down_cache(wd.cuda(), np.array([[2, 3, 4, 8, 6][e % 5] for e in range(8)], np.int32), pool_d, 16)
+        ora.enable_down_side(oracle.as_u16(wd))
+        gpu.set_channel_switch_down(sets_d)
+        ora.set_channel_switch_down(sets_d)
+    e = np.concatenate([np.full(c, i) for i, c in enumerate(counts)])[np.random.default_rng(4).permutation(T)]
+    lg = torch.zeros((T, 8))
+    lg[torch.arange(T), torch.from_numpy(e)] = 4.0
+    _check(cfg, gpu, ora, wl.activations(cfg, T, step=32), lg, np.arange(T))
+
+
+@pytest.mark.parametrize("T", [65, 96, 247, 248, 249])
+def test_both_ends_of_the_middle_sizes(T):
+    cfg, gpu, ora = _layer(256, n_experts=8, top_k=2, group_size=128)
+    _check(cfg, gpu, ora, wl.activations(cfg, T, step=33), wl.router_logits(cfg, T, step=33), np.arange(T))
