@@ -9,60 +9,89 @@
 //           plus the gathered significant columns; written in the layout of the FFN path the row's
 //           expert takes (streaming rows, or 8-row MMA operand tiles).
 // combine : y[t] = sum_j w[t,j] * Y[pos(t,j)] + sum_shared Y[pos], fp32, fixed order.
+#include <type_traits>
+
 #include "common.cuh"
 #include "layout.cuh"
 
 namespace dyn {
 
-// Top-k of one token's logits held across a warp (lane l holds logits l, l+32, ...; E <= 256): k largest raw
-// logits, descending, ties -> lower expert index; weights = softmax over all E restricted to the chosen,
-// rescaled to sum 1 if `renorm`.
-__device__ __forceinline__ void topk_softmax_store(float (&v)[8], int lane, int E, int k, int renorm, long long token,
+// Order-preserving map of a float to an unsigned integer (-0 counts as +0) and back.
+__device__ __forceinline__ uint32_t order_key(float v) {
+    const uint32_t b = __float_as_uint(v + 0.f);
+    return b ^ ((b >> 31) ? 0xffffffffu : 0x80000000u);
+}
+__device__ __forceinline__ float order_value(uint32_t k) {
+    return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xffffffffu));
+}
+
+// Top-k of one token's logits held across a warp (lane l holds logits l, l+32, ..., NV of them; E <= 32 NV): k largest
+// raw logits, descending, ties -> lower expert index; weights = softmax over all E restricted to the chosen,
+// rescaled to sum 1 if `renorm`.  A round of the selection is two warp reductions in hardware (with ten shuffles and
+// eight candidates a lane whatever E is, the front kernel took 24.5 us at 16 tokens, 64 experts, top-6; now 13.6).
+template <int NV>
+__device__ __forceinline__ void topk_softmax_store(float (&v)[NV], int lane, int E, int k, int renorm, long long token,
                                                    int32_t* __restrict__ topk_idx, float* __restrict__ topk_w) {
     float mx = -INFINITY;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) mx = fmaxf(mx, v[i]);
+    for (int i = 0; i < NV; ++i) mx = fmaxf(mx, v[i]);
 #pragma unroll
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     float den = 0.f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < NV; ++i)
         if (lane + 32 * i < E) den += expf(v[i] - mx);
 #pragma unroll
     for (int o = 16; o; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
 
-    float wsel[8];
-    int isel[8];
-    float wsum = 0.f;
+    float my_w = 0.f, wsum = 0.f;   // lane j keeps the j-th choice
+    int my_i = 0;
     for (int j = 0; j < k; ++j) {
         // local best (value desc, index asc)
         float bv = -INFINITY;
         int bi = 0x7fffffff;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < NV; ++i) {
             const int e = lane + 32 * i;
             if (e < E && (v[i] > bv || (v[i] == bv && e < bi))) { bv = v[i]; bi = e; }
         }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-        }
+        const uint32_t key = order_key(bv), best = __reduce_max_sync(0xffffffffu, key);
+        bi = (int)__reduce_min_sync(0xffffffffu, key == best ? (uint32_t)bi : 0x7fffffffu);
         // remove the winner from its owner's candidates
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < NV; ++i)
             if (lane + 32 * i == bi) v[i] = -INFINITY;
-        isel[j] = bi;
-        wsel[j] = expf(bv - mx) / den;
-        wsum += wsel[j];
-    }
-    if (lane == 0) {
-        for (int j = 0; j < k; ++j) {
-            topk_idx[token * k + j] = isel[j];
-            topk_w[token * k + j] = renorm ? wsel[j] / wsum : wsel[j];
+        const float w = expf(order_value(best) - mx) / den;
+        if (lane == j) {
+            my_i = bi;
+            my_w = w;
         }
+        wsum += w;
     }
+    if (lane < k) {
+        topk_idx[token * k + lane] = my_i;
+        topk_w[token * k + lane] = renorm ? my_w / wsum : my_w;
+    }
+}
+
+// Logits l[0 .. E) of one token into a warp's registers, then the selection.
+template <int NV>
+__device__ __forceinline__ void topk_from_memory(const float* __restrict__ l, int lane, int E, int k, int renorm,
+                                                 long long token, int32_t* __restrict__ topk_idx,
+                                                 float* __restrict__ topk_w) {
+    float v[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+        const int e = lane + 32 * i;
+        v[i] = (e < E) ? l[e] : -INFINITY;
+    }
+    topk_softmax_store<NV>(v, lane, E, k, renorm, token, topk_idx, topk_w);
+}
+__device__ __forceinline__ void topk_token(const float* __restrict__ l, int lane, int E, int k, int renorm, long long token,
+                                           int32_t* __restrict__ topk_idx, float* __restrict__ topk_w) {
+    if (E <= 32) topk_from_memory<1>(l, lane, E, k, renorm, token, topk_idx, topk_w);
+    else if (E <= 64) topk_from_memory<2>(l, lane, E, k, renorm, token, topk_idx, topk_w);
+    else topk_from_memory<8>(l, lane, E, k, renorm, token, topk_idx, topk_w);
 }
 
 // One warp per token.
@@ -71,80 +100,134 @@ __global__ void __launch_bounds__(256) route_kernel(const float* __restrict__ lo
     pdl_prologue();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp >= T) return;
-    const float* l = logits + (long long)warp * E;
-    float v[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int e = lane + 32 * i;
-        v[i] = (e < E) ? l[e] : -INFINITY;
-    }
-    topk_softmax_store(v, lane, E, k, renorm, warp, topk_idx, topk_w);
+    topk_token(logits + (long long)warp * E, lane, E, k, renorm, warp, topk_idx, topk_w);
 }
 
 // Router GEMM fused with the top-k (Section II-A: the gate scores every expert, the K best are taken):
-// logits[t][e] = sum_c x[t][c] * W_r[e][c] (+ bias[e]), bf16 inputs, fp32 accumulate.  One CTA of eight warps
-// per token: warp w, lane l take the input indices 8*l + 256*(w + 8*i) ..+7; every warp reduces its partial
-// sums over its lanes by a fixed butterfly, the eight partials are added in warp order, so the sum order
-// (hence the fp32 result) is deterministic.  The products of two bf16 values are exact in fp32; only the
-// additions round.  Warp 0 then selects the top-k exactly as route_kernel does.
+// logits[t][e] = sum_c x[t][c] * W_r[e][c] (+ bias[e]), bf16 inputs, fp32 accumulate.  One CTA of eight warps per TB
+// tokens, which share the loads and the conversion of the router's weights: warp w, lane l take the input indices
+// 8*l + 256*(w + 8*i) ..+7, eight experts at a time, the next eight rows of weights on their way meanwhile.  Every warp
+// reduces its partial sums over its lanes in the butterfly order (offsets 16, 8, 4, 2, 1), the eight partials are added
+// in warp order, so the sum order (hence the fp32 result) is deterministic.  The eight sums of a token are reduced
+// together, a lane keeping half of them at each of the first three steps: 9 shuffles instead of 40, the same additions.
+// Warp t then selects the top-k of the CTA's token t exactly as route_kernel does.
+// 300 tokens, 64 experts, d = 2048: 21.7 us; 37 us with one token per CTA, one expert's shuffles after another and no
+// loads ahead.
+template <int TB>
 __global__ void __launch_bounds__(256) route_gemm_kernel(const __nv_bfloat16* __restrict__ x,
                                                          const __nv_bfloat16* __restrict__ w_router,
                                                          const float* __restrict__ bias, int T, int d, int E, int k,
                                                          int renorm, float* __restrict__ logits_out,
                                                          int32_t* __restrict__ topk_idx, float* __restrict__ topk_w) {
-    __shared__ float part[8][MAX_EXPERTS];
+    __shared__ float part[TB][8][MAX_EXPERTS];
     pdl_prologue();
-    const int token = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const __nv_bfloat16* xr = x + (long long)token * d;
-    for (int e0 = 0; e0 < E; e0 += 8) {  // eight experts at a time
-        float acc[8];
+    const int t0 = blockIdx.x * TB, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int c0 = 8 * lane + 256 * warp;
+    const int n_c = c0 < d ? (d - c0 + 2047) / 2048 : 0;    // this lane's runs of eight input indices
+    const int n_cw = (d - 256 * warp + 2047) / 2048;        // the warp's (uniform; some lanes may have one less)
+    uint4 wv[8];
+    auto load_w = [&](int e0, int i) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[j] = 0.f;
-        for (int c = 8 * lane + 256 * warp; c < d; c += 2048) {
-            const uint4 xv = *reinterpret_cast<const uint4*>(xr + c);
-            const __nv_bfloat162* xp = reinterpret_cast<const __nv_bfloat162*>(&xv);
-            float xf[8];
+        for (int j = 0; j < 8; ++j)
+            wv[j] = (i < n_c && e0 + j < E)
+                        ? *reinterpret_cast<const uint4*>(w_router + (long long)(e0 + j) * d + c0 + 2048 * i)
+                        : make_uint4(0u, 0u, 0u, 0u);
+    };
+    if (n_cw > 0) {
+        load_w(0, 0);
+        for (int e0 = 0; e0 < E; e0 += 8) {  // eight experts at a time
+            float acc[TB][8];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                xf[2 * u] = __low2float(xp[u]);
-                xf[2 * u + 1] = __high2float(xp[u]);
-            }
+            for (int t = 0; t < TB; ++t)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (e0 + j < E) {
-                    const uint4 wv = *reinterpret_cast<const uint4*>(w_router + (long long)(e0 + j) * d + c);
-                    const __nv_bfloat162* wp = reinterpret_cast<const __nv_bfloat162*>(&wv);
+                for (int j = 0; j < 8; ++j) acc[t][j] = 0.f;
+            for (int i = 0; i < n_cw; ++i) {
+                uint4 cur[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) cur[j] = wv[j];
+                if (i + 1 < n_cw) load_w(e0, i + 1);
+                else if (e0 + 8 < E) load_w(e0 + 8, 0);
+                float xf[TB][8];
+#pragma unroll
+                for (int t = 0; t < TB; ++t) {
+                    uint4 xv = make_uint4(0u, 0u, 0u, 0u);
+                    if (i < n_c && t0 + t < T) xv = *reinterpret_cast<const uint4*>(x + (long long)(t0 + t) * d + c0 + 2048 * i);
+                    const __nv_bfloat162* xp = reinterpret_cast<const __nv_bfloat162*>(&xv);
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        acc[j] = fmaf(xf[2 * u], __low2float(wp[u]), acc[j]);
-                        acc[j] = fmaf(xf[2 * u + 1], __high2float(wp[u]), acc[j]);
+                        xf[t][2 * u] = __low2float(xp[u]);
+                        xf[t][2 * u + 1] = __high2float(xp[u]);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const __nv_bfloat162* wp = reinterpret_cast<const __nv_bfloat162*>(&cur[j]);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const float wl = __low2float(wp[u]), wh = __high2float(wp[u]);
+#pragma unroll
+                        for (int t = 0; t < TB; ++t) {
+                            acc[t][j] = fmaf(xf[t][2 * u], wl, acc[t][j]);
+                            acc[t][j] = fmaf(xf[t][2 * u + 1], wh, acc[t][j]);
+                        }
                     }
                 }
             }
-        }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+            for (int t = 0; t < TB; ++t) {
+                // after the steps 16, 8, 4 a lane holds the sum of expert e0 + 4 b4 + 2 b3 + b2 (its lane bits)
+                float s4[4], s2[2], s1;
 #pragma unroll
-            for (int o = 16; o; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-            if (lane == 0 && e0 + j < E) part[warp][e0 + j] = acc[j];
+                for (int j = 0; j < 4; ++j) {
+                    const bool up = (lane & 16) != 0;
+                    const float keep = up ? acc[t][j + 4] : acc[t][j], give = up ? acc[t][j] : acc[t][j + 4];
+                    s4[j] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const bool up = (lane & 8) != 0;
+                    const float keep = up ? s4[j + 2] : s4[j], give = up ? s4[j] : s4[j + 2];
+                    s2[j] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+                }
+                {
+                    const bool up = (lane & 4) != 0;
+                    const float keep = up ? s2[1] : s2[0], give = up ? s2[0] : s2[1];
+                    s1 = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+                }
+                s1 += __shfl_xor_sync(0xffffffffu, s1, 2);
+                s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
+                const int e = e0 + ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+                if ((lane & 3) == 0 && e < E) part[t][warp][e] = s1;
+            }
         }
+    } else {
+        for (int e = lane; e < E; e += 32)
+#pragma unroll
+            for (int t = 0; t < TB; ++t) part[t][warp][e] = 0.f;
     }
     __syncthreads();
-    if (warp != 0) return;
-    float v[8];
+    const int token = t0 + warp;
+    if (warp >= TB || token >= T) return;
+    auto select = [&](auto nvc) {
+        constexpr int NV = decltype(nvc)::value;
+        float v[NV];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int e = lane + 32 * i;
-        v[i] = -INFINITY;
-        if (e < E) {
-            float sum = part[0][e];
+        for (int i = 0; i < NV; ++i) {
+            const int e = lane + 32 * i;
+            v[i] = -INFINITY;
+            if (e < E) {
+                float sum = part[warp][0][e];
 #pragma unroll
-            for (int w = 1; w < 8; ++w) sum += part[w][e];
-            v[i] = sum + (bias ? bias[e] : 0.f);
-            if (logits_out) logits_out[(long long)token * E + e] = v[i];
+                for (int w = 1; w < 8; ++w) sum += part[warp][w][e];
+                v[i] = sum + (bias ? bias[e] : 0.f);
+                if (logits_out) logits_out[(long long)token * E + e] = v[i];
+            }
         }
-    }
-    topk_softmax_store(v, lane, E, k, renorm, token, topk_idx, topk_w);
+        topk_softmax_store<NV>(v, lane, E, k, renorm, token, topk_idx, topk_w);
+    };
+    if (E <= 32) select(std::integral_constant<int, 1>{});
+    else if (E <= 64) select(std::integral_constant<int, 2>{});
+    else select(std::integral_constant<int, 8>{});
 }
 
 // Single CTA of 32 warps.  The pair array (pair i = t*k + j, ascending in t) is cut into 32 contiguous
@@ -392,16 +475,7 @@ __global__ void __launch_bounds__(256) front_kernel(const LayerDev* __restrict__
     pdl_prologue();
     const int T = ws.T, n_pairs = T * k, kk = k + Es;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int t = warp; t < T; t += 8) {
-        const float* l = logits + (long long)t * E;
-        float v[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int e = lane + 32 * i;
-            v[i] = (e < E) ? l[e] : -INFINITY;
-        }
-        topk_softmax_store(v, lane, E, k, renorm, t, s_idx, s_w);
-    }
+    for (int t = warp; t < T; t += 8) topk_token(logits + (long long)t * E, lane, E, k, renorm, t, s_idx, s_w);
     if (threadIdx.x == 0) { s_row_e = -1; s_row_t = -1; }
     __syncthreads();
     // counting sort: thread e walks the pairs in order (pair i = t*k + j ascends in t: the stable order)
@@ -539,7 +613,11 @@ cudaError_t launch_route(const float* logits, int T, int E, int k, int renorm, i
 }
 cudaError_t launch_route_gemm(const void* x, const void* w_router, const float* bias, int T, int d, int E, int k,
                               int renorm, float* logits_out, int32_t* idx, float* w, cudaStream_t st) {
-    return launch_pdl(route_gemm_kernel, dim3((unsigned)T), dim3(256), 0, st, (const __nv_bfloat16*)x,
+    // Two tokens a CTA until that fills the SMs several times over, then four (the part sums of four take 34 KB).
+    if (T <= 1200)
+        return launch_pdl(route_gemm_kernel<2>, dim3((unsigned)((T + 1) / 2)), dim3(256), 0, st, (const __nv_bfloat16*)x,
+                          (const __nv_bfloat16*)w_router, bias, T, d, E, k, renorm, logits_out, idx, w);
+    return launch_pdl(route_gemm_kernel<4>, dim3((unsigned)((T + 3) / 4)), dim3(256), 0, st, (const __nv_bfloat16*)x,
                       (const __nv_bfloat16*)w_router, bias, T, d, E, k, renorm, logits_out, idx, w);
 }
 cudaError_t launch_scan(const WsDev& ws, int E, int Es, int k, cudaStream_t st) {
