@@ -30,7 +30,7 @@ cudaError_t launch_route(const float* logits, int T, int E, int k, int renorm, i
 cudaError_t launch_route_gemm(const void* x, const void* w_router, const float* bias, int T, int d, int E, int k,
                               int renorm, float* logits_out, int32_t* idx, float* w, cudaStream_t st);
 cudaError_t launch_scan(const WsDev& ws, int E, int Es, int k, cudaStream_t st);
-cudaError_t launch_gather(const LayerDev* L, const WsDev& ws, const void* x, cudaStream_t st);
+cudaError_t launch_gather(const LayerDev* L, const WsDev& ws, const void* x, int d, cudaStream_t st);
 bool front_fits(int T, int k);
 cudaError_t launch_front(const LayerDev* L, const WsDev& ws, const void* x, const float* logits, int E, int Es, int k,
                          int renorm, cudaStream_t st);
@@ -786,7 +786,7 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         else
             CUDA_TRY(launch_route(router_logits, T, D.n_experts, D.top_k, D.renormalize, ws.topk_idx, ws.topk_w, st));
         CUDA_TRY(launch_scan(ws, D.n_experts, D.n_shared, D.top_k, st));
-        CUDA_TRY(launch_gather(L, ws, x, st));
+        CUDA_TRY(launch_gather(L, ws, x, D.d_model, st));
     }
     if (ctx->collect_stats) {
         // row slices per expert: about two CTAs per SM in all; the partial sums live in the down GEMM's output buffer
