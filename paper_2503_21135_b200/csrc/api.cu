@@ -1,5 +1,6 @@
 // Host side of the C-ABI: context, arena / workspace layout, argument validation, launches.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -88,13 +89,6 @@ inline int s_pad_of(const dynamo_layer_desc& D) { return (D.max_sig + 15) / 16 *
 inline bool decode_sized(const dynamo_layer_desc& D, int T) {
     return (long long)T * (D.top_k + D.n_shared) <= DECODE_ROWS;
 }
-// K splits of the down GEMM on the streaming path.  One 256-row block of a Mixtral-shaped expert is a chain of 112
-// stages: a handful of small experts beside a 1000-token prompt took 107 us in 16 such chains per expert, 29 us in eight
-// times as many.  A split keeps four stages at least (a fine-grained expert has 11): an item pays about as much again
-// to start and to be added up.
-inline int ksplit_for(const dynamo_layer_desc& D, int T) {
-    return std::max(1, std::min(MAX_KSPLIT, D.d_ff / KC / (decode_sized(D, T) ? 1 : 4)));
-}
 // Batches that take the fold kernel: more tokens than the streaming kernel serves alone, and few enough that most
 // experts have one 64-row tile (the codes are expanded once per tile).  Layer of eight experts, top-2, 4096 x 14336:
 // 65 tokens 249 us (streaming kernel 255), 100 tokens 269 (streaming and pair kernel 357), 139: 311 (523),
@@ -102,6 +96,26 @@ inline int ksplit_for(const dynamo_layer_desc& D, int T) {
 // tokens: the fine-grained layer at 128 tokens 240 us (176), at 300 260 (212).
 inline bool fold_sized(const dynamo_layer_desc& D, int T) {
     return T > 2 * TC_MIN_ROWS && D.n_shared == 0 && (long long)T * D.top_k <= 62ll * D.n_experts;
+}
+// K splits of the down GEMM.  More splits are more items to balance and to hide latencies with; each pays for its start
+// and once more when the combine kernel adds it up.
+//  - One 256-row block of a Mixtral-shaped expert is a chain of 112 stages: 8 splits (1 token 71 us a pass, 80 with 4,
+//    100 with 2; 8 tokens 133, 137, 170).  The same for a handful of small experts beside a 1000-token prompt: 107 us in
+//    16 such chains per expert, 29 us in eight times as many.
+//  - A fine-grained expert has 11 stages: splits of at least four (4 tokens 67 us with 8 splits, 61 with 2 or 3; 16 tokens
+//    95 and 90), of two where there would be fewer items than SMs, and none once the row blocks alone are half a
+//    thousand items (64 tokens 157 with 8, 116 with 2, 112 with 1).
+//  - The fold kernel's persistent CTAs want two items each (139 tokens 301 us with 8 splits, 292 with 2).
+inline int ksplit_for(const dynamo_layer_desc& D, int T) {
+    const int n_kc = D.d_ff / KC;
+    if (!decode_sized(D, T)) return std::max(1, std::min(MAX_KSPLIT, n_kc / 4));
+    const double miss = std::pow(1.0 - (double)D.top_k / D.n_experts, T);   // an expert none of T tokens chooses
+    const int active = std::max(1, (int)(D.n_experts * (1.0 - miss) + 0.5)) + D.n_shared;
+    const int base = active * (D.d_model / RB);                              // items of one split
+    int ks = n_kc / 4;
+    if (fold_sized(D, T)) ks = std::min(ks, 296 / base);
+    else ks = std::min(std::max(ks, std::min(n_kc / 2, (148 + base - 1) / base)), 1024 / base);
+    return std::max(1, std::min(MAX_KSPLIT, ks));
 }
 inline int switch_ints_per_layer(const dynamo_layer_desc& D) { return D.n_experts * (2 * s_pad_of(D) + 1); }
 
