@@ -677,6 +677,26 @@ __global__ void __launch_bounds__(256) front_kernel(const LayerDev* __restrict__
                s_count[my_e] > ws.tc_min ? LAY_TILES : LAY_ROWS, warp, 8);
 }
 
+// x and the logits of a call on page-locked host buffers, over PCIe into the staging buffers: one launch that the front
+// kernel follows by its programmatic launch, where two copies on the copy engine each add a hand-over between engine and
+// SMs.  Bound by PCIe; every thread has its loads in flight at once.  Not launched programmatically itself: nothing of
+// it runs beside an earlier kernel.
+__global__ void __launch_bounds__(256) upload_kernel(const uint4* __restrict__ xh, uint4* __restrict__ xd, long long nx,
+                                                     const float* __restrict__ lh, float* __restrict__ ld, long long nl) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const long long i0 = (long long)blockIdx.x * 256 + threadIdx.x, step = (long long)gridDim.x * 256;
+    for (long long i = i0; i < nl; i += step) ld[i] = lh[i];
+    for (long long i = i0; i < nx; i += 4 * step) {
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + u * step < nx) v[u] = xh[i + u * step];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + u * step < nx) xd[i + u * step] = v[u];
+    }
+}
+
 // grid (T, ceil(d / 1024)): each thread owns four output columns of one token.
 __global__ void __launch_bounds__(256) combine_kernel(WsDev ws, int d, int k, int Es, void* __restrict__ y,
                                                       int y_f32, long long split_stride, int n_experts) {
@@ -746,6 +766,13 @@ cudaError_t launch_front(const LayerDev* L, const WsDev& ws, const void* x, cons
                          int renorm, cudaStream_t st) {
     return launch_pdl(front_kernel, dim3((unsigned)ws.Rpad), dim3(256), 0, st, L, ws, (const __nv_bfloat16*)x, logits, E,
                       Es, k, renorm);
+}
+cudaError_t launch_upload(const void* xh, void* xd, long long x_bytes, const float* lh, float* ld, long long n_logits,
+                          cudaStream_t st) {
+    const long long nx = x_bytes / 16;
+    const unsigned ctas = (unsigned)std::max(1ll, std::min(592ll, (nx + 255) / 256));
+    upload_kernel<<<ctas, 256, 0, st>>>((const uint4*)xh, (uint4*)xd, nx, lh, ld, n_logits);
+    return cudaGetLastError();
 }
 cudaError_t launch_combine(const WsDev& ws, int d, int k, int Es, void* y, int y_f32, long long split_stride,
                            int n_experts, cudaStream_t st) {

@@ -78,3 +78,35 @@ def test_middle_sized_batches(group_size, down):
 def test_both_ends_of_the_middle_sizes(T):
     cfg, gpu, ora = _layer(256, n_experts=8, top_k=2, group_size=128)
     _check(cfg, gpu, ora, wl.activations(cfg, T, step=33), wl.router_logits(cfg, T, step=33), np.arange(T))
+
+
+@pytest.mark.parametrize("cfg_kw", [dict(n_experts=8, d_ff=1024), dict(n_experts=48, d_ff=2048), dict(n_experts=24, d_ff=2048),
+                                    dict(n_experts=24, d_ff=2048, n_shared=1)])
+@pytest.mark.parametrize("T", [7, 9, 17, 25, 33, 49, 64])
+def test_items_of_every_size_on_the_streaming_path(cfg_kw, T):
+    """Small batches with a skewed router: the first expert has all the tokens, the second half of them, so experts take
+    one to eight passes of items of one, two or three tiles, with a remainder, in launches of few and of many items."""
+    cfg, gpu, ora = _layer(64, top_k=3, group_size=64, **cfg_kw)
+    lg = wl.router_logits(cfg, T, step=34)
+    lg[:, 0] += 20.0
+    lg[: (T + 1) // 2, 1] += 20.0
+    _check(cfg, gpu, ora, wl.activations(cfg, T, step=34), lg, np.arange(T))
+
+
+@pytest.mark.parametrize("T", [1, 5, 64, 70])
+@pytest.mark.parametrize("kind", ["pinned", "pageable", "results_pinned", "shifted"])
+def test_host_buffers_of_every_kind(kind, T):
+    """Page-locked and aligned buffers are read and written in place, others through copies: the same results."""
+    def buffer(t, pin):
+        flat = torch.empty(t.numel() + 8, dtype=t.dtype, pin_memory=pin)
+        off = 1 if kind == "shifted" else 0
+        return flat[off: off + t.numel()].view(t.shape).copy_(t)
+
+    cfg, gpu, _ = _layer(80, n_experts=5, top_k=2, group_size=64)
+    x, lg = wl.activations(cfg, T, step=35), wl.router_logits(cfg, T, step=35)
+    ins = kind in ("pinned", "shifted")
+    for dtype, code in ((torch.float32, binding.F32), (torch.bfloat16, binding.BF16)):
+        y = buffer(torch.zeros((T, cfg.d_model), dtype=dtype), kind != "pageable")
+        gpu.forward_host(buffer(x, ins), buffer(lg, ins), y, code)
+        assert gpu.poll_status() == 0
+        assert torch.equal(y, gpu.forward(x.cuda(), lg.cuda(), code).cpu())
