@@ -40,7 +40,8 @@ cudaError_t launch_front(const LayerDev* L, const WsDev& ws, const void* x, cons
 cudaError_t launch_combine(const WsDev& ws, int d, int k, int Es, void* y, int y_f32, long long split_stride,
                            int n_experts, cudaStream_t st);
 cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
-                              long long split_stride, int max_rows, int n_sms, int G, cudaStream_t st);
+                              long long split_stride, int tiles, long long n_items, bool long_rows, int n_sms, int G,
+                              cudaStream_t st);
 cudaError_t launch_ffn_fold(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
                             long long split_stride, int n_sms, int G, cudaStream_t st);
 cudaError_t setup_ffn_tc2(int n_sms, int* clusters_out);
@@ -99,6 +100,31 @@ inline bool decode_sized(const dynamo_layer_desc& D, int T) {
 inline bool fold_sized(const dynamo_layer_desc& D, int T) {
     return T > 2 * TC_MIN_ROWS && D.n_shared == 0 && (long long)T * D.top_k <= 62ll * D.n_experts;
 }
+// Routed experts that T tokens reach when all are equally likely.
+inline int active_experts(const dynamo_layer_desc& D, int T) {
+    const double miss = std::pow(1.0 - (double)D.top_k / D.n_experts, T);   // an expert none of the tokens chooses
+    return std::max(1, (int)(D.n_experts * (1.0 - miss) + 0.5));
+}
+// Passes that the streaming kernel makes over an expert's blocks in a batch of T tokens, with items of up to 8 * tiles
+// tokens; summed over the experts.
+inline long long stream_passes(const dynamo_layer_desc& D, int T, int tiles) {
+    const double per = 8.0 * tiles, rows = (double)T * D.top_k / D.n_experts;
+    return (long long)(active_experts(D, T) * std::max(1.0, rows / per + 0.5)) + D.n_shared * (int)((T + per - 1) / per);
+}
+// 8-token tiles of the streaming kernel's variant (where it is the only path).  Fewer tiles take fewer registers, so three
+// CTAs fit an SM and nothing spills, but an expert with more rows than an item holds is expanded once more.
+//  - One tile up to seven rows an expert: 12, 16, 24 and 28 tokens of a Mixtral-shaped layer 157, 181, 181, 199 us a pass
+//    against 172, 194, 192, 205 with two tiles and (24, 28) 196, 206 with three; two up to ten: 32 tokens 217, 209, 215
+//    with one, two, three tiles, 40: 235, 210, 222, 48: 293, 251, 238.
+//  - A shared expert has all the tokens: with 2 beside 64, one tile up to 40 of them (93 us, 98 with three; 48: 105, 101).
+//  - A launch that does not fill the SMs is a matter of latency, and the one-tile kernel is the shortest: 512-wide layer,
+//    64 tokens 29 us, 36 with three.
+inline int stream_tiles(const dynamo_layer_desc& D, int T, int n_rb13, int n_sms) {
+    const double rows = (double)T * D.top_k / D.n_experts;
+    if (T <= 8 || stream_passes(D, T, 1) * n_rb13 <= 3ll * n_sms) return 1;
+    if (D.n_shared) return rows <= 7 && T <= 40 ? 1 : 3;
+    return rows <= 7 ? 1 : (rows <= 10 || T <= 16) ? 2 : 3;
+}
 // K splits of the down GEMM.  More splits are more items to balance and to hide latencies with; each pays for its start
 // and once more when the combine kernel adds it up.
 //  - One 256-row block of a Mixtral-shaped expert is a chain of 112 stages: 8 splits (1 token 71 us a pass, 80 with 4,
@@ -111,9 +137,7 @@ inline bool fold_sized(const dynamo_layer_desc& D, int T) {
 inline int ksplit_for(const dynamo_layer_desc& D, int T) {
     const int n_kc = D.d_ff / KC;
     if (!decode_sized(D, T)) return std::max(1, std::min(MAX_KSPLIT, n_kc / 4));
-    const double miss = std::pow(1.0 - (double)D.top_k / D.n_experts, T);   // an expert none of T tokens chooses
-    const int active = std::max(1, (int)(D.n_experts * (1.0 - miss) + 0.5)) + D.n_shared;
-    const int base = active * (D.d_model / RB);                              // items of one split
+    const int base = (active_experts(D, T) + D.n_shared) * (D.d_model / RB);   // items of one split
     int ks = n_kc / 4;
     if (fold_sized(D, T)) ks = std::min(ks, 296 / base);
     else ks = std::min(std::max(ks, std::min(n_kc / 2, (148 + base - 1) / base)), 1024 / base);
@@ -823,13 +847,16 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
         CUDA_TRY(launch_ffn_fold(L, ws, 0, ctx->host_layer.n_rb2, ws.ksplit, n, split_stride, ctx->n_sms, D.group_size, st));
     } else {
-        const int max_rows = use_tc ? std::min(T, ctx->tc_min_rows) : T;  // rows one expert can have on the streaming path
-        CUDA_TRY(launch_ffn_stream(L, ws, 1, ctx->host_layer.n_rb13, 1, n, split_stride, max_rows, ctx->n_sms,
+        const int n_rb13 = ctx->host_layer.n_rb13, n_rb2 = ctx->host_layer.n_rb2;
+        const int tiles = use_tc ? 3 : stream_tiles(D, T, n_rb13, ctx->n_sms);
+        const long long passes = stream_passes(D, T, tiles);
+        const bool long_rows = (use_tc ? std::min(T, ctx->tc_min_rows) : T) > 32;   // an expert on this path
+        CUDA_TRY(launch_ffn_stream(L, ws, 1, n_rb13, 1, n, split_stride, tiles, passes * n_rb13, long_rows, ctx->n_sms,
                                    D.group_size, st));
         if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, ctx->host_layer.n_rb13, n, ctx->tc2_clusters[1], st));
         if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
-        CUDA_TRY(launch_ffn_stream(L, ws, 0, ctx->host_layer.n_rb2, ws.ksplit, n, split_stride, max_rows, ctx->n_sms,
-                                   D.group_size, st));
+        CUDA_TRY(launch_ffn_stream(L, ws, 0, n_rb2, ws.ksplit, n, split_stride, tiles, passes * n_rb2 * ws.ksplit,
+                                   long_rows, ctx->n_sms, D.group_size, st));
         if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, ctx->host_layer.n_rb2, n, ctx->tc2_clusters[0], st));
     }
     if (ctx->prof_ev[2]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[2], st));

@@ -36,10 +36,10 @@ constexpr int CONSUMER_WARPS = 16 / APW;
 constexpr int FFN_THREADS = (CONSUMER_WARPS + 1) * 32;
 constexpr int SMEM_HEADER = 2048;     // barriers, poison flag, per-expert item prefix table
 constexpr int MAX_STAGES = 16;        // ring queue depth; the ring itself is byte-granular
-// Tokens per work item.  24, not 32: with at most three 8-token tiles the two accumulator sets of a warp fit the 96
-// registers that two resident CTAs leave a thread (four tiles spilled ~1.3 KB of loads per thread into the
-// loops); an expert of 25-32 rows takes a second, short pass over its blocks, which hits L2.
-constexpr int CHUNK_TOKENS = 24;
+// Most tokens of a work item: 8 per tile of the kernel variant.  An expert with more rows takes further passes over its
+// blocks, which hit L2.  At most 24, not 32: with three 8-token tiles the two accumulator sets of a warp fit the 96
+// registers that two resident CTAs leave a thread (four tiles spilled ~1.3 KB of loads per thread into the loops).
+template <int MAXNT8> constexpr int chunk_tokens = 8 * MAXNT8;
 
 struct FfnParams {
     const LayerDev* L;
@@ -83,22 +83,17 @@ static_assert(sizeof(FfnSmem) <= SMEM_HEADER, "header too small");
 struct Cursor {
     int sec = 0, y = 0;
 };
-// The expert position whose items hold index g; y is not beyond it.  A short walk, then bisection.
+// The expert position whose items hold index g; y is not beyond it.  Steps of eight, then of one.
 __device__ __forceinline__ int seek(const int* prefix, int g, int y, int n) {
-    for (int i = 0; i < 8; ++i, ++y)
-        if (g < prefix[y + 1]) return y;
-    int hi = n - 1;
-    while (y < hi) {
-        const int mid = (y + hi) >> 1;
-        if (g < prefix[mid + 1]) hi = mid;
-        else y = mid + 1;
-    }
+    while (y + 8 < n && g >= prefix[y + 8]) y += 8;
+    while (g >= prefix[y + 1]) ++y;
     return y;
 }
-template <bool SECT>
+template <int MAXNT8>
 __device__ __forceinline__ Item decode_item(const FfnParams& p, const FfnSmem* S, int g, Cursor& cur) {
+    constexpr int CHUNK_TOKENS = chunk_tokens<MAXNT8>;
     int e, cnt, tc, rbs;
-    if (SECT && S->sectioned) {
+    if (MAXNT8 == 3 && S->sectioned) {
         const int sec = g < S->sec_base[1] ? 0 : (g < S->sec_base[2] ? 1 : 2);
         if (sec != cur.sec) {
             cur.sec = sec;
@@ -147,8 +142,10 @@ __device__ __forceinline__ void mma16816_z(float (&d)[4], const uint32_t (&a)[4]
 }
 
 // Consumer side of one work item.  `stage_it` is the CTA-wide ring position, `item_idx` the number of
-// items this CTA has finished (parity of the epilogue barrier / h tile).
-template <int BITS, int NT8, bool GATEUP, int G>
+// items this CTA has finished (parity of the epilogue barrier / h tile).  SPLIT_SMALL: K splits behind the first may write
+// the compact partial rows of small experts beside large ones, which only a launch with items of three tiles has; the
+// address of such a row costs the two-tile kernels registers that they spill (16 tokens, down launch 55.7 -> 58.0 us).
+template <int BITS, int NT8, bool GATEUP, int G, bool SPLIT_SMALL>
 __device__ __forceinline__ bool consume_item(const FfnParams& p, FfnSmem* S, uint8_t* stages, uint8_t* htiles,
                                              const Item& im, int& stage_it, int item_idx, bool& clamped) {
     constexpr int NS = MAX_STAGES;
@@ -330,7 +327,12 @@ __device__ __forceinline__ bool consume_item(const FfnParams& p, FfnSmem* S, uin
         }
     } else {
         const int d = L->d;
-        float* yb = ypart_row(p.ws, im.split, p.split_stride, im.e, p.n_experts, im.row0, p.ws.off_pad[im.e], d);
+        float* yb = p.ws.ypart + (size_t)im.split * p.split_stride;
+        int row0 = im.row0;
+        if constexpr (SPLIT_SMALL) {
+            yb = ypart_row(p.ws, im.split, p.split_stride, im.e, p.n_experts, im.row0, p.ws.off_pad[im.e], d);
+            row0 = 0;
+        }
 #pragma unroll
         for (int a = 0; a < APW; ++a)
 #pragma unroll
@@ -339,7 +341,7 @@ __device__ __forceinline__ bool consume_item(const FfnParams& p, FfnSmem* S, uin
                 for (int c = 0; c < 4; ++c) {
                     const int tok = 8 * j + 2 * tid4 + (c & 1);
                     const int n = im.rb * RB + (atom0 + a) * 16 + gid + ((c >> 1) ? 8 : 0);
-                    if (tok < im.nvalid) yb[(size_t)tok * d + n] = total[a][j][c];
+                    if (tok < im.nvalid) yb[(size_t)(row0 + tok) * d + n] = total[a][j][c];
                 }
     }
     return true;
@@ -351,12 +353,12 @@ template <int BITS, bool GATEUP, int MAXNT8, int G>
 __device__ __forceinline__ bool consume_dispatch(const FfnParams& p, FfnSmem* S, uint8_t* stages, uint8_t* htiles,
                                                  const Item& im, int& stage_it, int item_idx, bool& clamped) {
     const int nt8 = (im.nvalid + 7) >> 3;
-    if (MAXNT8 == 1 || nt8 == 1) return consume_item<BITS, 1, GATEUP, G>(p, S, stages, htiles, im, stage_it, item_idx, clamped);
+    if (MAXNT8 == 1 || nt8 == 1) return consume_item<BITS, 1, GATEUP, G, MAXNT8 == 3>(p, S, stages, htiles, im, stage_it, item_idx, clamped);
     if constexpr (MAXNT8 >= 2) {
         if (MAXNT8 == 2 || nt8 == 2)
-            return consume_item<BITS, 2, GATEUP, G>(p, S, stages, htiles, im, stage_it, item_idx, clamped);
+            return consume_item<BITS, 2, GATEUP, G, MAXNT8 == 3>(p, S, stages, htiles, im, stage_it, item_idx, clamped);
     }
-    if constexpr (MAXNT8 >= 3) return consume_item<BITS, 3, GATEUP, G>(p, S, stages, htiles, im, stage_it, item_idx, clamped);
+    if constexpr (MAXNT8 >= 3) return consume_item<BITS, 3, GATEUP, G, MAXNT8 == 3>(p, S, stages, htiles, im, stage_it, item_idx, clamped);
     return false;
 }
 
@@ -387,6 +389,7 @@ __global__ void __launch_bounds__(FFN_THREADS, (MAXNT8 <= 2 && APW == 2) ? 3 : 2
         // layer of 66 experts, 16 tokens: 44.5 + 29.3 us for the two launches, 42.6 + 25.8 with the scan; 512-wide
         // layer of 8 experts, 64 tokens: 18.3 + 11.2 -> 17.7 + 10.5).
         const int per_chunk = p.n_rb * p.ksplit, n1 = p.n_experts + 1;
+        constexpr int CHUNK_TOKENS = chunk_tokens<MAXNT8>;
         const bool sect = MAXNT8 == 3 && p.sectioned;   // sections: chunks of 3, 2, 1 tiles
         int run[3] = {0, 0, 0};
         for (int y0 = 0; y0 < p.n_experts; y0 += 32) {
@@ -481,7 +484,7 @@ __global__ void __launch_bounds__(FFN_THREADS, (MAXNT8 <= 2 && APW == 2) ? 3 : 2
                 break;
             }
             bool first = true;
-            const Item im = decode_item<MAXNT8 == 3>(p, S, g, y);
+            const Item im = decode_item<MAXNT8>(p, S, g, y);
             const ExpertDev& ex = L->ex[im.e];
             const int blk_bytes = ex.blk_bytes;
             int kc0 = 0, kc1 = n_kc;
@@ -555,7 +558,7 @@ __global__ void __launch_bounds__(FFN_THREADS, (MAXNT8 <= 2 && APW == 2) ? 3 : 2
             g = S->first_item[s0];
         }
         if (g < 0 || g >= n_items) break;
-        const Item im = decode_item<MAXNT8 == 3>(p, S, g, y);
+        const Item im = decode_item<MAXNT8>(p, S, g, y);
         bool ok;
         switch (L->ex[im.e].bits) {
             case 2: ok = consume_dispatch<2, GATEUP, MAXNT8, G>(p, S, stages, htiles, im, stage_it, item_idx, clamped); break;
@@ -586,13 +589,17 @@ static cudaError_t launch_one(const FfnParams& p, int n_ctas, int G, cudaStream_
     return G == 64 ? launch_one_g<GATEUP, MAXNT8, 64>(p, n_ctas, st) : launch_one_g<GATEUP, MAXNT8, 128>(p, n_ctas, st);
 }
 
-// max_rows: upper bound of the rows one expert can have in this forward (selects the kernel variant);
-// n_sms: SM count (the persistent grid is 2 or 3 CTAs per SM).
+// tiles: 8-token tiles of the kernel variant (1..3); n_items: about how many items the launch has; long_rows: an expert
+// can have more than 32 rows.
+//
+// Three CTAs per SM hide more of each other's latencies, two have rings half as large again and leave room for the next
+// kernel's CTAs: three pay once every one has an item (1, 2, 3 and 4 tokens of a Mixtral-shaped layer: 68, 107, 130, 130
+// us a pass with two, 81, 104, 114, 114 with three; fine-grained, 4 and 16 tokens: 50 and 76, 61 and 72; 512-wide layer
+// of 64 tokens: 29 and 38).  The kernel of three tiles needs the registers of two.
 cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
-                              long long split_stride, int max_rows, int n_sms, int G, cudaStream_t st) {
-    // three CTAs per SM pay off once every CTA has several items to walk; at 1-3 tokens a CTA sees one or two
-    const bool small = max_rows >= 4 && max_rows <= 16;
-    const bool three = small && APW == 2;
+                              long long split_stride, int tiles, long long n_items, bool long_rows, int n_sms, int G,
+                              cudaStream_t st) {
+    const bool three = tiles < 3 && APW == 2 && n_items > 3 * n_sms;
     const int smem_bytes = three ? 74 * 1024 : 110 * 1024;
     const int n_ctas = (three ? 3 : 2) * n_sms;
     FfnParams p;
@@ -601,15 +608,14 @@ cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, in
     p.ksplit = ksplit;
     p.split_stride = split_stride;
     p.smem_bytes = smem_bytes;
-    // two h tiles (double-buffered across items) behind the ring; the small variants hold at most 16 tokens
-    p.htile_bytes = (small ? 16 : CHUNK_TOKENS) * XROW;
+    p.htile_bytes = 8 * tiles * XROW;   // two h tiles (double-buffered across items) behind the ring
     p.ring_bytes = (smem_bytes - SMEM_HEADER - (gateup ? 2 * p.htile_bytes : 0)) & ~127;
     p.n_rb = n_rb;
     p.n_experts = n_experts;
     p.work_ctr = ws.status + (gateup ? 4 : 5);
-    p.sectioned = (max_rows > 32 && n_experts <= MAX_SECT_EXPERTS) ? 1 : 0;   // measured: +3 % at 64 tokens, -1 % at 32
-    if (small && max_rows <= 8) return gateup ? launch_one<true, 1>(p, n_ctas, G, st) : launch_one<false, 1>(p, n_ctas, G, st);
-    if (small) return gateup ? launch_one<true, 2>(p, n_ctas, G, st) : launch_one<false, 2>(p, n_ctas, G, st);
+    p.sectioned = (long_rows && n_experts <= MAX_SECT_EXPERTS) ? 1 : 0;   // measured: +3 % at 64 tokens, -1 % at 32
+    if (tiles == 1) return gateup ? launch_one<true, 1>(p, n_ctas, G, st) : launch_one<false, 1>(p, n_ctas, G, st);
+    if (tiles == 2) return gateup ? launch_one<true, 2>(p, n_ctas, G, st) : launch_one<false, 2>(p, n_ctas, G, st);
     return gateup ? launch_one<true, 3>(p, n_ctas, G, st) : launch_one<false, 3>(p, n_ctas, G, st);
 }
 

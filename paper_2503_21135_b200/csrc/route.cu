@@ -710,13 +710,18 @@ __global__ void __launch_bounds__(256) combine_kernel(WsDev ws, int d, int k, in
     for (int j = 0; j < kk; ++j) {
         const int r = ws.pos[t * kk + j];
         const float w = (j < k) ? ws.topk_w[t * k + j] : 1.0f;
-        float s[4] = {0.f, 0.f, 0.f, 0.f};
         const int e = ws.row_expert[r];
         const int ns = (ws.counts[e] > ws.tc_min) ? 1 : ws.ksplit;  // the tensor-core path does not split K
-        for (int sp = 0; sp < ns; ++sp) {
-            const float4 v =
-                *reinterpret_cast<const float4*>(ypart_row(ws, sp, split_stride, e, n_experts, r, ws.off_pad[e], d) + c);
-            s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
+        const float* src = ws.ypart + (long long)r * d + c;
+        const float4 v0 = *reinterpret_cast<const float4*>(src);
+        float s[4] = {v0.x, v0.y, v0.z, v0.w};
+        if (ns > 1) {
+            src = ws.ysmall ? ypart_row(ws, 1, split_stride, e, n_experts, r, ws.off_pad[e], d) + c : src + split_stride;
+            const long long step = ws.ysmall ? (long long)n_experts * TC_MIN_ROWS * d : split_stride;
+            for (int sp = 1; sp < ns; ++sp, src += step) {
+                const float4 v = *reinterpret_cast<const float4*>(src);
+                s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
+            }
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[i] = fmaf(w, s[i], acc[i]);
