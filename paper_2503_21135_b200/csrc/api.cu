@@ -40,8 +40,8 @@ cudaError_t launch_front(const LayerDev* L, const WsDev& ws, const void* x, cons
 cudaError_t launch_combine(const WsDev& ws, int d, int k, int Es, void* y, int y_f32, long long split_stride,
                            int n_experts, cudaStream_t st);
 cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
-                              long long split_stride, int tiles, long long n_items, bool long_rows, int n_sms, int G,
-                              cudaStream_t st);
+                              long long split_stride, int tiles, long long n_items, bool long_rows, bool fills,
+                              int n_sms, int G, cudaStream_t st);
 cudaError_t launch_ffn_fold(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
                             long long split_stride, int n_sms, int G, cudaStream_t st);
 cudaError_t setup_ffn_tc2(int n_sms, int* clusters_out);
@@ -851,13 +851,16 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         const int tiles = use_tc ? 3 : stream_tiles(D, T, n_rb13, ctx->n_sms);
         const long long passes = stream_passes(D, T, tiles);
         const bool long_rows = (use_tc ? std::min(T, ctx->tc_min_rows) : T) > 32;   // an expert on this path
-        CUDA_TRY(launch_ffn_stream(L, ws, 1, n_rb13, 1, n, split_stride, tiles, passes * n_rb13, long_rows, ctx->n_sms,
-                                   D.group_size, st));
-        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, ctx->host_layer.n_rb13, n, ctx->tc2_clusters[1], st));
+        // The pair kernel goes first where there is one: its clusters walk a fixed list and leave the last round uneven,
+        // and the streaming kernel's queue fills the SMs as they come free (fine-grained layer, 300 tokens: 244 us a pass
+        // with the streaming kernel first and a launch waiting for the other, 229 so; 2048: 499, 483).
+        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, n_rb13, n, ctx->tc2_clusters[1], st));
+        CUDA_TRY(launch_ffn_stream(L, ws, 1, n_rb13, 1, n, split_stride, tiles, passes * n_rb13, long_rows, use_tc,
+                                   ctx->n_sms, D.group_size, st));
         if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
+        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, n_rb2, n, ctx->tc2_clusters[0], st));
         CUDA_TRY(launch_ffn_stream(L, ws, 0, n_rb2, ws.ksplit, n, split_stride, tiles, passes * n_rb2 * ws.ksplit,
-                                   long_rows, ctx->n_sms, D.group_size, st));
-        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, ctx->host_layer.n_rb2, n, ctx->tc2_clusters[0], st));
+                                   long_rows, use_tc, ctx->n_sms, D.group_size, st));
     }
     if (ctx->prof_ev[2]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[2], st));
     if (ctx->down_active) {  // significant hidden units: add what their 8-bit columns of W_down change

@@ -336,6 +336,12 @@ __device__ __forceinline__ void pdl_prologue() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// A pair of launches that do not need each other's results.  The first waits, reads what the second may write (the status
+// word), and only then lets the second start: all that came before the pair has completed and flushed by the time that a
+// CTA of the second runs.  The second does not wait until its end, where every CTA does: whoever waits for its completion
+// has waited for both.  In between it takes the SMs that the first no longer fills.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,

@@ -182,7 +182,7 @@ __device__ __forceinline__ void t2_dequant_half(const uint8_t* st, uint32_t a_co
 template <bool GATEUP>
 __global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p) {
     extern __shared__ __align__(1024) uint8_t smem[];
-    pdl_prologue();
+    pdl_wait();
     const LayerDev* L = p.L;
     const int G = L->G;
     const int K = GATEUP ? L->d : L->f;
@@ -201,6 +201,7 @@ __global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p
     // completed, and every cluster of this persistent grid starts at launch), so they leave together, before any
     // barrier or tensor memory exists.
     if (*p.ws.status & STATUS_TIMEOUT) return;
+    pdl_trigger();   // the streaming kernel of the smaller experts may fill the SMs from here on
     // Item table (identical in both CTAs of the pair): experts above the row threshold contribute
     // (256-token tiles x row blocks) items.
     for (int i = threadIdx.x; i < p.n_experts; i += T2_THREADS) {

@@ -110,3 +110,25 @@ def test_host_buffers_of_every_kind(kind, T):
         gpu.forward_host(buffer(x, ins), buffer(lg, ins), y, code)
         assert gpu.poll_status() == 0
         assert torch.equal(y, gpu.forward(x.cuda(), lg.cuda(), code).cpu())
+
+
+@pytest.mark.parametrize("large", [1, 3, 7])
+def test_small_experts_run_beside_large_ones(large):
+    """The kernels of large and of small experts overlap: forwards of different inputs that follow one another without a
+    wait in between give what each gives alone."""
+    cfg, gpu, _ = _layer(700, n_experts=8, top_k=1, group_size=64)
+    runs = []
+    for i, T in enumerate((700, 640, 300)):
+        e = np.where(np.arange(T) % 16 < 15, np.arange(T) % large, large + np.arange(T) % (8 - large))
+        lg = torch.zeros((T, 8))
+        lg[torch.arange(T), torch.from_numpy((e + i) % 8)] = 4.0
+        x = wl.activations(cfg, T, step=36 + i).cuda()
+        runs.append((x, lg.cuda()))
+    alone = []
+    for x, lg in runs:
+        alone.append(gpu.forward(x, lg, binding.F32).clone())
+        torch.cuda.synchronize()
+    for _ in range(5):
+        got = [gpu.forward(x, lg, binding.F32) for x, lg in runs]
+        assert all(torch.equal(a, b) for a, b in zip(got, alone))
+    assert gpu.poll_status() == 0 and gpu.debug_check_guards() == 0
