@@ -697,7 +697,10 @@ __global__ void __launch_bounds__(256) upload_kernel(const uint4* __restrict__ x
     }
 }
 
-// grid (T, ceil(d / 1024)): each thread owns four output columns of one token.
+// grid (T, ceil(d / 1024)): each thread owns four output columns of one token.  KS > 0: every expert's result is in KS
+// copies of ypart (the K splits, known to the compiler, no lookups in front of their loads: 8 tokens of 4096 in 8 splits
+// 6.0 -> 5.2 us); 0: any forward.
+template <int KS>
 __global__ void __launch_bounds__(256) combine_kernel(WsDev ws, int d, int k, int Es, void* __restrict__ y,
                                                       int y_f32, long long split_stride, int n_experts) {
     pdl_prologue();
@@ -707,21 +710,33 @@ __global__ void __launch_bounds__(256) combine_kernel(WsDev ws, int d, int k, in
     const int c = (blockIdx.y * blockDim.x + threadIdx.x) * 4;
     if (c >= d) return;
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int j = 0; j < kk; ++j) {
+    if constexpr (KS > 0) {
+#pragma unroll 2
+        for (int j = 0; j < kk; ++j) {
+            const float* src = ws.ypart + (long long)ws.pos[t * kk + j] * d + c;
+            const float w = (j < k) ? ws.topk_w[t * k + j] : 1.0f;
+            float4 v[KS];
+#pragma unroll
+            for (int sp = 0; sp < KS; ++sp) v[sp] = *reinterpret_cast<const float4*>(src + sp * split_stride);
+            float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int sp = 0; sp < KS; ++sp) {
+                s[0] += v[sp].x; s[1] += v[sp].y; s[2] += v[sp].z; s[3] += v[sp].w;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] = fmaf(w, s[i], acc[i]);
+        }
+    }
+    for (int j = KS > 0 ? kk : 0; j < kk; ++j) {
         const int r = ws.pos[t * kk + j];
         const float w = (j < k) ? ws.topk_w[t * k + j] : 1.0f;
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
         const int e = ws.row_expert[r];
         const int ns = (ws.counts[e] > ws.tc_min) ? 1 : ws.ksplit;  // the tensor-core path does not split K
-        const float* src = ws.ypart + (long long)r * d + c;
-        const float4 v0 = *reinterpret_cast<const float4*>(src);
-        float s[4] = {v0.x, v0.y, v0.z, v0.w};
-        if (ns > 1) {
-            src = ws.ysmall ? ypart_row(ws, 1, split_stride, e, n_experts, r, ws.off_pad[e], d) + c : src + split_stride;
-            const long long step = ws.ysmall ? (long long)n_experts * TC_MIN_ROWS * d : split_stride;
-            for (int sp = 1; sp < ns; ++sp, src += step) {
-                const float4 v = *reinterpret_cast<const float4*>(src);
-                s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
-            }
+        for (int sp = 0; sp < ns; ++sp) {
+            const float4 v =
+                *reinterpret_cast<const float4*>(ypart_row(ws, sp, split_stride, e, n_experts, r, ws.off_pad[e], d) + c);
+            s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[i] = fmaf(w, s[i], acc[i]);
@@ -781,8 +796,13 @@ cudaError_t launch_upload(const void* xh, void* xd, long long x_bytes, const flo
 }
 cudaError_t launch_combine(const WsDev& ws, int d, int k, int Es, void* y, int y_f32, long long split_stride,
                            int n_experts, cudaStream_t st) {
-    return launch_pdl(combine_kernel, dim3((unsigned)ws.T, (unsigned)((d + 1023) / 1024)), dim3(256), 0, st, ws, d, k, Es,
-                      y, y_f32, split_stride, n_experts);
+    const bool uniform = ws.tc_min == 0x7fffffff && !ws.ysmall;
+    auto kernel = uniform && ws.ksplit == 8   ? combine_kernel<8>
+                  : uniform && ws.ksplit == 2 ? combine_kernel<2>
+                  : uniform && ws.ksplit == 1 ? combine_kernel<1>
+                                              : combine_kernel<0>;
+    return launch_pdl(kernel, dim3((unsigned)ws.T, (unsigned)((d + 1023) / 1024)), dim3(256), 0, st, ws, d, k, Es, y, y_f32,
+                      split_stride, n_experts);
 }
 
 }  // namespace dyn
