@@ -40,7 +40,7 @@ cudaError_t launch_front(const LayerDev* L, const WsDev& ws, const void* x, cons
 cudaError_t launch_combine(const WsDev& ws, int d, int k, int Es, void* y, int y_f32, long long split_stride,
                            int n_experts, cudaStream_t st);
 cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
-                              long long split_stride, int tiles, long long n_items, bool long_rows, bool fills,
+                              long long split_stride, int tiles, long long n_items, bool long_rows, bool fills, bool leads,
                               int n_sms, int G, cudaStream_t st);
 cudaError_t launch_ffn_fold(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
                             long long split_stride, int n_sms, int G, cudaStream_t st);
@@ -828,7 +828,10 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         CUDA_TRY(launch_scan(ws, D.n_experts, D.n_shared, D.top_k, st));
         CUDA_TRY(launch_gather(L, ws, x, D.d_model, st));
     }
-    if (ctx->collect_stats) {
+    const bool use_tc = ws.tc_min != 0x7fffffff;                  // experts above 32 rows take the tcgen05 path
+    const long long split_stride = (long long)ws.Rpad * D.d_model;  // partials of one K split: [Rpad][d]
+    auto collect_stats = [&]() -> dynamo_status {   // beside the gate/up kernels: it only has to be done before the down launch
+        if (!ctx->collect_stats) return DYNAMO_OK;
         // row slices per expert: about two CTAs per SM in all; the partial sums live in the down GEMM's output buffer
         // (at least 8 * (E + Es) rows of d floats, idle until the down launch), which bounds the slice count
         const int P_pad = ctx->host_layer.P_pad;
@@ -838,12 +841,12 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         CUDA_TRY(launch_stats(L, ws, x, (float*)(ctx->arena + ctx->A.stats), ws.ypart,
                               (int32_t*)(ctx->arena + ctx->A.stats_ctr), D.n_experts, n_slices, st));
         ctx->launches += 1;
-    }
-    const bool use_tc = ws.tc_min != 0x7fffffff;                  // experts above 32 rows take the tcgen05 path
-    const long long split_stride = (long long)ws.Rpad * D.d_model;  // partials of one K split: [Rpad][d]
+        return DYNAMO_OK;
+    };
     if (ctx->prof_ev[0]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[0], st));
     if (ws.fold) {
         CUDA_TRY(launch_ffn_fold(L, ws, 1, ctx->host_layer.n_rb13, 1, n, split_stride, ctx->n_sms, D.group_size, st));
+        if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
         if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
         CUDA_TRY(launch_ffn_fold(L, ws, 0, ctx->host_layer.n_rb2, ws.ksplit, n, split_stride, ctx->n_sms, D.group_size, st));
     } else {
@@ -856,11 +859,12 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         // with the streaming kernel first and a launch waiting for the other, 229 so; 2048: 499, 483).
         if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, n_rb13, n, ctx->tc2_clusters[1], st));
         CUDA_TRY(launch_ffn_stream(L, ws, 1, n_rb13, 1, n, split_stride, tiles, passes * n_rb13, long_rows, use_tc,
-                                   ctx->n_sms, D.group_size, st));
+                                   ctx->collect_stats, ctx->n_sms, D.group_size, st));
+        if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
         if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
         if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, n_rb2, n, ctx->tc2_clusters[0], st));
         CUDA_TRY(launch_ffn_stream(L, ws, 0, n_rb2, ws.ksplit, n, split_stride, tiles, passes * n_rb2 * ws.ksplit,
-                                   long_rows, use_tc, ctx->n_sms, D.group_size, st));
+                                   long_rows, use_tc, ctx->down_active, ctx->n_sms, D.group_size, st));
     }
     if (ctx->prof_ev[2]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[2], st));
     if (ctx->down_active) {  // significant hidden units: add what their 8-bit columns of W_down change

@@ -124,16 +124,16 @@ constexpr int FIX_MAX_SIG = 256;  // capacity of a significant set
 // h of the group's rows at the expert's significant hidden units goes to shared memory (unscaled: the buffer holds h
 // times a power of two that depends on the base bit-width and the position); every thread accumulates its two
 // output columns over its slice of the set (differences loaded eight slots ahead: independent loads), the slices
-// are summed through shared memory and added to the down GEMM's result.  KS = 4 for decode-sized batches, where
+// are summed through shared memory and added to the down GEMM's result: only that waits for the down launch, beside whose
+// last items the rest runs (see pdl_trigger in common.cuh; fine-grained layer, 16 tokens: 10 us behind it).  KS = 4 for decode-sized batches, where
 // the kernel is a chain of memory latencies and more, shorter chains run in parallel; 1 otherwise.
 template <int KS>
-__global__ void __launch_bounds__(FIX_THREADS) down_fix_kernel(const LayerDev* __restrict__ L,
-                                                               const DownDev* __restrict__ D2, WsDev ws) {
+__device__ __forceinline__ void down_fix_cta(const LayerDev* __restrict__ L, const DownDev* __restrict__ D2,
+                                             const WsDev& ws) {
     constexpr int PAIRS = FIX_THREADS / KS;
     __shared__ __align__(16) float hs[FIX_MAX_SIG][FIX_ROWS];
     __shared__ int pl[FIX_MAX_SIG], ch[FIX_MAX_SIG];
     __shared__ float red[KS > 1 ? (KS - 1) * FIX_ROWS * 2 * PAIRS : 1];
-    pdl_prologue();
     const int row0 = blockIdx.x * FIX_ROWS;
     if (row0 >= ws.off_pad[L->E + L->Es]) return;
     const int e = ws.row_expert[row0];
@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(FIX_THREADS) down_fix_kernel(const LayerDev* _
             }
     }
     if (!col_ok) return;
+    pdl_wait();
 #pragma unroll
     for (int r = 0; r < FIX_ROWS; ++r)
         if (r < nrows) {  // K split 0; the combine adds the splits
@@ -223,6 +224,13 @@ __global__ void __launch_bounds__(FIX_THREADS) down_fix_kernel(const LayerDev* _
             v.y += acc[r][1];
             *y = v;
         }
+}
+template <int KS>
+__global__ void __launch_bounds__(FIX_THREADS) down_fix_kernel(const LayerDev* __restrict__ L,
+                                                               const DownDev* __restrict__ D2, WsDev ws) {
+    pdl_trigger();
+    down_fix_cta<KS>(L, D2, ws);
+    pdl_wait();
 }
 
 // Logical 8-bit codes [d][f] (0 outside the cached / the significant channels) and parameters [d][f/G].

@@ -52,7 +52,7 @@ struct FfnParams {
     int n_rb;                // 256-row weight blocks of the matrix
     int n_experts;
     int32_t* work_ctr;       // device counter of this launch's work queue (zeroed by the scan kernel)
-    int fills;               // launched behind the pair kernel on the same forward: see pdl_trigger
+    int fills, leads;        // the launch before, the one behind does not wait for this one's start: see pdl_trigger
     int sectioned;           // items ordered by tile count first (batches where an expert can have more than 32 rows)
 };
 
@@ -363,8 +363,8 @@ __device__ __forceinline__ bool consume_dispatch(const FfnParams& p, FfnSmem* S,
 
 template <bool GATEUP, int MAXNT8, int G>
 __device__ __forceinline__ void stream_cta(const FfnParams& p, uint8_t* smem) {
-    // after an expired wait nothing new starts; one answer for the CTA, for a kernel beside this one may write the word
-    if (__syncthreads_or(*p.ws.status & STATUS_TIMEOUT)) return;
+    // after an expired wait nothing new starts; beside the pair kernel, which may write the word, one answer for the CTA
+    if (MAXNT8 == 3 ? __syncthreads_or(*p.ws.status & STATUS_TIMEOUT) : *p.ws.status & STATUS_TIMEOUT) return;
     const LayerDev* L = p.L;
     FfnSmem* S = reinterpret_cast<FfnSmem*>(smem);
     uint8_t* stages = smem + SMEM_HEADER;
@@ -578,8 +578,9 @@ template <bool GATEUP, int MAXNT8, int G>
 __global__ void __launch_bounds__(FFN_THREADS, (MAXNT8 <= 2 && APW == 2) ? 3 : 2) ffn_stream_kernel(const FfnParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
     const bool fills = MAXNT8 == 3 && p.fills;
+    if (!fills && p.leads) pdl_wait();
     pdl_trigger();
-    if (!fills) pdl_wait();
+    if (!fills && !p.leads) pdl_wait();
     stream_cta<GATEUP, MAXNT8, G>(p, smem);
     if (fills) pdl_wait();
 }
@@ -599,14 +600,15 @@ static cudaError_t launch_one(const FfnParams& p, int n_ctas, int G, cudaStream_
 }
 
 // tiles: 8-token tiles of the kernel variant (1..3); n_items: about how many items the launch has; long_rows: an expert
-// can have more than 32 rows; fills: the launch before is the pair kernel's, on other experts.
+// can have more than 32 rows; fills: the launch before is the pair kernel's, on other experts; leads: the
+// launch behind starts beside this one.
 //
 // Three CTAs per SM hide more of each other's latencies, two have rings half as large again and leave room for the next
 // kernel's CTAs: three pay once every one has an item (1, 2, 3 and 4 tokens of a Mixtral-shaped layer: 68, 107, 130, 130
 // us a pass with two, 81, 104, 114, 114 with three; fine-grained, 4 and 16 tokens: 50 and 76, 61 and 72; 512-wide layer
 // of 64 tokens: 29 and 38).  The kernel of three tiles needs the registers of two.
 cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
-                              long long split_stride, int tiles, long long n_items, bool long_rows, bool fills,
+                              long long split_stride, int tiles, long long n_items, bool long_rows, bool fills, bool leads,
                               int n_sms, int G, cudaStream_t st) {
     const bool three = tiles < 3 && APW == 2 && n_items > 3 * n_sms;
     const int smem_bytes = three ? 74 * 1024 : 110 * 1024;
@@ -623,6 +625,7 @@ cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, in
     p.n_experts = n_experts;
     p.work_ctr = ws.status + (gateup ? 4 : 5);
     p.fills = fills;
+    p.leads = leads;
     p.sectioned = (long_rows && n_experts <= MAX_SECT_EXPERTS) ? 1 : 0;   // measured: +3 % at 64 tokens, -1 % at 32
     if (tiles == 1) return gateup ? launch_one<true, 1>(p, n_ctas, G, st) : launch_one<false, 1>(p, n_ctas, G, st);
     if (tiles == 2) return gateup ? launch_one<true, 2>(p, n_ctas, G, st) : launch_one<false, 2>(p, n_ctas, G, st);
