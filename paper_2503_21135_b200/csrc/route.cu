@@ -699,8 +699,8 @@ __global__ void __launch_bounds__(256) upload_kernel(const uint4* __restrict__ x
 
 // grid (T, ceil(d / 1024)): each thread owns four output columns of one token.  KS > 0: every expert's result is in KS
 // copies of ypart (the K splits, known to the compiler, no lookups in front of their loads: 8 tokens of 4096 in 8 splits
-// 6.0 -> 5.2 us); 0: any forward.
-template <int KS>
+// 6.0 -> 5.2 us); 0: any forward, the first copies of U of a token's rows (U divides their number) loaded at once.
+template <int KS, int U>
 __global__ void __launch_bounds__(256) combine_kernel(WsDev ws, int d, int k, int Es, void* __restrict__ y,
                                                       int y_f32, long long split_stride, int n_experts) {
     pdl_prologue();
@@ -727,19 +727,29 @@ __global__ void __launch_bounds__(256) combine_kernel(WsDev ws, int d, int k, in
             for (int i = 0; i < 4; ++i) acc[i] = fmaf(w, s[i], acc[i]);
         }
     }
-    for (int j = KS > 0 ? kk : 0; j < kk; ++j) {
-        const int r = ws.pos[t * kk + j];
-        const float w = (j < k) ? ws.topk_w[t * k + j] : 1.0f;
-        float s[4] = {0.f, 0.f, 0.f, 0.f};
-        const int e = ws.row_expert[r];
-        const int ns = (ws.counts[e] > ws.tc_min) ? 1 : ws.ksplit;  // the tensor-core path does not split K
-        for (int sp = 0; sp < ns; ++sp) {
-            const float4 v =
-                *reinterpret_cast<const float4*>(ypart_row(ws, sp, split_stride, e, n_experts, r, ws.off_pad[e], d) + c);
-            s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
-        }
+    for (int j0 = KS > 0 ? kk : 0; j0 < kk; j0 += U) {
+        int r[U];
+        float4 s[U];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] = fmaf(w, s[i], acc[i]);
+        for (int u = 0; u < U; ++u) r[u] = ws.pos[t * kk + j0 + u];
+#pragma unroll
+        for (int u = 0; u < U; ++u) s[u] = *reinterpret_cast<const float4*>(ws.ypart + (long long)r[u] * d + c);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int j = j0 + u;
+            const float w = (j < k) ? ws.topk_w[t * k + j] : 1.0f;
+            const int e = ws.row_expert[r[u]];
+            const int ns = (ws.counts[e] > ws.tc_min) ? 1 : ws.ksplit;  // the tensor-core path does not split K
+            for (int sp = 1; sp < ns; ++sp) {
+                const float4 v = *reinterpret_cast<const float4*>(
+                    ypart_row(ws, sp, split_stride, e, n_experts, r[u], ws.off_pad[e], d) + c);
+                s[u].x += v.x; s[u].y += v.y; s[u].z += v.z; s[u].w += v.w;
+            }
+            acc[0] = fmaf(w, s[u].x, acc[0]);
+            acc[1] = fmaf(w, s[u].y, acc[1]);
+            acc[2] = fmaf(w, s[u].z, acc[2]);
+            acc[3] = fmaf(w, s[u].w, acc[3]);
+        }
     }
     if (y_f32) {
         *reinterpret_cast<float4*>((float*)y + (long long)t * d + c) = make_float4(acc[0], acc[1], acc[2], acc[3]);
@@ -797,10 +807,13 @@ cudaError_t launch_upload(const void* xh, void* xd, long long x_bytes, const flo
 cudaError_t launch_combine(const WsDev& ws, int d, int k, int Es, void* y, int y_f32, long long split_stride,
                            int n_experts, cudaStream_t st) {
     const bool uniform = ws.tc_min == 0x7fffffff && !ws.ysmall;
-    auto kernel = uniform && ws.ksplit == 8   ? combine_kernel<8>
-                  : uniform && ws.ksplit == 2 ? combine_kernel<2>
-                  : uniform && ws.ksplit == 1 ? combine_kernel<1>
-                                              : combine_kernel<0>;
+    auto kernel = uniform && ws.ksplit == 8   ? combine_kernel<8, 1>
+                  : uniform && ws.ksplit == 4 ? combine_kernel<4, 1>
+                  : uniform && ws.ksplit == 2 ? combine_kernel<2, 1>
+                  : uniform && ws.ksplit == 1 ? combine_kernel<1, 1>
+                                              : (k + Es) % 4 == 0         ? combine_kernel<0, 4>
+                  : (k + Es) % 2 == 0         ? combine_kernel<0, 2>
+                                              : combine_kernel<0, 1>;
     return launch_pdl(kernel, dim3((unsigned)ws.T, (unsigned)((d + 1023) / 1024)), dim3(256), 0, st, ws, d, k, Es, y, y_f32,
                       split_stride, n_experts);
 }
