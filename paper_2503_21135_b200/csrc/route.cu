@@ -384,44 +384,54 @@ __device__ __forceinline__ void gather_row(const LayerDev* __restrict__ L, const
     const float sc1 = __uint_as_float((uint32_t)(127 + x_scale_exp(bits, 4 * lane + 2)) << 23);
     const int rg = row >> 3, rr = row & 7;
     bool clamped = false;
-    for (int c = part; c < n_kc; c += n_parts) {
-        const int k0 = c * KC + lane * 4;
-        float v[4] = {0.f, 0.f, 0.f, 0.f};
-        if (t >= 0) {
-            const uint2 raw = *reinterpret_cast<const uint2*>(xr + k0);
-            const __nv_bfloat162 p0 = *reinterpret_cast<const __nv_bfloat162*>(&raw.x);
-            const __nv_bfloat162 p1 = *reinterpret_cast<const __nv_bfloat162*>(&raw.y);
-            v[0] = __low2float(p0); v[1] = __high2float(p0); v[2] = __low2float(p1); v[3] = __high2float(p1);
+    // four chunks at a time, their loads in flight together: a chunk's load, mask and sum are a chain of latencies
+    for (int c0 = part; c0 < n_kc; c0 += 4 * n_parts) {
+        uint2 raw[4];
+        uint32_t mw[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = clamp_act(v[i], clamped);
-            if (sw) {
-                const uint32_t mw = mask[k0 >> 5] >> (k0 & 31);
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if ((mw >> i) & 1u) v[i] = 0.f;
+        for (int u = 0; u < 4; ++u) {
+            const int c = c0 + u * n_parts, k0 = c * KC + lane * 4;
+            raw[u] = make_uint2(0u, 0u);
+            mw[u] = 0u;
+            if (c < n_kc && t >= 0) {
+                raw[u] = *reinterpret_cast<const uint2*>(xr + k0);
+                if (sw) mw[u] = __ldg(mask + (k0 >> 5)) >> (k0 & 31);
             }
         }
-        float hv[4];
-        float sum = 0.f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            hv[i] = __half2float(__float2half_rn(v[i]));
-            sum += hv[i];
-        }
-        // sum over the 16 lanes of each half chunk (64 k), fixed butterfly order
+        for (int u = 0; u < 4; ++u) {
+            const int c = c0 + u * n_parts;
+            if (c >= n_kc) break;
+            const __nv_bfloat162 p0 = *reinterpret_cast<const __nv_bfloat162*>(&raw[u].x);
+            const __nv_bfloat162 p1 = *reinterpret_cast<const __nv_bfloat162*>(&raw[u].y);
+            float v[4] = {__low2float(p0), __high2float(p0), __low2float(p1), __high2float(p1)};
 #pragma unroll
-        for (int o = 8; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        const __half2 oa = __floats2half2_rn(hv[0] * sc0, hv[1] * sc0), ob = __floats2half2_rn(hv[2] * sc1, hv[3] * sc1);
-        uint2 packed;
-        packed.x = *reinterpret_cast<const uint32_t*>(&oa);
-        packed.y = *reinterpret_cast<const uint32_t*>(&ob);
-        if (!tc) {
-            uint8_t* out = ws.xperm + act_off(c, row, ws.Rcap);
-            *reinterpret_cast<uint2*>(out + lane * 8) = packed;
-            if ((lane & 15) == 0) *reinterpret_cast<float*>(out + XROW_SUM_OFF + (lane >> 4) * 4) = sum;
-        } else {
-            uint8_t* out = ws.xperm + tile_off(c, seg0, (row - seg0) >> 3, ws.Rcap);
-            *reinterpret_cast<uint2*>(out + (lane >> 1) * 128 + rr * 16 + (lane & 1) * 8) = packed;
+            for (int i = 0; i < 4; ++i) {
+                v[i] = clamp_act(v[i], clamped);
+                if ((mw[u] >> i) & 1u) v[i] = 0.f;
+            }
+            float hv[4];
+            float sum = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                hv[i] = __half2float(__float2half_rn(v[i]));
+                sum += hv[i];
+            }
+            // sum over the 16 lanes of each half chunk (64 k), fixed butterfly order
+#pragma unroll
+            for (int o = 8; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            const __half2 oa = __floats2half2_rn(hv[0] * sc0, hv[1] * sc0), ob = __floats2half2_rn(hv[2] * sc1, hv[3] * sc1);
+            uint2 packed;
+            packed.x = *reinterpret_cast<const uint32_t*>(&oa);
+            packed.y = *reinterpret_cast<const uint32_t*>(&ob);
+            if (!tc) {
+                uint8_t* out = ws.xperm + act_off(c, row, ws.Rcap);
+                *reinterpret_cast<uint2*>(out + lane * 8) = packed;
+                if ((lane & 15) == 0) *reinterpret_cast<float*>(out + XROW_SUM_OFF + (lane >> 4) * 4) = sum;
+            } else {
+                uint8_t* out = ws.xperm + tile_off(c, seg0, (row - seg0) >> 3, ws.Rcap);
+                *reinterpret_cast<uint2*>(out + (lane >> 1) * 128 + rr * 16 + (lane & 1) * 8) = packed;
+            }
         }
     }
     if (clamped && ws.status) atomicOr(ws.status, STATUS_RANGE);
@@ -568,6 +578,7 @@ __global__ void __launch_bounds__(256) gather_group_kernel(const LayerDev* __res
 // counting sort of all T * k pairs in shared memory (a few hundred pairs at most), then gathers its own row; CTA 0
 // also writes the routing outputs and the row tables the later kernels read.  Same results as the three kernels.
 constexpr int FRONT_MAX_PAIRS = 128;
+constexpr int FRONT_BATCHES = FRONT_MAX_PAIRS / 32;
 constexpr int FRONT_MAX_TOKENS = 16;   // beyond this the three separate kernels are faster (measured at 32 and 64 tokens)
 __global__ void __launch_bounds__(256) front_kernel(const LayerDev* __restrict__ L, WsDev ws,
                                                     const __nv_bfloat16* __restrict__ x,
@@ -575,24 +586,34 @@ __global__ void __launch_bounds__(256) front_kernel(const LayerDev* __restrict__
     __shared__ int s_idx[FRONT_MAX_PAIRS];
     __shared__ float s_w[FRONT_MAX_PAIRS];
     __shared__ int s_rank[FRONT_MAX_PAIRS];
+    __shared__ int s_hist[FRONT_BATCHES][MAX_EXPERTS];
     __shared__ int s_count[MAX_EXPERTS + 1], s_off[MAX_EXPERTS + 1], s_pad[MAX_EXPERTS + 1];
     __shared__ int s_row_e, s_row_t;
     pdl_prologue();
     const int T = ws.T, n_pairs = T * k, kk = k + Es;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int t = warp; t < T; t += 8) topk_token(logits + (long long)t * E, lane, E, k, renorm, t, s_idx, s_w);
+    for (int i = threadIdx.x; i < FRONT_BATCHES * E; i += blockDim.x) s_hist[i / E][i % E] = 0;
     if (threadIdx.x == 0) { s_row_e = -1; s_row_t = -1; }
     __syncthreads();
-    // counting sort: thread e walks the pairs in order (pair i = t*k + j ascends in t: the stable order)
+    // counting sort (pair i = t*k + j ascends in t: the stable order), one warp per 32 pairs: a pair's rank is the number
+    // of its expert's pairs in the batches before its own, plus those on lower lanes
+    const unsigned same = __match_any_sync(0xffffffffu, threadIdx.x < n_pairs ? s_idx[threadIdx.x] : -1);
+    const int below = __popc(same & ((1u << lane) - 1));
+    if (threadIdx.x < n_pairs && below == 0) s_hist[warp][s_idx[threadIdx.x]] = __popc(same);
+    __syncthreads();
     for (int e = threadIdx.x; e < E + Es; e += blockDim.x) {
-        int c = 0;
+        int c = e < E ? 0 : T;
         if (e < E) {
-            for (int i = 0; i < n_pairs; ++i)
-                if (s_idx[i] == e) s_rank[i] = c++;
-        } else {
-            c = T;
+#pragma unroll
+            for (int b = 0; b < FRONT_BATCHES; ++b) c += s_hist[b][e];
         }
         s_count[e] = c;
+    }
+    if (threadIdx.x < n_pairs) {
+        int r = below;
+        for (int b = 0; b < warp; ++b) r += s_hist[b][s_idx[threadIdx.x]];
+        s_rank[threadIdx.x] = r;
     }
     __syncthreads();
     if (warp == 0) {
