@@ -29,7 +29,8 @@ __device__ __forceinline__ float order_value(uint32_t k) {
 // Top-k of one token's logits held across a warp (lane l holds logits l, l+32, ..., NV of them; E <= 32 NV): k largest
 // raw logits, descending, ties -> lower expert index; weights = softmax over all E restricted to the chosen,
 // rescaled to sum 1 if `renorm`.  A round of the selection is two warp reductions in hardware (with ten shuffles and
-// eight candidates a lane whatever E is, the front kernel took 24.5 us at 16 tokens, 64 experts, top-6; now 13.6).
+// eight candidates a lane whatever E is, the front kernel took 24.5 us at 16 tokens, 64 experts, top-6; 13.6 so), and
+// the weights are worked out once behind the rounds, a lane each (the pass of those 16 tokens 68.5 -> 65.8 us).
 template <int NV>
 __device__ __forceinline__ void topk_softmax_store(float (&v)[NV], int lane, int E, int k, int renorm, long long token,
                                                    int32_t* __restrict__ topk_idx, float* __restrict__ topk_w) {
@@ -45,7 +46,7 @@ __device__ __forceinline__ void topk_softmax_store(float (&v)[NV], int lane, int
 #pragma unroll
     for (int o = 16; o; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
 
-    float my_w = 0.f, wsum = 0.f;   // lane j keeps the j-th choice
+    uint32_t my_key = 0u;   // lane j keeps the j-th choice
     int my_i = 0;
     for (int j = 0; j < k; ++j) {
         // local best (value desc, index asc)
@@ -62,13 +63,15 @@ __device__ __forceinline__ void topk_softmax_store(float (&v)[NV], int lane, int
 #pragma unroll
         for (int i = 0; i < NV; ++i)
             if (lane + 32 * i == bi) v[i] = -INFINITY;
-        const float w = expf(order_value(best) - mx) / den;
         if (lane == j) {
             my_i = bi;
-            my_w = w;
+            my_key = best;
         }
-        wsum += w;
     }
+    const float my_w = lane < k ? expf(order_value(my_key) - mx) / den : 0.f;
+    float wsum = 0.f;
+    if (renorm)
+        for (int j = 0; j < k; ++j) wsum += __shfl_sync(0xffffffffu, my_w, j);   // in the order of the choices
     if (lane < k) {
         topk_idx[token * k + lane] = my_i;
         topk_w[token * k + lane] = renorm ? my_w / wsum : my_w;
@@ -470,7 +473,7 @@ __device__ __forceinline__ void gather_row(const LayerDev* __restrict__ L, const
 
 __global__ void __launch_bounds__(256) gather_kernel(const LayerDev* __restrict__ L, WsDev ws,
                                                      const __nv_bfloat16* __restrict__ x) {
-    pdl_prologue();
+    pdl_wait();   // no early start for the next kernel: see front_kernel
     const int row = blockIdx.x;
     if (row >= ws.off_pad[L->E + L->Es]) return;
     const int e = ws.row_expert[row];
@@ -577,9 +580,8 @@ __global__ void __launch_bounds__(256) gather_group_kernel(const LayerDev* __res
 // whole forward takes tens of microseconds).  One CTA per physical row; every CTA repeats the routing and the
 // counting sort of all T * k pairs in shared memory (a few hundred pairs at most), then gathers its own row; CTA 0
 // also writes the routing outputs and the row tables the later kernels read.  Same results as the three kernels.
-constexpr int FRONT_MAX_PAIRS = 128;
+constexpr int FRONT_MAX_PAIRS = 96;
 constexpr int FRONT_BATCHES = FRONT_MAX_PAIRS / 32;
-constexpr int FRONT_MAX_TOKENS = 16;   // beyond this the three separate kernels are faster (measured at 32 and 64 tokens)
 __global__ void __launch_bounds__(256) front_kernel(const LayerDev* __restrict__ L, WsDev ws,
                                                     const __nv_bfloat16* __restrict__ x,
                                                     const float* __restrict__ logits, int E, int Es, int k, int renorm) {
@@ -589,7 +591,11 @@ __global__ void __launch_bounds__(256) front_kernel(const LayerDev* __restrict__
     __shared__ int s_hist[FRONT_BATCHES][MAX_EXPERTS];
     __shared__ int s_count[MAX_EXPERTS + 1], s_off[MAX_EXPERTS + 1], s_pad[MAX_EXPERTS + 1];
     __shared__ int s_row_e, s_row_t;
-    pdl_prologue();
+    // No early start for the next kernel: a streaming CTA has nine warps, seven of which a quarter of an SM's registers
+    // holds, so three of them fit only if their odd warps fall on different quarters.  CTAs that settled beside this
+    // kernel's took other places, and the third waited for the first two to end, 70 us later, on 20 of 148 SMs (8 and 16
+    // tokens of 4096: 166 and 4 x 180 us, 157 and 4 x 174 without; 64 tokens of 512: 28 and 25.5).
+    pdl_wait();
     const int T = ws.T, n_pairs = T * k, kk = k + Es;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int t = warp; t < T; t += 8) topk_token(logits + (long long)t * E, lane, E, k, renorm, t, s_idx, s_w);
@@ -812,7 +818,10 @@ cudaError_t launch_gather(const LayerDev* L, const WsDev& ws, const void* x, int
     }
     return launch_pdl(gather_kernel, dim3((unsigned)ws.Rpad), dim3(256), 0, st, L, ws, (const __nv_bfloat16*)x);
 }
-bool front_fits(int T, int k) { return T <= FRONT_MAX_TOKENS && T * k <= FRONT_MAX_PAIRS; }
+// Beyond this the three kernels are faster: top-2 of 8 experts, 20, 24, 32, 48, 64 tokens of 4096: 172, 173, 210, 237, 245 us a
+// pass with this kernel, 180, 180, 210, 234, 241 with three (512-wide: 24 and 32 tokens 26 and 27, 32 and 31; 64: 31, 28);
+// top-6 of 64: 8, 16, 20 tokens 53.8, 65.8, 75 and 57.1, 65.5, 70.
+bool front_fits(int T, int k) { return T <= 32 && T * k <= FRONT_MAX_PAIRS; }
 cudaError_t launch_front(const LayerDev* L, const WsDev& ws, const void* x, const float* logits, int E, int Es, int k,
                          int renorm, cudaStream_t st) {
     return launch_pdl(front_kernel, dim3((unsigned)ws.Rpad), dim3(256), 0, st, L, ws, (const __nv_bfloat16*)x, logits, E,
