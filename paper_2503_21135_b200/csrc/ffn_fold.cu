@@ -631,16 +631,14 @@ __device__ __noinline__ void ff_fold_role(const FfParams& p, FfRole R, uint8_t* 
     FfPos pos;
     for (int g = blockIdx.x; g < R.total && ok; g += gridDim.x, ++ic) {
         const FfItem im = ff_item_uni(p.ksplit, R.tab, g, cur, R.n_kc);
-        if (NT == 16 || im.n_mma <= 16) {
+        if (im.n_mma <= 16)
             ok = ff_fold_item<GATEUP, 16, NT, NB, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
-        } else if constexpr (NT >= 32) {
-            if (NT == 32 || im.n_mma <= 32)
-                ok = ff_fold_item<GATEUP, 32, NT, NB, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
-            else if (im.n_mma <= 48)
-                ok = ff_fold_item<GATEUP, 48, NT, NB, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
-            else
-                ok = ff_fold_item<GATEUP, NT, NT, NB, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
-        }
+        else if (im.n_mma <= 32)
+            ok = ff_fold_item<GATEUP, 32, NT, NB, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
+        else if (im.n_mma <= 48)
+            ok = ff_fold_item<GATEUP, 48, NT, NB, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
+        else
+            ok = ff_fold_item<GATEUP, NT, NT, NB, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
     }
     if (clamped) atomicOr(p.ws.status, STATUS_RANGE);
 }
@@ -708,8 +706,7 @@ __device__ __noinline__ void ff_mma_role(const FfParams& p, FfRole R) {
 
 template <bool GATEUP, int NT, int G>
 __global__ void __launch_bounds__(FF_THREADS, 1) ffn_fold_kernel(const __grid_constant__ FfParams p) {
-    constexpr int NA = NT == 64 ? 2 : 3;
-    constexpr int NB = NT == 16 ? 4 : 2;
+    constexpr int NA = 2, NB = 2;
     static_assert(128 * NA + 2 * NT * NB <= (int)FF_TMEM_COLS, "tensor memory");
     extern __shared__ __align__(1024) uint8_t smem[];
     FfShared* S = reinterpret_cast<FfShared*>(smem);

@@ -1,8 +1,8 @@
 // Streaming grouped dequant-GEMM for small token counts per expert (decode path, and the generic
 // fallback for any size): HBM-bound, judged on packed-weight bytes per second.
 //
-// PERSISTENT grid (two or three CTAs per SM).  A work item = one (expert, 256-row weight block, chunk of <= 24
-// tokens, K split); items are ordered costliest first (most 8-token tiles first from 33 rows per expert on, then
+// PERSISTENT grid (two or three CTAs per SM).  A work item = one (expert, 256-row weight block, chunk of <= 8,
+// 16 or 24 tokens by the variant, K split); items are ordered costliest first (most 8-token tiles first from 33 rows per expert on, then
 // heaviest bit-width) and handed out from a device counter, a CTA's first item statically.  Inside a CTA ONE
 // producer thread streams the packed blocks (codes + params, contiguous per 256 x 128 block) and the matching
 // activation slices into a shared-memory ring with bulk async copies completing on mbarriers; it runs ahead across
