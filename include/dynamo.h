@@ -151,8 +151,9 @@ dynamo_status dynamo_set_switch_mode(dynamo_ctx* ctx, int32_t mode);
  *   x             : dev bf16 [T, d], 16-byte aligned (as y must be; misaligned -> ERR_ALIGN)
  *   router_logits : dev fp32 [T, E]   (the router GEMM is outside this path)
  *   y             : dev [T, d], bf16 or fp32 per y_dtype
- * topk = the k largest logits (ties -> lower index), weights = softmax over all E restricted to
- * the chosen k (rescaled to sum 1 if renormalize).  y[t] = sum_j w[t,j] * FFN_{e_j}(x[t]) +
+ * topk = the k largest logits (ties -> lower index; k different experts whatever the logits are: masked ones
+ * (-infinity) follow the others, a NaN follows every number), weights = softmax over all E restricted to
+ * the chosen k (rescaled to sum 1 if renormalize; NaN for a token with a NaN logit).  y[t] = sum_j w[t,j] * FFN_{e_j}(x[t]) +
  * sum_shared FFN_s(x[t]), summed in fp32 in that order.  T = 0 is a no-op. */
 dynamo_status dynamo_moe_forward(dynamo_ctx* ctx, const void* x, const float* router_logits, int32_t T,
                                  void* y, int32_t y_dtype, const dynamo_debug_out* dbg, void* stream);

@@ -14,21 +14,13 @@
 
 #include "common.cuh"
 #include "layout.cuh"
+#include "topk_rule.h"
 
 namespace dyn {
 
-// Order-preserving map of a float to an unsigned integer (-0 counts as +0) and back.
-__device__ __forceinline__ uint32_t order_key(float v) {
-    const uint32_t b = __float_as_uint(v + 0.f);
-    return b ^ ((b >> 31) ? 0xffffffffu : 0x80000000u);
-}
-__device__ __forceinline__ float order_value(uint32_t k) {
-    return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xffffffffu));
-}
-
 // Top-k of one token's logits held across a warp (lane l holds logits l, l+32, ..., NV of them; E <= 32 NV): k largest
-// raw logits, descending, ties -> lower expert index; weights = softmax over all E restricted to the chosen,
-// rescaled to sum 1 if `renorm`.  A round of the selection is two warp reductions in hardware (with ten shuffles and
+// raw logits in the order of topk_rule.h, ties -> lower expert index; weights = softmax over all E restricted to the
+// chosen, rescaled to sum 1 if `renorm`.  A round of the selection is two warp reductions in hardware (with ten shuffles and
 // eight candidates a lane whatever E is, the front kernel took 24.5 us at 16 tokens, 64 experts, top-6; 13.6 so), and
 // the weights are worked out once behind the rounds, a lane each (the pass of those 16 tokens 68.5 -> 65.8 us).
 template <int NV>
@@ -46,29 +38,32 @@ __device__ __forceinline__ void topk_softmax_store(float (&v)[NV], int lane, int
 #pragma unroll
     for (int o = 16; o; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
 
-    uint32_t my_key = 0u;   // lane j keeps the j-th choice
+    // The selection works on keys: a taken expert is marked, not given a value that a logit may have, and a NaN has a
+    // place in the order, so the k choices are k different experts whatever the logits are (masked with -infinity, NaN).
+    uint32_t key[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) key[i] = lane + 32 * i < E ? topk_key(v[i]) : TOPK_TAKEN;
+    uint32_t my_key = TOPK_NAN;   // lane j keeps the j-th choice
     int my_i = 0;
     for (int j = 0; j < k; ++j) {
         // local best (value desc, index asc)
-        float bv = -INFINITY;
-        int bi = 0x7fffffff;
+        uint32_t bk = key[0];
+        int bi = lane;
 #pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            const int e = lane + 32 * i;
-            if (e < E && (v[i] > bv || (v[i] == bv && e < bi))) { bv = v[i]; bi = e; }
-        }
-        const uint32_t key = order_key(bv), best = __reduce_max_sync(0xffffffffu, key);
-        bi = (int)__reduce_min_sync(0xffffffffu, key == best ? (uint32_t)bi : 0x7fffffffu);
+        for (int i = 1; i < NV; ++i)
+            if (key[i] > bk) { bk = key[i]; bi = lane + 32 * i; }
+        const uint32_t best = __reduce_max_sync(0xffffffffu, bk);
+        bi = (int)__reduce_min_sync(0xffffffffu, bk == best ? (uint32_t)bi : 0x7fffffffu);
         // remove the winner from its owner's candidates
 #pragma unroll
         for (int i = 0; i < NV; ++i)
-            if (lane + 32 * i == bi) v[i] = -INFINITY;
+            if (lane + 32 * i == bi) key[i] = TOPK_TAKEN;
         if (lane == j) {
             my_i = bi;
             my_key = best;
         }
     }
-    const float my_w = lane < k ? expf(order_value(my_key) - mx) / den : 0.f;
+    const float my_w = lane < k ? expf(topk_value(my_key) - mx) / den : 0.f;
     float wsum = 0.f;
     if (renorm)
         for (int j = 0; j < k; ++j) wsum += __shfl_sync(0xffffffffu, my_w, j);   // in the order of the choices

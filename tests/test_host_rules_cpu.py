@@ -1,0 +1,87 @@
+"""Rules that the kernels and the host entry share with plain C++ (headers under csrc/), compiled here for the CPU."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import oracle
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2503_21135_b200", "csrc")
+
+
+def _compile(tmp_path_factory, name, source):
+    d = tmp_path_factory.mktemp(name)
+    src, lib = str(d / "shim.cpp"), str(d / "shim.so")
+    with open(src, "w") as f:
+        f.write(source)
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-Wall", "-Werror", "-shared", "-fPIC", "-I", CSRC, "-o", lib, src])
+    return ctypes.CDLL(lib)
+
+
+@pytest.fixture(scope="module")
+def topk(tmp_path_factory):
+    """The rounds of the device's selection over the keys of one token."""
+    lib = _compile(tmp_path_factory, "topk", """
+        #include "topk_rule.h"
+        extern "C" void select(const float* l, int E, int k, int* idx) {
+            uint32_t key[256];
+            for (int e = 0; e < E; ++e) key[e] = dyn::topk_key(l[e]);
+            for (int j = 0; j < k; ++j) {
+                int b = 0;
+                for (int e = 1; e < E; ++e) if (key[e] > key[b]) b = e;
+                idx[j] = b;
+                key[b] = dyn::TOPK_TAKEN;
+            }
+        }
+        extern "C" uint32_t key(float v) { return dyn::topk_key(v); }
+        extern "C" float value(uint32_t k) { return dyn::topk_value(k); }
+        """)
+    lib.key.restype, lib.key.argtypes = ctypes.c_uint32, [ctypes.c_float]
+    lib.value.restype, lib.value.argtypes = ctypes.c_float, [ctypes.c_uint32]
+
+    def select(logits, k):
+        lg = np.ascontiguousarray(logits, np.float32)
+        idx = np.empty((lg.shape[0], k), np.int32)
+        for t in range(lg.shape[0]):
+            row = np.ascontiguousarray(lg[t])
+            lib.select(row.ctypes.data_as(ctypes.c_void_p), lg.shape[1], k, idx[t].ctypes.data_as(ctypes.c_void_p))
+        return idx
+
+    return lib, select
+
+
+def test_keys_order_the_logits(topk):
+    lib, _ = topk
+    v = np.array([-np.inf, -3e38, -1.5, -1e-45, 0.0, 1e-45, 2.0, 3e38, np.inf], np.float32)
+    keys = [lib.key(x) for x in v]
+    assert keys == sorted(set(keys))
+    assert lib.key(-0.0) == lib.key(0.0)
+    assert [lib.value(k) for k in keys] == v.tolist()
+    for bits in (0x7fc00000, 0xffc00000, 0x7f800001, 0xffffffff):
+        nan = np.array([bits], np.uint32).view(np.float32)[0]
+        assert 0 < lib.key(nan) < keys[0] and np.isnan(lib.value(lib.key(nan)))
+
+
+@pytest.mark.parametrize("E,k", [(1, 1), (8, 2), (8, 8), (40, 3), (64, 6), (256, 8)])
+def test_selection_follows_the_oracle_and_stays_in_range(topk, E, k):
+    _, select = topk
+    rng = np.random.default_rng(E * 10 + k)
+    lg = rng.standard_normal((40, E)).astype(np.float32)
+    lg[5:10] = np.round(lg[5:10])                       # ties
+    lg[10:20][rng.random((10, E)) < 0.7] = -np.inf      # masked experts, fewer left than k among them
+    lg[20] = -np.inf
+    lg[21] = 0.0
+    lg[21, ::2] = -0.0
+    assert np.array_equal(select(lg, k), oracle.route(lg, k)[0])
+    nan = lg.copy()
+    nan[22:30][rng.random((8, E)) < 0.7] = np.nan
+    nan[30] = np.nan
+    nan[10:20][rng.random((10, E)) < 0.3] = np.nan
+    got = select(nan, k)
+    assert got.min() >= 0 and got.max() < E
+    assert all(len(set(row)) == k for row in got.tolist())
+    for t in range(40):                                 # numbers first, among them the order of the numbers alone
+        n = min(k, int(np.isfinite(nan[t]).sum()))
+        assert np.array_equal(got[t, :n], oracle.route(np.where(np.isnan(nan[t]), -np.inf, nan[t])[None], k)[0][0, :n])
