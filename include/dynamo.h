@@ -173,9 +173,11 @@ dynamo_status dynamo_moe_forward_router(dynamo_ctx* ctx, const void* x, const vo
                                         const float* router_bias, int32_t T, void* y, int32_t y_dtype,
                                         float* logits_out, const dynamo_debug_out* dbg, void* stream);
 
-/* Same forward with HOST buffers: copies x and the logits to the device, runs the forward,
- * copies y back and synchronises the stream before returning.  Pinned host memory makes the
- * copies asynchronous with respect to other streams; pageable memory works too. */
+/* Same forward with HOST buffers; synchronises the stream before returning.  Every kind of host memory works.
+ * Pageable buffers are copied to and from staging buffers in the workspace.  A page-locked buffer of up to 8 MB
+ * (x and the logits together, y by itself) that is 16-byte aligned and lies within ONE cudaHostAlloc allocation or
+ * cudaHostRegister registration is read or written by the kernels themselves; any other is copied.  The buffers must
+ * stay allocated and registered, x and the logits unchanged, until the call returns. */
 dynamo_status dynamo_moe_forward_host(dynamo_ctx* ctx, const void* x_host, const float* logits_host, int32_t T,
                                       void* y_host, int32_t y_dtype, void* stream);
 

@@ -5,8 +5,11 @@
 #include <new>
 #include <vector>
 
+#include <cuda.h>
+
 #include "../../include/dynamo.h"
 #include "common.cuh"
+#include "host_range.h"
 
 namespace dyn {
 cudaError_t launch_pack_blocks(const void* src_a, const void* src_b, int n_rows_blocks, int K, int G, int bits,
@@ -889,18 +892,43 @@ dynamo_status dynamo_moe_forward_router(dynamo_ctx* ctx, const void* x, const vo
     return forward_impl(ctx, x, nullptr, w_router, router_bias, logits_out, T, y, y_dtype, dbg, stream);
 }
 
-// The device's address of a page-locked host buffer, or NULL where there is none (pageable or device memory, a buffer
-// that is locked at one end only, an address that 16-byte accesses do not suit).
+// Start and size of the allocation or registration that a device address belongs to; false where the driver has none.
+// (The driver call is looked up at run time: the library loads on machines that have no driver.)
+static bool allocation_of(const void* dev, uint64_t* start, uint64_t* size) {
+    using Fn = CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+    static const Fn query = []() -> Fn {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return (Fn)fn;
+    }();
+    CUpointer_attribute what[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    CUdeviceptr s = 0;
+    size_t n = 0;
+    void* to[2] = {&s, &n};
+    if (!query || query(2, what, to, (CUdeviceptr)dev) != CUDA_SUCCESS) return false;
+    *start = (uint64_t)s;
+    *size = (uint64_t)n;
+    return true;
+}
+
+// The device's address of a page-locked host buffer, or NULL where there is none: pageable or device memory, an address
+// that 16-byte accesses do not suit, a buffer that no single allocation or registration covers (between two of them there
+// may be pages that are not locked, which a kernel must not touch).
 static void* mapped_address(const void* p, size_t bytes) {
-    cudaPointerAttributes a, b;
+    cudaPointerAttributes a;
     if (((uintptr_t)p & 15)) return nullptr;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
-        cudaPointerGetAttributes(&b, (const char*)p + bytes - 1) != cudaSuccess) {
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer ||
-        ((uintptr_t)a.devicePointer & 15) || (char*)b.devicePointer != (char*)a.devicePointer + (bytes - 1))
+    if (a.type != cudaMemoryTypeHost || !a.devicePointer || ((uintptr_t)a.devicePointer & 15)) return nullptr;
+    uint64_t start, size;
+    if (!allocation_of(a.devicePointer, &start, &size) || !range_covers(start, size, (uint64_t)(uintptr_t)a.devicePointer, bytes))
         return nullptr;
     return a.devicePointer;
 }

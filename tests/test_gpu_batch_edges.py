@@ -107,9 +107,14 @@ def test_host_buffers_of_every_kind(kind, T):
     ins = kind in ("pinned", "shifted")
     for dtype, code in ((torch.float32, binding.F32), (torch.bfloat16, binding.BF16)):
         y = buffer(torch.zeros((T, cfg.d_model), dtype=dtype), kind != "pageable")
+        before = gpu.kernel_launches()
         gpu.forward_host(buffer(x, ins), buffer(lg, ins), y, code)
+        launched = gpu.kernel_launches() - before
         assert gpu.poll_status() == 0
+        before = gpu.kernel_launches()
         assert torch.equal(y, gpu.forward(x.cuda(), lg.cuda(), code).cpu())
+        # one launch more where the kernels read the buffers themselves
+        assert launched - (gpu.kernel_launches() - before) == (1 if kind == "pinned" else 0)
 
 
 @pytest.mark.parametrize("large", [1, 3, 7])

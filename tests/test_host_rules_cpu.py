@@ -85,3 +85,28 @@ def test_selection_follows_the_oracle_and_stays_in_range(topk, E, k):
     for t in range(40):                                 # numbers first, among them the order of the numbers alone
         n = min(k, int(np.isfinite(nan[t]).sum()))
         assert np.array_equal(got[t, :n], oracle.route(np.where(np.isnan(nan[t]), -np.inf, nan[t])[None], k)[0][0, :n])
+
+
+@pytest.fixture(scope="module")
+def covers(tmp_path_factory):
+    lib = _compile(tmp_path_factory, "covers", """
+        #include "host_range.h"
+        extern "C" bool covers(uint64_t start, uint64_t size, uint64_t p, uint64_t bytes) {
+            return dyn::range_covers(start, size, p, bytes);
+        }
+        """)
+    lib.covers.restype, lib.covers.argtypes = ctypes.c_bool, [ctypes.c_uint64] * 4
+    return lib.covers
+
+
+def test_a_buffer_has_to_lie_within_one_registration(covers):
+    page = 4096
+    first, second = (16 * page, 2 * page), (24 * page, 2 * page)      # pages 18 .. 23 between them are not registered
+    assert covers(*first, 16 * page, 2 * page) and covers(*first, 17 * page, page) and covers(*first, 18 * page - 16, 16)
+    assert not covers(*first, 18 * page - 16, 17)
+    assert not covers(*first, 17 * page, second[0] + second[1] - 17 * page)   # both ends registered, the middle not
+    assert not covers(*second, 17 * page, second[0] + second[1] - 17 * page)
+    assert not covers(*first, 15 * page, 3 * page)
+    assert not covers(0, 0, 16 * page, 1) and not covers(*first, 16 * page, 2 ** 64 - 1)
+    top = 2 ** 64 - page
+    assert covers(top, page - 1, top, page - 1) and not covers(top, page - 1, top + 8, page)
