@@ -328,20 +328,31 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], 
 }
 
 // ---- programmatic dependent launch -----------------------------------------------------------
-// Every kernel of a forward is launched with the programmatic-stream-serialization attribute and
-// starts with pdl_prologue(): it lets the next kernel's CTAs be scheduled early (they park in their
-// own pdl_prologue) and then waits until the preceding kernel has completed and flushed its
-// memory, so launch latency overlaps the previous kernel's tail without changing the data flow.
-__device__ __forceinline__ void pdl_prologue() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-// A pair of launches that do not need each other's results.  The first waits, reads what the second may write (the status
-// word), and only then lets the second start: all that came before the pair has completed and flushed by the time that a
-// CTA of the second runs.  The second does not wait until its end, where every CTA does: whoever waits for its completion
-// has waited for both.  In between it takes the SMs that the first no longer fills.
+// Every kernel of a forward is launched with the programmatic-stream-serialization attribute.  What a kernel does first
+// decides how it overlaps its neighbours:
+//   pdl_prologue     lets the next kernel's CTAs be scheduled early (launch latency overlaps this kernel) and waits until the
+//                    preceding kernel has completed and flushed its memory: no change to the data flow (router, scan, group
+//                    gather, combine, and the streaming kernel where nothing runs beside it).
+//   pdl_wait alone   the next kernel starts behind this one's end (front and gather kernels, see front_kernel).
+//   pdl_wait, then pdl_trigger, and pdl_early_start in the next kernel: the two do not need each other's results and run
+//                    side by side.  The first waits, reads what the second may write (the status word), and only then lets
+//                    the second start: all that came before the pair has completed and flushed by the time that a CTA of
+//                    the second runs.  The second does not wait until its end, where every CTA does: whoever waits for its
+//                    completion has waited for both.  In between it takes the SMs that the first no longer fills (pair,
+//                    fold and streaming kernels in front; streaming, statistics and d_ff-correction kernels behind).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_prologue() {
+    pdl_trigger();
+    pdl_wait();
+}
+// What the second reads before its wait (rows and tables of the gather, h of the gate/up launches) has reached the L2 when
+// it starts: the grids that wrote it have completed.  Only its SM's first-level cache may still hold lines from before,
+// which a wait of its own would have dropped: an acquire fence in place of that.
+__device__ __forceinline__ void pdl_early_start() {   // every thread of the CTA
+    if (threadIdx.x == 0) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    __syncthreads();
+}
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,

@@ -229,6 +229,7 @@ template <int KS>
 __global__ void __launch_bounds__(FIX_THREADS) down_fix_kernel(const LayerDev* __restrict__ L,
                                                                const DownDev* __restrict__ D2, WsDev ws) {
     pdl_trigger();
+    pdl_early_start();
     down_fix_cta<KS>(L, D2, ws);
     pdl_wait();
 }

@@ -737,8 +737,8 @@ __global__ void __launch_bounds__(FF_THREADS, 1) ffn_fold_kernel(const __grid_co
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     // Everything above overlaps the tail of the preceding kernel.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait();
+    pdl_trigger();
 
     const LayerDev* L = p.L;
     int32_t* status = p.ws.status;

@@ -578,9 +578,15 @@ template <bool GATEUP, int MAXNT8, int G>
 __global__ void __launch_bounds__(FFN_THREADS, (MAXNT8 <= 2 && APW == 2) ? 3 : 2) ffn_stream_kernel(const FfnParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
     const bool fills = MAXNT8 == 3 && p.fills;
-    if (!fills && p.leads) pdl_wait();
-    pdl_trigger();
-    if (!fills && !p.leads) pdl_wait();
+    if (fills) {
+        pdl_trigger();
+        pdl_early_start();
+    } else if (p.leads) {
+        pdl_wait();
+        pdl_trigger();
+    } else {
+        pdl_prologue();
+    }
     stream_cta<GATEUP, MAXNT8, G>(p, smem);
     if (fills) pdl_wait();
 }

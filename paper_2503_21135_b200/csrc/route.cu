@@ -705,7 +705,7 @@ __global__ void __launch_bounds__(256) front_kernel(const LayerDev* __restrict__
 // it runs beside an earlier kernel.
 __global__ void __launch_bounds__(256) upload_kernel(const uint4* __restrict__ xh, uint4* __restrict__ xd, long long nx,
                                                      const float* __restrict__ lh, float* __restrict__ ld, long long nl) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_trigger();
     const long long i0 = (long long)blockIdx.x * 256 + threadIdx.x, step = (long long)gridDim.x * 256;
     for (long long i = i0; i < nl; i += step) ld[i] = lh[i];
     for (long long i = i0; i < nx; i += 4 * step) {

@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(256) stats_kernel(const LayerDev* __restrict__
                                                     const __nv_bfloat16* __restrict__ x, float* __restrict__ stats,
                                                     float* __restrict__ part, int32_t* __restrict__ ctr) {
     pdl_trigger();
+    pdl_early_start();
     stats_cta(L, ws, x, stats, part, ctr);
     pdl_wait();
 }

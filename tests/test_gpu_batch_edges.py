@@ -137,3 +137,59 @@ def test_small_experts_run_beside_large_ones(large):
         got = [gpu.forward(x, lg, binding.F32) for x, lg in runs]
         assert all(torch.equal(a, b) for a, b in zip(got, alone))
     assert gpu.poll_status() == 0 and gpu.debug_check_guards() == 0
+
+
+def _everything_on(cfg, gpu, ora):
+    """Hidden-unit sets on the d_ff side and activation statistics."""
+    wd = wl.layer_weights(cfg)[2]
+    pool_d = wl.cache_pool_down(cfg, 32)
+    sets_d = wl.sig_sets_down(cfg, pool_d, 16)
+    bits = np.array([[2, 3, 4, 8, 6][e % 5] for e in range(cfg.n_experts)] + [8] * cfg.n_shared, np.int32)
+    gpu.pack_down_cache(wd.cuda(), bits, pool_d, 16)
+    gpu.set_channel_switch_down(sets_d)
+    ora.enable_down_side(oracle.as_u16(wd))
+    ora.set_channel_switch_down(sets_d)
+    gpu.set_stats_collection(True)
+
+
+def _few_large_experts(T, shift):
+    """Router logits of a top-1 layer of eight experts: three of them with most of the tokens, five with a few."""
+    e = (np.where(np.arange(T) % 16 < 15, np.arange(T) % 3, 3 + np.arange(T) % 5) + shift) % 8
+    lg = torch.zeros((T, 8))
+    lg[torch.arange(T), torch.from_numpy(e)] = 4.0
+    return lg
+
+
+@pytest.mark.parametrize("T", [100, 700])   # fold kernel; pair and streaming kernels side by side
+def test_overlapping_launches_in_a_captured_graph(T):
+    cfg, gpu, ora = _layer(700, n_experts=8, top_k=1, group_size=128)
+    _everything_on(cfg, gpu, ora)
+    xs, ls = torch.zeros((T, cfg.d_model), dtype=torch.bfloat16, device="cuda"), torch.zeros((T, 8), device="cuda")
+    ys = torch.empty((T, cfg.d_model), device="cuda")
+    inputs = [(wl.activations(cfg, T, step=51 + i).cuda(), _few_large_experts(T, i).cuda()) for i in range(2)]
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        gpu.forward(xs, ls, binding.F32, y=ys)
+    torch.cuda.current_stream().wait_stream(side)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        gpu.forward(xs, ls, binding.F32, y=ys)
+        gpu.forward(xs, ls, binding.F32, y=ys)
+    for x, lg in inputs:
+        want, stats = [], []
+        for replay in (False, True):
+            gpu.select_significant(0, reset=True)
+            if replay:
+                xs.copy_(x)
+                ls.copy_(lg)
+                graph.replay()
+                want.append(ys.clone())
+            else:
+                gpu.forward(x, lg, binding.F32)
+                want.append(gpu.forward(x, lg, binding.F32))
+            stats.append(gpu.channel_stats().clone())
+        torch.cuda.synchronize()
+        assert torch.equal(want[0], want[1]) and torch.equal(stats[0], stats[1])
+    assert gpu.poll_status() == 0 and gpu.debug_check_guards() == 0
