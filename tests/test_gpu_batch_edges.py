@@ -123,12 +123,15 @@ def test_small_experts_run_beside_large_ones(large):
     wait in between give what each gives alone."""
     cfg, gpu, _ = _layer(700, n_experts=8, top_k=1, group_size=64)
     runs = []
-    for i, T in enumerate((700, 640, 300)):
+    for i, T in enumerate((700, 640, 520)):   # (up to 496 tokens one kernel takes all experts of this layer)
         e = np.where(np.arange(T) % 16 < 15, np.arange(T) % large, large + np.arange(T) % (8 - large))
         lg = torch.zeros((T, 8))
         lg[torch.arange(T), torch.from_numpy((e + i) % 8)] = 4.0
         x = wl.activations(cfg, T, step=36 + i).cuda()
         runs.append((x, lg.cuda()))
+    before = gpu.kernel_launches()
+    gpu.forward(*runs[-1], binding.F32)
+    assert gpu.kernel_launches() - before == 8   # the two kernels side by side
     alone = []
     for x, lg in runs:
         alone.append(gpu.forward(x, lg, binding.F32).clone())
@@ -158,6 +161,36 @@ def _few_large_experts(T, shift):
     lg = torch.zeros((T, 8))
     lg[torch.arange(T), torch.from_numpy(e)] = 4.0
     return lg
+
+
+@pytest.mark.parametrize("n_shared", [0, 1])
+def test_statistics_and_hidden_unit_sets_beside_the_pair_kernel(n_shared):
+    """Statistics start beside the gate/up kernels and use the down launch's output as scratch, the d_ff-side correction
+    starts beside the down kernels: forwards that follow one another without a wait, all against the oracle."""
+    cfg, gpu, ora = _layer(700, n_experts=8, top_k=1, group_size=64, n_shared=n_shared)
+    _everything_on(cfg, gpu, ora)
+    runs = [(wl.activations(cfg, T, step=41 + i), _few_large_experts(T, i)) for i, T in enumerate((700, 520, 633))]
+    dev = [(x.cuda(), lg.cuda()) for x, lg in runs]
+    before = gpu.kernel_launches()
+    outs = [gpu.forward(x, lg, binding.F32) for x, lg in dev]
+    assert gpu.kernel_launches() - before == 3 * 10   # pair and streaming kernels, statistics, correction
+    got = gpu.channel_stats().cpu().numpy().astype(np.float64)
+    torch.cuda.synchronize()
+    assert gpu.poll_status() == 0 and gpu.debug_check_guards() == 0
+    pool = wl.cache_pool(cfg)
+    stats, n_add = np.zeros((8, cfg.cache_size)), np.zeros(8)
+    for (x, lg), y in zip(runs, outs):
+        idx, _ = oracle.route(lg.numpy(), 1)
+        stats = oracle.channel_stats_update(stats, oracle.as_u16(x), idx, pool)
+        n_add += np.bincount(idx.ravel(), minlength=8) + 1
+        toks = np.arange(0, x.shape[0], 9, dtype=np.int32)
+        ref = ora.forward(oracle.as_u16(x), lg.numpy(), tokens=toks)["y"][toks]
+        assert rel_err(y.cpu().numpy()[toks], ref) <= TOL
+    # fp32 accumulation of n non-negative terms: |fl(sum) - sum| <= n * 2^-24 * sum
+    assert np.all(np.abs(got - stats) <= n_add[:, None] * 2.0 ** -24 * stats)
+    for _ in range(5):
+        again = [gpu.forward(x, lg, binding.F32) for x, lg in dev]
+        assert all(torch.equal(a, b) for a, b in zip(again, outs))
 
 
 @pytest.mark.parametrize("T", [100, 700])   # fold kernel; pair and streaming kernels side by side

@@ -123,7 +123,7 @@ def test_down_side_target_precision(lay, target):
             assert np.array_equal(q.cpu().numpy(), expect), e
             assert int(expect.max()) <= 2 ** hb[e] - 1
             assert np.array_equal(_u16(s), ref.s) and np.array_equal(_u16(m), ref.m), e
-        for T in (40, 200):                      # streaming kernel only; tcgen05 kernel for the popular experts
+        for T in (40, 200):                      # streaming kernel; fold kernel
             y, ref = _forward(lay, T, step=50 + T)
             assert rel_err(y.cpu().numpy(), ref) <= TOL
         # a target equal to the base bit-width: every difference is zero, the forward is the base forward bit for bit
