@@ -137,9 +137,10 @@ inline int stream_tiles(const dynamo_layer_desc& D, int T, int n_rb13, int n_sms
 //    95 and 90), of two where there would be fewer items than SMs, and none once the row blocks alone are half a
 //    thousand items (64 tokens 157 with 8, 116 with 2, 112 with 1).
 //  - The fold kernel's persistent CTAs want two items each (139 tokens 301 us with 8 splits, 292 with 2).
+inline int ksplit_beside_large(const dynamo_layer_desc& D) { return std::max(1, std::min(MAX_KSPLIT, D.d_ff / KC / 4)); }
 inline int ksplit_for(const dynamo_layer_desc& D, int T) {
     const int n_kc = D.d_ff / KC;
-    if (!decode_sized(D, T)) return std::max(1, std::min(MAX_KSPLIT, n_kc / 4));
+    if (!decode_sized(D, T)) return ksplit_beside_large(D);
     const int base = (active_experts(D, T) + D.n_shared) * (D.d_model / RB);   // items of one split
     int ks = n_kc / 4;
     if (fold_sized(D, T)) ks = std::min(ks, 296 / base);
@@ -285,7 +286,9 @@ void ws_layout(const dynamo_layer_desc& D, WsLayout& W) {
     const size_t ks = std::min<size_t>(MAX_KSPLIT, f / KC);
     const size_t small_rows = std::min<size_t>(R, DECODE_ROWS);
     W.ypart = take(std::max(Rp, ks * (small_rows + 8 * n)) * d * 4);   // fp32 rows of the down GEMM, per K split
-    W.ysmall = R > DECODE_ROWS ? take((ks - 1) * n * TC_MIN_ROWS * d * 4) : W.ypart;   // (unused below that size)
+    // splits behind the first of small experts beside large ones; only forwards of more than DECODE_ROWS rows have any
+    const size_t ks_small = R > DECODE_ROWS ? ksplit_beside_large(D) : 1;
+    W.ysmall = ks_small > 1 ? take((ks_small - 1) * n * TC_MIN_ROWS * d * 4) : W.ypart;
     W.stage_x = take(T * d * 2);
     W.stage_logits = take(T * (size_t)D.n_experts * 4);
     W.stage_y = take(T * d * 4);

@@ -68,6 +68,17 @@ def test_arena_bytes_and_bits_validation(lib):
     assert binding.dynamo_arena_bytes(ds, np.array(list(bits) + [8], np.int32))[0] == 0
 
 
+@pytest.mark.parametrize("d_ff,copies", [(512, 0), (1024, 1), (1408, 1), (2048, 3), (14336, 7)])
+def test_workspace_holds_no_more_partial_rows_than_a_forward_uses(lib, d_ff, copies):
+    """From 1025 rows on the workspace also holds the K splits behind the first of experts with up to 32 rows: as many as
+    the down GEMM takes there, a quarter of its 128-wide chunks and at most 8."""
+    kw = dict(d_model=2048, d_ff=d_ff, n_experts=64, n_shared=2, top_k=6, group_size=64)
+    bits = np.array([4] * 64 + [8] * 2, np.int32)
+    small, large = (binding.dynamo_arena_bytes(_desc(max_tokens=t, **kw), bits)[2] for t in (128, 129))
+    # (the other buffers grow by eight rows of inputs and hidden values)
+    assert copies * 66 * 32 * 2048 * 4 <= large - small <= copies * 66 * 32 * 2048 * 4 + (1 << 20)
+
+
 def test_cache_share_of_weight_storage(lib):
     # The channel cache of ~1 % of the channels costs about 1 % of the 16-bit weight storage
     # (the paper's 152.8 MB = 1.02 % figure is this ratio): P/d of the gate/up originals.
