@@ -349,7 +349,9 @@ dynamo_status dynamo_assign_bits(const double* x, int32_t n, int32_t dim, int32_
 
 /* Measurement hook: three cudaEvent_t handles (any may be NULL) that every following forward records on
  * its stream before the gate/up FFN launch, after it, and after the down FFN launch, so that a
- * harness can time the dominant kernels in place.  Pass NULLs to switch it off. */
+ * harness can time the dominant kernels in place.  With events installed the statistics kernel
+ * (dynamo_set_stats_collection) runs in front of the first one, in no interval, instead of beside
+ * the gate/up launch.  Pass NULLs to switch it off. */
 dynamo_status dynamo_set_profile_events(dynamo_ctx* ctx, void* before_gateup, void* after_gateup, void* after_down);
 
 /* Number of kernels the library launched through this context since creation (host counter). */

@@ -51,7 +51,7 @@ cudaError_t setup_ffn_tc2(int n_sms, int* clusters_out);
 cudaError_t launch_ffn_tc2(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int n_experts, int n_clusters,
                            cudaStream_t st);
 cudaError_t launch_stats(const LayerDev* L, const WsDev& ws, const void* x, float* stats, float* part, int32_t* ctr, int E,
-                         int n_slices, cudaStream_t st);
+                         int n_slices, int beside, cudaStream_t st);
 cudaError_t launch_select(const LayerDev* L, float* stats, int E, int P, int n_sel, int reset, int32_t* chosen,
                           cudaStream_t st);
 cudaError_t launch_expire_wait(int32_t* status, unsigned long long limit_ns, cudaStream_t st);
@@ -836,8 +836,11 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
     }
     const bool use_tc = ws.tc_min != 0x7fffffff;                  // experts above 32 rows take the tcgen05 path
     const long long split_stride = (long long)ws.Rpad * D.d_model;  // partials of one K split: [Rpad][d]
-    auto collect_stats = [&]() -> dynamo_status {   // beside the gate/up kernels: it only has to be done before the down launch
-        if (!ctx->collect_stats) return DYNAMO_OK;
+    // The statistics only have to be done before the down launch and run beside the gate/up kernels; in front of all of them
+    // where profile events time those.
+    const bool timed = ctx->prof_ev[0] || ctx->prof_ev[1] || ctx->prof_ev[2];
+    const bool stats_beside = ctx->collect_stats && !timed;
+    auto collect_stats = [&]() -> dynamo_status {
         // row slices per expert: about two CTAs per SM in all; the partial sums live in the down GEMM's output buffer
         // (at least 8 * (E + Es) rows of d floats, idle until the down launch), which bounds the slice count
         const int P_pad = ctx->host_layer.P_pad;
@@ -845,14 +848,17 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         n_slices = std::max(1, std::min(n_slices, 8 * D.d_model / std::max(P_pad, 1)));
         if ((long long)T * D.top_k <= 16ll * D.n_experts) n_slices = 1;  // a few rows per expert: one pass is shorter
         CUDA_TRY(launch_stats(L, ws, x, (float*)(ctx->arena + ctx->A.stats), ws.ypart,
-                              (int32_t*)(ctx->arena + ctx->A.stats_ctr), D.n_experts, n_slices, st));
+                              (int32_t*)(ctx->arena + ctx->A.stats_ctr), D.n_experts, n_slices, stats_beside, st));
         ctx->launches += 1;
         return DYNAMO_OK;
     };
+    if (ctx->collect_stats && timed)
+        if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
     if (ctx->prof_ev[0]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[0], st));
     if (ws.fold) {
         CUDA_TRY(launch_ffn_fold(L, ws, 1, ctx->host_layer.n_rb13, 1, n, split_stride, ctx->n_sms, D.group_size, st));
-        if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
+        if (stats_beside)
+            if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
         if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
         CUDA_TRY(launch_ffn_fold(L, ws, 0, ctx->host_layer.n_rb2, ws.ksplit, n, split_stride, ctx->n_sms, D.group_size, st));
     } else {
@@ -865,8 +871,9 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         // with the streaming kernel first and a launch waiting for the other, 229 so; 2048: 499, 483).
         if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, n_rb13, n, ctx->tc2_clusters[1], st));
         CUDA_TRY(launch_ffn_stream(L, ws, 1, n_rb13, 1, n, split_stride, tiles, passes * n_rb13, long_rows, use_tc,
-                                   ctx->collect_stats, ctx->n_sms, D.group_size, st));
-        if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
+                                   stats_beside, ctx->n_sms, D.group_size, st));
+        if (stats_beside)
+            if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
         if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
         if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, n_rb2, n, ctx->tc2_clusters[0], st));
         CUDA_TRY(launch_ffn_stream(L, ws, 0, n_rb2, ws.ksplit, n, split_stride, tiles, passes * n_rb2 * ws.ksplit,

@@ -58,9 +58,13 @@ __device__ __forceinline__ void stats_cta(const LayerDev* __restrict__ L, const 
 }
 __global__ void __launch_bounds__(256) stats_kernel(const LayerDev* __restrict__ L, WsDev ws,
                                                     const __nv_bfloat16* __restrict__ x, float* __restrict__ stats,
-                                                    float* __restrict__ part, int32_t* __restrict__ ctr) {
-    pdl_trigger();
-    pdl_early_start();
+                                                    float* __restrict__ part, int32_t* __restrict__ ctr, int beside) {
+    if (beside) {
+        pdl_trigger();
+        pdl_early_start();
+    } else {
+        pdl_prologue();
+    }
     stats_cta(L, ws, x, stats, part, ctr);
     pdl_wait();
 }
@@ -100,11 +104,12 @@ __global__ void __launch_bounds__(256) select_kernel(const LayerDev* __restrict_
     if (threadIdx.x == 0) L->sig_cnt[e] = cnt;
 }
 
-// part: scratch of E * n_slices * P_pad floats; ctr: E zero-initialised counters (left at zero).
+// part: scratch of E * n_slices * P_pad floats; ctr: E zero-initialised counters (left at zero); beside: the launch before
+// is a gate/up kernel's that lets this one start beside it (otherwise the kernel waits for its predecessor).
 cudaError_t launch_stats(const LayerDev* L, const WsDev& ws, const void* x, float* stats, float* part, int32_t* ctr, int E,
-                         int n_slices, cudaStream_t st) {
+                         int n_slices, int beside, cudaStream_t st) {
     return launch_pdl(stats_kernel, dim3((unsigned)E, (unsigned)n_slices), dim3(256), 0, st, L, ws,
-                      (const __nv_bfloat16*)x, stats, part, ctr);
+                      (const __nv_bfloat16*)x, stats, part, ctr, beside);
 }
 
 cudaError_t launch_select(const LayerDev* L, float* stats, int E, int P, int n_sel, int reset, int32_t* chosen,

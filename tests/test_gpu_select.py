@@ -159,3 +159,31 @@ def test_selection_errors(tiny):
     assert st == binding.STATUS_NAMES.index("ERR_SHAPE")
     st = binding.load().dynamo_select_significant(None, 1, 0, None, None, None)
     assert st == binding.STATUS_NAMES.index("ERR_NULL")
+
+
+def test_profile_events_leave_the_statistics_out():
+    """Between the events before and after the gate/up launch (and after the down launch) lie the FFN kernels alone, with
+    statistics on as without: a layer whose statistics take longer than its FFN (all channels cached, 128 hidden units)."""
+    cfg = wl.scaled(CFG, d_ff=128, n_experts=1, top_k=1, max_sig=8, cache_size=512, zipf=None)
+    wg, wu, wd, bits, pool, sets = make_inputs(cfg)
+    gpu = make_gpu_layer(cfg, wg, wu, wd, bits, pool, max_tokens=4096)
+    T = 4096
+    x, lg = wl.activations(cfg, T, step=35).cuda(), wl.router_logits(cfg, T, step=35).cuda()
+    took, y = {}, {}
+    evs = [torch.cuda.Event(enable_timing=True) for _ in range(3)]
+    for e in evs:
+        e.record()
+    for on in (False, True):
+        gpu.set_stats_collection(on)
+        y[on] = gpu.forward(x, lg, binding.F32)
+        gpu.set_profile_events(evs)
+        spans = []
+        for _ in range(20):
+            assert torch.equal(gpu.forward(x, lg, binding.F32), y[on])
+            torch.cuda.synchronize()
+            spans.append((evs[0].elapsed_time(evs[1]), evs[1].elapsed_time(evs[2])))
+        gpu.set_profile_events(None)
+        took[on] = np.median(np.array(spans), axis=0)
+    gpu.set_stats_collection(False)
+    assert torch.equal(y[False], y[True])
+    assert np.all(took[True] <= 1.3 * took[False]), took
