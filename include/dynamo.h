@@ -225,8 +225,8 @@ enum { DYNAMO_OPERAND_FP16 = 0, DYNAMO_OPERAND_BF16 = 1 };
 dynamo_status dynamo_set_operand_dtype(dynamo_ctx* ctx, int32_t operand_dtype);
 
 /* Path selection: experts that receive more than `rows` tokens in a forward run on the paired tcgen05 kernel, the
- * others on the streaming kernel.  32 (the default and the maximum) also lets the library take one kernel for all
- * experts of a middle-sized batch; 0 switches the tcgen05 kernels off.  All paths implement the same arithmetic
+ * others on the streaming kernel.  32 (the default and the maximum) also lets the library take a third kernel for
+ * all but the most popular experts of a middle-sized batch; 0 switches the tcgen05 kernels off.  All paths implement the same arithmetic
  * definition. */
 dynamo_status dynamo_set_tc_min_rows(dynamo_ctx* ctx, int32_t rows);
 

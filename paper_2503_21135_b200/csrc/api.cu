@@ -49,7 +49,7 @@ cudaError_t launch_ffn_fold(const LayerDev* L, const WsDev& ws, int gateup, int 
                             long long split_stride, int n_sms, int G, cudaStream_t st);
 cudaError_t setup_ffn_tc2(int n_sms, int* clusters_out);
 cudaError_t launch_ffn_tc2(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int n_experts, int n_clusters,
-                           cudaStream_t st);
+                           int fills, cudaStream_t st);
 cudaError_t launch_stats(const LayerDev* L, const WsDev& ws, const void* x, float* stats, float* part, int32_t* ctr, int E,
                          int n_slices, int beside, cudaStream_t st);
 cudaError_t launch_select(const LayerDev* L, float* stats, int E, int P, int n_sel, int reset, int32_t* chosen,
@@ -100,8 +100,30 @@ inline bool decode_sized(const dynamo_layer_desc& D, int T) {
 // 65 tokens 249 us (streaming kernel 255), 100 tokens 269 (streaming and pair kernel 357), 139: 311 (523),
 // 200: 344 (465), 256 (64 rows an expert): 462 (468), 500: 671 (541).  Not with shared experts, whose rows are all the
 // tokens: the fine-grained layer at 128 tokens 240 us (176), at 300 260 (212).
-inline bool fold_sized(const dynamo_layer_desc& D, int T) {
-    return T > 2 * TC_MIN_ROWS && D.n_shared == 0 && (long long)T * D.top_k <= 62ll * D.n_experts;
+// Small experts keep a CTA for 16 stages at a time, and its start and its end weigh: where there are many of them, only
+// between a mean of 20 rows (the streaming kernel's second pass begins at 25) and 40 (an expert's second tile at 65).
+// 64 experts of 2048 x 1408, top-6, even router, against streaming and pair kernel: 100 tokens 146 us (131), 200 (19 rows)
+// 178 (169), 250: 194 (219), 375: 222 (253), 520 (49 rows) 263 (240), 660: 329 (248); Zipf router: 660 tokens 327 (232).
+// Where all their items are one round of the SMs it is the number of launches that counts (eight experts of 512 x 1024,
+// 100 tokens: 37 us, 57).
+inline bool fold_sized(const dynamo_layer_desc& D, int T, int n_sms) {
+    const long long rows = (long long)T * D.top_k, E = D.n_experts;
+    if (T <= 2 * TC_MIN_ROWS || D.n_shared || rows > 62 * E) return false;
+    const int n_rb = 2 * D.d_ff / RB, n_kc = D.d_model / KC;
+    if (n_rb * n_kc >= 256 || E * n_rb <= n_sms) return true;
+    return rows >= 20 * E && rows <= 40 * E;
+}
+// Rows from which an expert of such a batch leaves for the pair kernel, which expands it once per 256 of them.
+constexpr int FOLD_ROWS = 128;
+// Whether the pair kernel is launched beside the fold kernel.  The host does not know the router's choice; without a
+// popular expert the two launches cost next to nothing (139 tokens of eight 4096 x 14336 experts, even router: 300 us
+// with and without), with one they pay once the tiles of the k experts that may have all the tokens make more than one
+// and a half rounds of the SMs.  That layer, all tokens on two experts: 130 tokens 218 us (245 without), 200: 229 (330);
+// Zipf router: 180 tokens 362 (402).  16 experts of 2048 x 4096, one expert with all tokens: 140 tokens 149 (119), so not
+// below; 300 tokens on two experts 100 (115), 490: 104 (140).  (What that leaves: 16 experts of 2048 x 1408, all of 300
+// tokens on two of them, 81 us where the streaming and pair kernels take 69.)
+inline bool pair_beside_fold(const dynamo_layer_desc& D, int T, int n_sms) {
+    return T > FOLD_ROWS && 2ll * D.top_k * ((T + 63) / 64) * (2 * D.d_ff / RB) > 3ll * n_sms;
 }
 // Routed experts that T tokens reach when all are equally likely.
 inline int active_experts(const dynamo_layer_desc& D, int T) {
@@ -138,13 +160,13 @@ inline int stream_tiles(const dynamo_layer_desc& D, int T, int n_rb13, int n_sms
 //    thousand items (64 tokens 157 with 8, 116 with 2, 112 with 1).
 //  - The fold kernel's persistent CTAs want two items each (139 tokens 301 us with 8 splits, 292 with 2).
 inline int ksplit_beside_large(const dynamo_layer_desc& D) { return std::max(1, std::min(MAX_KSPLIT, D.d_ff / KC / 4)); }
-inline int ksplit_for(const dynamo_layer_desc& D, int T) {
+inline int ksplit_for(const dynamo_layer_desc& D, int T, int n_sms) {
     const int n_kc = D.d_ff / KC;
     if (!decode_sized(D, T)) return ksplit_beside_large(D);
     const int base = (active_experts(D, T) + D.n_shared) * (D.d_model / RB);   // items of one split
     int ks = n_kc / 4;
-    if (fold_sized(D, T)) ks = std::min(ks, 296 / base);
-    else ks = std::min(std::max(ks, std::min(n_kc / 2, (148 + base - 1) / base)), 1024 / base);
+    if (fold_sized(D, T, n_sms)) ks = std::min(ks, 2 * n_sms / base);
+    else ks = std::min(std::max(ks, std::min(n_kc / 2, (n_sms + base - 1) / base)), 1024 / base);
     return std::max(1, std::min(MAX_KSPLIT, ks));
 }
 inline int switch_ints_per_layer(const dynamo_layer_desc& D) { return D.n_experts * (2 * s_pad_of(D) + 1); }
@@ -364,18 +386,18 @@ WsDev make_ws(const dynamo_ctx* c, int T) {
     w.status = (int32_t*)(b + c->W.status);
     w.T = T;
     w.R = T * (D.top_k + D.n_shared);
-    w.ksplit = ksplit_for(D, T);
+    w.ksplit = ksplit_for(D, T, c->n_sms);
     w.off_pad = (int32_t*)(b + c->W.off_pad);
     w.Rpad = w.R + 8 * (D.n_experts + D.n_shared);
     w.Rcap = D.max_tokens * (D.top_k + D.n_shared) + 8 * (D.n_experts + D.n_shared) + ROW_PAD;
     // No expert can exceed T rows.  Up to twice the threshold the streaming kernel takes a large expert as
     // chunks of 24 tokens (the later passes over its blocks hit L2), which costs less than two more launches.
     w.tc_min = (c->tc_min_rows != 0x7fffffff && T > 2 * c->tc_min_rows) ? c->tc_min_rows : 0x7fffffff;
-    // Middle-sized batches: one kernel for all experts (see fold_sized).
-    w.fold = c->tc_min_rows == TC_MIN_ROWS && fold_sized(D, T);
-    if (w.fold) w.tc_min = 0x7fffffff;
-    // The streaming path alone (no row limit per expert): its splits need whole copies of ypart.
-    if (w.tc_min == 0x7fffffff && w.ysmall) {
+    // Middle-sized batches: one kernel for all experts but the most popular (see fold_sized, pair_beside_fold).
+    w.fold = c->tc_min_rows == TC_MIN_ROWS && fold_sized(D, T, c->n_sms);
+    if (w.fold) w.tc_min = pair_beside_fold(D, T, c->n_sms) ? FOLD_ROWS : 0x7fffffff;
+    // K splits of experts with more than 32 rows (fold kernel, streaming kernel alone) need whole copies of ypart.
+    if ((w.fold || w.tc_min == 0x7fffffff) && w.ysmall) {
         w.ysmall = nullptr;
         w.ksplit = 1;
     }
@@ -834,7 +856,7 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         CUDA_TRY(launch_scan(ws, D.n_experts, D.n_shared, D.top_k, st));
         CUDA_TRY(launch_gather(L, ws, x, D.d_model, st));
     }
-    const bool use_tc = ws.tc_min != 0x7fffffff;                  // experts above 32 rows take the tcgen05 path
+    const bool use_tc = ws.tc_min != 0x7fffffff;                  // experts above a number of rows take the pair kernel
     const long long split_stride = (long long)ws.Rpad * D.d_model;  // partials of one K split: [Rpad][d]
     // The statistics only have to be done before the down launch and run beside the gate/up kernels; in front of all of them
     // where profile events time those.
@@ -856,11 +878,15 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
     if (ctx->prof_ev[0]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[0], st));
     if (ws.fold) {
+        // The fold kernel goes first: a launch of the pair kernel in front of it cost 3.5 us even where it had no expert to
+        // work on (139 tokens, two launches: 306 us a pass, 299 so), behind it the clusters start where its CTAs have ended.
         CUDA_TRY(launch_ffn_fold(L, ws, 1, ctx->host_layer.n_rb13, 1, n, split_stride, ctx->n_sms, D.group_size, st));
+        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, ctx->host_layer.n_rb13, n, ctx->tc2_clusters[1], 1, st));
         if (stats_beside)
             if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
         if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
         CUDA_TRY(launch_ffn_fold(L, ws, 0, ctx->host_layer.n_rb2, ws.ksplit, n, split_stride, ctx->n_sms, D.group_size, st));
+        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, ctx->host_layer.n_rb2, n, ctx->tc2_clusters[0], 1, st));
     } else {
         const int n_rb13 = ctx->host_layer.n_rb13, n_rb2 = ctx->host_layer.n_rb2;
         const int tiles = use_tc ? 3 : stream_tiles(D, T, n_rb13, ctx->n_sms);
@@ -869,13 +895,13 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         // The pair kernel goes first where there is one: its clusters walk a fixed list and leave the last round uneven,
         // and the streaming kernel's queue fills the SMs as they come free (fine-grained layer, 300 tokens: 244 us a pass
         // with the streaming kernel first and a launch waiting for the other, 229 so; 2048: 499, 483).
-        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, n_rb13, n, ctx->tc2_clusters[1], st));
+        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, n_rb13, n, ctx->tc2_clusters[1], 0, st));
         CUDA_TRY(launch_ffn_stream(L, ws, 1, n_rb13, 1, n, split_stride, tiles, passes * n_rb13, long_rows, use_tc,
                                    stats_beside, ctx->n_sms, D.group_size, st));
         if (stats_beside)
             if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
         if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
-        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, n_rb2, n, ctx->tc2_clusters[0], st));
+        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, n_rb2, n, ctx->tc2_clusters[0], 0, st));
         CUDA_TRY(launch_ffn_stream(L, ws, 0, n_rb2, ws.ksplit, n, split_stride, tiles, passes * n_rb2 * ws.ksplit,
                                    long_rows, use_tc, ctx->down_active, ctx->n_sms, D.group_size, st));
     }

@@ -92,8 +92,8 @@ struct WsDev {
     int32_t* off_pad;     // [E_tot + 1]
     int32_t Rpad;
     int32_t Rcap;         // rows allocated in the activation buffers (their chunk pitch)
-    int32_t fold;         // 1: every expert takes the fold kernel (operand tiles with their group sums)
-    int32_t tc_min;       // experts with more rows than this take the tcgen05 path (INT_MAX: none)
+    int32_t tc_min;       // experts with more rows than this take the pair kernel (INT_MAX: none)
+    int32_t fold;         // 1: all the others take the fold kernel, 0: the streaming kernel
     int32_t h_bf16;       // 1: hidden activations are rounded to bf16 before they become the down GEMM's operand
 };
 
@@ -201,6 +201,15 @@ __device__ __forceinline__ void mbar_arrive_remote(uint64_t* bar, uint32_t cta) 
         "mbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}" ::"r"(smem_u32(bar)),
         "r"(cta)
         : "memory");
+}
+// A word of the leader's shared memory (CTA 0 of the cluster, same offset), behind a cluster barrier.
+__device__ __forceinline__ int ld_leader(const int* p) {
+    int v;
+    asm volatile("{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %1, 0;\n\tld.shared::cluster.b32 %0, [ra];\n\t}"
+                 : "=r"(v)
+                 : "r"(smem_u32(p))
+                 : "memory");
+    return v;
 }
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
     uint32_t ok;

@@ -143,7 +143,7 @@ __device__ __forceinline__ void down_fix_cta(const LayerDev* __restrict__ L, con
     const int nrows = min(FIX_ROWS, ws.off_pad[e] + n_e - row0);
     if (cnt <= 0 || nrows <= 0) return;
     const int seg0 = ws.off_pad[e];
-    const bool tile_layout = ws.fold || n_e > ws.tc_min;  // which FFN kernel wrote this expert's h
+    const bool fold = ws.fold && n_e <= ws.tc_min, tile_layout = fold || n_e > ws.tc_min;  // which FFN kernel wrote this expert's h
     const int bits = L->ex[e].bits, S2 = D2->S2, d = L->d;
     for (int i = threadIdx.x; i < cnt; i += FIX_THREADS) {
         pl[i] = D2->sig_pool[(long long)e * S2 + i];
@@ -156,7 +156,7 @@ __device__ __forceinline__ void down_fix_cta(const LayerDev* __restrict__ L, con
         if (r < nrows) {
             const int c = ch[i], kc = c >> 7, kk = c & 127;
             const uint8_t* p = tile_layout
-                                   ? ws.hbuf + (ws.fold ? act_off(kc, row0, ws.Rcap) : tile_off(kc, seg0, (row0 - seg0) >> 3, ws.Rcap)) + ((kk >> 3) * 8 + r) * 16 + (kk & 7) * 2
+                                   ? ws.hbuf + (fold ? act_off(kc, row0, ws.Rcap) : tile_off(kc, seg0, (row0 - seg0) >> 3, ws.Rcap)) + ((kk >> 3) * 8 + r) * 16 + (kk & 7) * 2
                                    : ws.hbuf + act_off(kc, row0 + r, ws.Rcap) + kk * 2;
             const float unscale = __uint_as_float((uint32_t)(127 - x_scale_exp(bits, kk)) << 23);
             v = __half2float(*reinterpret_cast<const __half*>(p)) * unscale;

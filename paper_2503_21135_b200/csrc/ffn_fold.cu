@@ -1,5 +1,5 @@
-// Grouped dequant-GEMM for middle-sized batches (experts of a few dozen rows): tcgen05 with the INTEGER CODES as the A
-// operand and scale / zero-point folded in once per quantization group.
+// Grouped dequant-GEMM for middle-sized batches (experts of a few dozen rows; beside the pair kernel, which takes popular
+// ones): tcgen05 with the INTEGER CODES as the A operand and scale / zero-point folded in once per quantization group.
 //
 // What bounds it.  A 256 x 128 weight block is 9 to 34 KB; at the copy bandwidth of HBM an SM's share of it takes 390
 // (2 bits) to 1440 cycles (8 bits).  Its sixteen MMAs (two tiles of M = 128 rows, K = 16 each) run N / 2 cycles each,

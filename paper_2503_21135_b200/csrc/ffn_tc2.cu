@@ -70,6 +70,7 @@ struct T2Params {
     WsDev ws;
     int n_rb;       // 256-row weight blocks of this GEMM
     int n_experts;  // experts listed in L->order
+    int fills;      // the launch before is the fold kernel's, on the smaller experts: this one starts beside it
 };
 
 struct T2Bars {
@@ -81,6 +82,7 @@ struct T2Bars {
     uint64_t d_empty;                    // leader only: 32 epilogue warps of the pair have read their accumulators
     uint32_t tmem_base;
     volatile int poison;
+    int off;                             // leader only: an expired wait was on record when the pair started (fills)
 };
 static_assert(sizeof(T2Bars) <= T2_OFF_PREFIX, "barrier block overlaps the item table");
 
@@ -180,9 +182,7 @@ __device__ __forceinline__ void t2_dequant_half(const uint8_t* st, uint32_t a_co
 }
 
 template <bool GATEUP>
-__global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p) {
-    extern __shared__ __align__(1024) uint8_t smem[];
-    pdl_wait();
+__device__ __forceinline__ void tc2_cta(const T2Params& p, uint8_t* smem, bool fills) {
     const LayerDev* L = p.L;
     const int G = L->G;
     const int K = GATEUP ? L->d : L->f;
@@ -199,9 +199,11 @@ __global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p
 
     // After an expired wait nothing new starts.  Both CTAs of a pair read the same word (the preceding kernel has
     // completed, and every cluster of this persistent grid starts at launch), so they leave together, before any
-    // barrier or tensor memory exists.
-    if (*p.ws.status & STATUS_TIMEOUT) return;
-    pdl_trigger();   // the streaming kernel of the smaller experts may fill the SMs from here on
+    // barrier or tensor memory exists.  (Beside the fold kernel, which may write the word, the leader's answer holds.)
+    if (!fills) {
+        if (*p.ws.status & STATUS_TIMEOUT) return;
+        pdl_trigger();   // the streaming kernel of the smaller experts may fill the SMs from here on
+    }
     // Item table (identical in both CTAs of the pair): experts above the row threshold contribute
     // (256-token tiles x row blocks) items.
     for (int i = threadIdx.x; i < p.n_experts; i += T2_THREADS) {
@@ -225,7 +227,7 @@ __global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p
         if (lane == 0) prefix[0] = 0;
     }
     __syncthreads();
-    const int total = prefix[p.n_experts];
+    int total = prefix[p.n_experts];
     // Nothing for this pair: both CTAs see the same table and leave together, before the cluster barrier.
     if (cluster_id >= total) return;
 
@@ -245,6 +247,7 @@ __global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p
         mbar_init(&B->d_full, 1);
         mbar_init(&B->d_empty, 2 * T2_DEQ_WARPS);
         B->poison = 0;
+        if (fills) B->off = *p.ws.status & STATUS_TIMEOUT;
         fence_barrier_init();
     }
     if (warp == T2_W_MMA) {
@@ -257,6 +260,7 @@ __global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p
     __syncthreads();
     cluster_sync_all();  // both CTAs' barriers are initialised before anybody arrives remotely
     tc_fence_after();
+    if (fills && ld_leader(&B->off)) total = 0;   // no role finds an item
     const uint32_t tbase = B->tmem_base;
     volatile int* poison = &B->poison;
     int32_t* status = p.ws.status;
@@ -439,7 +443,8 @@ __global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p
         // The first T2_LEAD stages of the NEXT item are dequantized before this item's epilogue: their A buffers come
         // free while the last MMAs of this item still run, so when the epilogue hands the accumulators back the MMA
         // warp finds two stages ready instead of waiting for a whole dequantization visit.
-        T2Item w = t2_decode_item<GATEUP>(p, prefix, cluster_id, cursor, n_kc, rank);
+        T2Item w;
+        if (cluster_id < total) w = t2_decode_item<GATEUP>(p, prefix, cluster_id, cursor, n_kc, rank);
         int lead_done = 0;                       // stages of w already dequantized (as the previous item's lead)
         for (int g = cluster_id; g < total && ok; g += n_clusters, ++ic) {
             const int bits = w.bits;
@@ -526,6 +531,20 @@ __global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p
     }
 }
 
+template <bool GATEUP>
+__global__ void __launch_bounds__(T2_THREADS, 1) ffn_tc2_kernel(const T2Params p) {
+    extern __shared__ __align__(1024) uint8_t smem[];
+    if (p.fills) {
+        pdl_trigger();
+        pdl_early_start();
+    } else {
+        pdl_wait();
+    }
+    tc2_cta<GATEUP>(p, smem, p.fills != 0);
+    // one pair that waits is enough: the grid completes behind it
+    if (p.fills && blockIdx.x < 2) pdl_wait();
+}
+
 // Persistent grid: as many CTA pairs as can be resident at once on the current device (pairs must share a TPC; not
 // every SM may be pairable), so that the static round-robin over clusters has no second wave.  Also raises the
 // kernels' shared-memory limit.  Called once per context at pack time, with the layer's device current.
@@ -563,12 +582,13 @@ cudaError_t setup_ffn_tc2(int n_sms, int* clusters_out) {
 // n_rb: 256-row weight blocks; n_experts: experts in L->order; n_clusters: CTA pairs of the persistent grid
 // (from setup_ffn_tc2 on this device).
 cudaError_t launch_ffn_tc2(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int n_experts, int n_clusters,
-                           cudaStream_t st) {
+                           int fills, cudaStream_t st) {
     T2Params p;
     p.L = L;
     p.ws = ws;
     p.n_rb = n_rb;
     p.n_experts = n_experts;
+    p.fills = fills;
     if (n_clusters < 1) return cudaErrorInvalidConfiguration;
     return gateup ? launch_pdl_cluster(ffn_tc2_kernel<true>, dim3((unsigned)(2 * n_clusters)), dim3(T2_THREADS),
                                        (size_t)T2_SMEM_BYTES, 2u, st, p)

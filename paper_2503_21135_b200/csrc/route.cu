@@ -487,8 +487,8 @@ __global__ void __launch_bounds__(256) gather_group_kernel(const LayerDev* __res
     const int row0 = 8 * blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (row0 >= ws.off_pad[L->E + L->Es]) return;
     const int e = ws.row_expert[row0], seg0 = ws.off_pad[e];
-    const bool fold = ws.fold != 0;
-    if (!fold && ws.counts[e] <= ws.tc_min) {   // a small expert: a warp per row
+    const bool small = ws.counts[e] <= ws.tc_min, fold = small && ws.fold;
+    if (small && !fold) {   // a warp per row
         gather_row(L, ws, x, row0 + warp, ws.row_token[row0 + warp], e, seg0, LAY_ROWS, blockIdx.y, gridDim.y);
         return;
     }

@@ -226,3 +226,46 @@ def test_overlapping_launches_in_a_captured_graph(T):
         torch.cuda.synchronize()
         assert torch.equal(want[0], want[1]) and torch.equal(stats[0], stats[1])
     assert gpu.poll_status() == 0 and gpu.debug_check_guards() == 0
+
+
+@pytest.mark.parametrize("group_size", [64, 128])
+@pytest.mark.parametrize("counts", [[128, 129, 1, 0, 17, 64, 65, 81], [496, 0, 0, 0, 0, 0, 0, 0], [96, 60, 72, 48, 128, 0, 40, 4],
+                                    [0, 257, 0, 0, 7, 0, 130, 0]])
+def test_popular_experts_of_a_middle_sized_batch(counts, group_size):
+    """Experts of more than 128 rows leave for the pair kernel, which starts beside the fold kernel: row counts on both
+    sides of that limit, one expert with everything, none that leaves; with statistics and hidden-unit sets (they read
+    either kernel's layout)."""
+    T = sum(counts)
+    cfg, gpu, ora = _layer(T, n_experts=8, top_k=1, group_size=group_size, d_model=1024, d_ff=4096)
+    _everything_on(cfg, gpu, ora)
+    e = np.concatenate([np.full(c, i) for i, c in enumerate(counts)])[np.random.default_rng(5).permutation(T)]
+    lg = torch.zeros((T, 8))
+    lg[torch.arange(T), torch.from_numpy(e)] = 4.0
+    x = wl.activations(cfg, T, step=71)
+    xd, ld = x.cuda(), lg.cuda()
+    before = gpu.kernel_launches()
+    first = gpu.forward(xd, ld, binding.F32)
+    assert gpu.kernel_launches() - before == 10
+    for _ in range(5):
+        assert torch.equal(gpu.forward(xd, ld, binding.F32), first)
+    ends = [t for i in range(8) if counts[i] for t in np.flatnonzero(e == i)[[0, -1]]]
+    toks = np.unique(np.array(ends + list(range(0, T, 31)), np.int32))
+    _check(cfg, gpu, ora, x, lg, toks)
+    stats = oracle.channel_stats_update(np.zeros((8, cfg.cache_size)), oracle.as_u16(x), e[:, None].astype(np.int32), wl.cache_pool(cfg))
+    got = gpu.channel_stats().cpu().numpy() / 8.0     # eight forwards of the same tokens
+    assert np.all(np.abs(got - stats) <= (np.array(counts)[:, None] + 9) * 2.0 ** -24 * stats)
+
+
+@pytest.mark.parametrize("T,launches", [(319, 8), (321, 6), (600, 8), (641, 8)])
+def test_many_small_experts_in_a_middle_sized_batch(T, launches):
+    """32 small experts, top-2, a skewed router, on both sides of the rows per expert from which and up to which they take
+    the fold kernel, and of the rows beyond which nothing is split along K."""
+    cfg, gpu, ora = _layer(641, n_experts=32, top_k=2, group_size=64, d_ff=2048)
+    lg = wl.router_logits(cfg, T, step=72)
+    lg -= 1.2 * torch.log(torch.arange(1.0, 33.0))
+    assert torch.bincount(lg.topk(2, 1)[1].flatten(), minlength=32).max() > 128
+    before = gpu.kernel_launches()
+    x = wl.activations(cfg, T, step=72)
+    gpu.forward(x.cuda(), lg.cuda(), binding.F32)
+    assert gpu.kernel_launches() - before == launches   # streaming and pair, fold, fold and pair, streaming and pair kernel
+    _check(cfg, gpu, ora, x, lg, np.arange(0, T, 7))
