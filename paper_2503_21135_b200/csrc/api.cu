@@ -43,8 +43,8 @@ cudaError_t launch_front(const LayerDev* L, const WsDev& ws, const void* x, cons
 cudaError_t launch_combine(const WsDev& ws, int d, int k, int Es, void* y, int y_f32, long long split_stride,
                            int n_experts, cudaStream_t st);
 cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
-                              long long split_stride, int tiles, long long n_items, bool long_rows, bool fills, bool leads,
-                              int n_sms, int G, cudaStream_t st);
+                              long long split_stride, int tiles, long long n_items, bool long_rows, int few, bool fills,
+                              bool leads, int n_sms, int G, cudaStream_t st);
 cudaError_t launch_ffn_fold(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
                             long long split_stride, int n_sms, int G, cudaStream_t st);
 cudaError_t setup_ffn_tc2(int n_sms, int* clusters_out);
@@ -149,6 +149,15 @@ inline int stream_tiles(const dynamo_layer_desc& D, int T, int n_rb13, int n_sms
     if (T <= 8 || stream_passes(D, T, 1) * n_rb13 <= 3ll * n_sms) return 1;
     if (D.n_shared) return rows <= 7 && T <= 40 ? 1 : 3;
     return rows <= 7 ? 1 : (rows <= 10 || T <= 16) ? 2 : 3;
+}
+// Whether the three-tile variant is launched as well and the device chooses between the two by the passes that the
+// experts' rows come to (ffn_stream.cu).  The host knows only their mean: with a popular expert, items of one or two tiles
+// expand its large blocks once more per 8 or 16 rows.  Eight experts of 4096 x 14336, Zipf router: 20 tokens 155 us (168 with
+// one tile alone, 151 three), 28: 188 (203, 180), 40: 242 (265 with two, 234 three); all tokens on two experts: 17 tokens
+// 120 (137, 108).  Even router: 16 tokens 170 (171), 24: 184 (184), 40: 205 (207): the launch that does nothing costs nothing.
+// Small experts gain nothing from three tiles (16 of 2048 x 4096, Zipf router, 40 tokens: 79 us with one tile, 83).
+inline bool either_variant(const dynamo_layer_desc& D, int T) {
+    return T > 8 && D.n_shared == 0 && (2 * D.d_ff / RB) * (D.d_model / KC) >= 2048;
 }
 // K splits of the down GEMM.  More splits are more items to balance and to hide latencies with; each pays for its start
 // and once more when the combine kernel adds it up.
@@ -892,18 +901,26 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         const int tiles = use_tc ? 3 : stream_tiles(D, T, n_rb13, ctx->n_sms);
         const long long passes = stream_passes(D, T, tiles);
         const bool long_rows = (use_tc ? std::min(T, ctx->tc_min_rows) : T) > 32;   // an expert on this path
+        const int few = !use_tc && tiles < 3 && either_variant(D, T) ? tiles : 0;
         // The pair kernel goes first where there is one: its clusters walk a fixed list and leave the last round uneven,
         // and the streaming kernel's queue fills the SMs as they come free (fine-grained layer, 300 tokens: 244 us a pass
         // with the streaming kernel first and a launch waiting for the other, 229 so; 2048: 499, 483).
         if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, n_rb13, n, ctx->tc2_clusters[1], 0, st));
-        CUDA_TRY(launch_ffn_stream(L, ws, 1, n_rb13, 1, n, split_stride, tiles, passes * n_rb13, long_rows, use_tc,
-                                   stats_beside, ctx->n_sms, D.group_size, st));
+        CUDA_TRY(launch_ffn_stream(L, ws, 1, n_rb13, 1, n, split_stride, tiles, passes * n_rb13, long_rows, few, use_tc,
+                                   stats_beside || few, ctx->n_sms, D.group_size, st));
+        if (few)
+            CUDA_TRY(launch_ffn_stream(L, ws, 1, n_rb13, 1, n, split_stride, 3, 0, long_rows, few, true, stats_beside,
+                                       ctx->n_sms, D.group_size, st));
         if (stats_beside)
             if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
         if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
         if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, n_rb2, n, ctx->tc2_clusters[0], 0, st));
         CUDA_TRY(launch_ffn_stream(L, ws, 0, n_rb2, ws.ksplit, n, split_stride, tiles, passes * n_rb2 * ws.ksplit,
-                                   long_rows, use_tc, ctx->down_active, ctx->n_sms, D.group_size, st));
+                                   long_rows, few, use_tc, ctx->down_active || few, ctx->n_sms, D.group_size, st));
+        if (few)
+            CUDA_TRY(launch_ffn_stream(L, ws, 0, n_rb2, ws.ksplit, n, split_stride, 3, 0, long_rows, few, true,
+                                       ctx->down_active, ctx->n_sms, D.group_size, st));
+        ctx->launches += few ? 2 : 0;
     }
     if (ctx->prof_ev[2]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[2], st));
     if (ctx->down_active) {  // significant hidden units: add what their 8-bit columns of W_down change

@@ -52,7 +52,8 @@ struct FfnParams {
     int n_rb;                // 256-row weight blocks of the matrix
     int n_experts;
     int32_t* work_ctr;       // device counter of this launch's work queue (zeroed by the scan kernel)
-    int fills, leads;        // the launch before, the one behind does not wait for this one's start: see pdl_trigger
+    int fills, leads;        // this launch runs beside the one before it, the one behind beside this one: see pdl_trigger
+    int few;                 // tiles of the smaller variant where two are launched and one does all the work, 0: one launch
     int sectioned;           // items ordered by tile count first (batches where an expert can have more than 32 rows)
 };
 
@@ -361,7 +362,7 @@ __device__ __forceinline__ bool consume_dispatch(const FfnParams& p, FfnSmem* S,
     return false;
 }
 
-template <bool GATEUP, int MAXNT8, int G>
+template <bool GATEUP, int MAXNT8, int G, bool EITHER>
 __device__ __forceinline__ void stream_cta(const FfnParams& p, uint8_t* smem) {
     // after an expired wait nothing new starts; beside the pair kernel, which may write the word, one answer for the CTA
     if (MAXNT8 == 3 ? __syncthreads_or(*p.ws.status & STATUS_TIMEOUT) : *p.ws.status & STATUS_TIMEOUT) return;
@@ -382,7 +383,7 @@ __device__ __forceinline__ void stream_cta(const FfnParams& p, uint8_t* smem) {
         fence_barrier_init();
     }
     if (warp == 0) {
-        // Items per expert, heaviest bit-width first; experts above tc_min rows take the tcgen05 path.  One lane per
+        // Items per expert, heaviest bit-width first; experts above tc_min rows are the pair kernel's.  One lane per
         // expert and a warp scan: one thread that walks the experts waits for its loads expert by expert (fine-grained
         // layer of 66 experts, 16 tokens: 44.5 + 29.3 us for the two launches, 42.6 + 25.8 with the scan; 512-wide
         // layer of 8 experts, 64 tokens: 18.3 + 11.2 -> 17.7 + 10.5).
@@ -408,6 +409,20 @@ __device__ __forceinline__ void stream_cta(const FfnParams& p, uint8_t* smem) {
                 if (y < p.n_experts) S->prefix[s * n1 + y + 1] = run[s] + v[s];
                 run[s] += __shfl_sync(0xffffffffu, v[s], 31);
             }
+        }
+        if constexpr (EITHER) {   // whose items suit the rows that the router gave the experts?
+            int n_few = 0, n_three = 0;
+            for (int y = lane; y < p.n_experts; y += 32) {
+                const int cnt = p.ws.counts[y];
+                n_few += (cnt + 8 * p.few - 1) / (8 * p.few);
+                n_three += (cnt + 23) / 24;
+            }
+            n_few = __reduce_add_sync(0xffffffffu, n_few);
+            n_three = __reduce_add_sync(0xffffffffu, n_three);
+            // a pass of one tile over an expert's blocks takes about 4/5 of the time of one of up to three, of two 10/11,
+            // and the second launch starts 4 us after the first
+            const bool few = p.few == 1 ? 10 * n_few <= 13 * n_three : 5 * n_few <= 6 * n_three;
+            if (few == (MAXNT8 == 3)) run[0] = run[1] = run[2] = 0;   // the other launch's turn
         }
         if (lane == 0) {
             S->prefix[0] = 0;
@@ -573,8 +588,10 @@ __device__ __forceinline__ void stream_cta(const FfnParams& p, uint8_t* smem) {
     if (clamped) atomicOr(p.ws.status, STATUS_RANGE);
 }
 
-// MAXNT8: most 8-token tiles of an item (the smaller variants need fewer registers and run three CTAs per SM).
-template <bool GATEUP, int MAXNT8, int G>
+// MAXNT8: most 8-token tiles of an item (the smaller variants need fewer registers and run three CTAs per SM).  EITHER: one
+// of two launches, of p.few and of three tiles, of which one does all the work (a template parameter: a test of p.few in
+// every variant's prologue cost 16 fine-grained tokens 1.4 us).
+template <bool GATEUP, int MAXNT8, int G, bool EITHER>
 __global__ void __launch_bounds__(FFN_THREADS, (MAXNT8 <= 2 && APW == 2) ? 3 : 2) ffn_stream_kernel(const FfnParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
     const bool fills = MAXNT8 == 3 && p.fills;
@@ -587,17 +604,17 @@ __global__ void __launch_bounds__(FFN_THREADS, (MAXNT8 <= 2 && APW == 2) ? 3 : 2
     } else {
         pdl_prologue();
     }
-    stream_cta<GATEUP, MAXNT8, G>(p, smem);
-    if (fills) pdl_wait();
+    stream_cta<GATEUP, MAXNT8, G, EITHER>(p, smem);
+    // (of a launch that may have had nothing to do, one CTA that waits is enough: the grid completes behind it)
+    if (fills && (!EITHER || blockIdx.x == 0)) pdl_wait();
 }
 
 template <bool GATEUP, int MAXNT8, int G>
 static cudaError_t launch_one_g(const FfnParams& p, int n_ctas, cudaStream_t st) {
-    cudaError_t err = cudaFuncSetAttribute(ffn_stream_kernel<GATEUP, MAXNT8, G>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem_bytes);
+    auto kernel = p.few ? ffn_stream_kernel<GATEUP, MAXNT8, G, true> : ffn_stream_kernel<GATEUP, MAXNT8, G, false>;
+    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem_bytes);
     if (err != cudaSuccess) return err;
-    return launch_pdl(ffn_stream_kernel<GATEUP, MAXNT8, G>, dim3((unsigned)n_ctas), dim3(FFN_THREADS),
-                      (size_t)p.smem_bytes, st, p);
+    return launch_pdl(kernel, dim3((unsigned)n_ctas), dim3(FFN_THREADS), (size_t)p.smem_bytes, st, p);
 }
 // The group size (64 or 128) is a template parameter: the group bookkeeping of the inner loop folds away.
 template <bool GATEUP, int MAXNT8>
@@ -606,16 +623,16 @@ static cudaError_t launch_one(const FfnParams& p, int n_ctas, int G, cudaStream_
 }
 
 // tiles: 8-token tiles of the kernel variant (1..3); n_items: about how many items the launch has; long_rows: an expert
-// can have more than 32 rows; fills: the launch before is the pair kernel's, on other experts; leads: the
-// launch behind starts beside this one.
+// can have more than 32 rows; few: see FfnParams; fills: the launch before works on other experts or may leave all to this
+// one, which starts beside it (three tiles only); leads: the launch behind starts beside this one.
 //
 // Three CTAs per SM hide more of each other's latencies, two have rings half as large again and leave room for the next
 // kernel's CTAs: three pay once every one has an item (1, 2, 3 and 4 tokens of a Mixtral-shaped layer: 68, 107, 130, 130
 // us a pass with two, 81, 104, 114, 114 with three; fine-grained, 4 and 16 tokens: 50 and 76, 61 and 72; 512-wide layer
 // of 64 tokens: 29 and 38).  The kernel of three tiles needs the registers of two.
 cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
-                              long long split_stride, int tiles, long long n_items, bool long_rows, bool fills, bool leads,
-                              int n_sms, int G, cudaStream_t st) {
+                              long long split_stride, int tiles, long long n_items, bool long_rows, int few, bool fills,
+                              bool leads, int n_sms, int G, cudaStream_t st) {
     const bool three = tiles < 3 && APW == 2 && n_items > 3 * n_sms;
     const int smem_bytes = three ? 74 * 1024 : 110 * 1024;
     const int n_ctas = (three ? 3 : 2) * n_sms;
@@ -629,7 +646,8 @@ cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, in
     p.ring_bytes = (smem_bytes - SMEM_HEADER - (gateup ? 2 * p.htile_bytes : 0)) & ~127;
     p.n_rb = n_rb;
     p.n_experts = n_experts;
-    p.work_ctr = ws.status + (gateup ? 4 : 5);
+    p.work_ctr = ws.status + (few && tiles == 3 ? 6 : 4) + (gateup ? 0 : 1);
+    p.few = few;
     p.fills = fills;
     p.leads = leads;
     p.sectioned = (long_rows && n_experts <= MAX_SECT_EXPERTS) ? 1 : 0;   // measured: +3 % at 64 tokens, -1 % at 32

@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(1024) scan_kernel(WsDev ws, int E, int Es, int
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
     const int kk = k + Es;
     // work-queue counters of this forward's streaming launches (callers that only route pass no status block)
-    if (ws.status && blockIdx.x == 0 && threadIdx.x < 2) ws.status[4 + threadIdx.x] = 0;
+    if (ws.status && blockIdx.x == 0 && threadIdx.x < 4) ws.status[4 + threadIdx.x] = 0;
     const int per_warp = ((n_pairs + 31) / 32 + nwarps - 1) / nwarps * 32;  // whole 32-pair batches per segment
     const int seg_lo = min(n_pairs, warp * per_warp), seg_hi = min(n_pairs, seg_lo + per_warp);
     const unsigned lt = (1u << lane) - 1;
@@ -660,7 +660,7 @@ __global__ void __launch_bounds__(256) front_kernel(const LayerDev* __restrict__
         }
     }
     if (blockIdx.x == 0) {
-        if (threadIdx.x < 2) ws.status[4 + threadIdx.x] = 0;   // work-queue counters of the two streaming launches
+        if (threadIdx.x < 4) ws.status[4 + threadIdx.x] = 0;   // work-queue counters of the streaming launches
         // the outputs and tables of the route and scan kernels
         for (int i = threadIdx.x; i < n_pairs; i += blockDim.x) {
             const int e = s_idx[i], r = s_rank[i], t = i / k, j = i - t * k;

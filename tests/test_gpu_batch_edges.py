@@ -269,3 +269,22 @@ def test_many_small_experts_in_a_middle_sized_batch(T, launches):
     gpu.forward(x.cuda(), lg.cuda(), binding.F32)
     assert gpu.kernel_launches() - before == launches   # streaming and pair, fold, fold and pair, streaming and pair kernel
     _check(cfg, gpu, ora, x, lg, np.arange(0, T, 7))
+
+
+@pytest.mark.parametrize("group_size", [64, 128])
+def test_either_streaming_variant_of_a_small_batch(group_size):
+    """Large experts, 9 to 32 tokens: two variants are launched and the device takes the one whose items suit the experts'
+    rows.  Routers on both sides of the choice for items of one and of two tiles; with statistics and hidden-unit sets."""
+    cfg, gpu, ora = _layer(32, n_experts=3, top_k=1, group_size=group_size, d_model=2048, d_ff=16384)
+    _everything_on(cfg, gpu, ora)
+    for counts in ([9, 0, 0], [8, 8, 4], [9, 9, 2], [20, 0, 0], [4, 1, 16], [28, 0, 0], [17, 10, 1], [10, 10, 10], [0, 16, 12]):
+        T = sum(counts)
+        e = np.concatenate([np.full(c, i) for i, c in enumerate(counts)])[np.random.default_rng(T).permutation(T)]
+        lg = torch.zeros((T, 3))
+        lg[torch.arange(T), torch.from_numpy(e)] = 4.0
+        x = wl.activations(cfg, T, step=81)
+        before = gpu.kernel_launches()
+        gpu.forward(x.cuda(), lg.cuda(), binding.F32)
+        assert gpu.kernel_launches() - before == 8   # front, two of either FFN launch, statistics, correction, combine
+        ends = [t for i in range(3) if counts[i] for t in np.flatnonzero(e == i)[[0, -1]]]
+        _check(cfg, gpu, ora, x, lg, np.unique(np.array(ends, np.int32)))
