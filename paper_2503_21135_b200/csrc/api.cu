@@ -34,9 +34,9 @@ cudaError_t launch_route(const float* logits, int T, int E, int k, int renorm, i
 cudaError_t launch_route_gemm(const void* x, const void* w_router, const float* bias, int T, int d, int E, int k,
                               int renorm, float* logits_out, int32_t* idx, float* w, cudaStream_t st);
 cudaError_t launch_upload(const void* xh, void* xd, long long x_bytes, const float* lh, float* ld, long long n_logits,
-                          cudaStream_t st);
+                          int n_sms, cudaStream_t st);
 cudaError_t launch_scan(const WsDev& ws, int E, int Es, int k, cudaStream_t st);
-cudaError_t launch_gather(const LayerDev* L, const WsDev& ws, const void* x, int d, cudaStream_t st);
+cudaError_t launch_gather(const LayerDev* L, const WsDev& ws, const void* x, int d, int n_sms, cudaStream_t st);
 bool front_fits(int T, int k);
 cudaError_t launch_front(const LayerDev* L, const WsDev& ws, const void* x, const float* logits, int E, int Es, int k,
                          int renorm, cudaStream_t st);
@@ -863,7 +863,7 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         else
             CUDA_TRY(launch_route(router_logits, T, D.n_experts, D.top_k, D.renormalize, ws.topk_idx, ws.topk_w, st));
         CUDA_TRY(launch_scan(ws, D.n_experts, D.n_shared, D.top_k, st));
-        CUDA_TRY(launch_gather(L, ws, x, D.d_model, st));
+        CUDA_TRY(launch_gather(L, ws, x, D.d_model, ctx->n_sms, st));
     }
     const bool use_tc = ws.tc_min != 0x7fffffff;                  // experts above a number of rows take the pair kernel
     const long long split_stride = (long long)ws.Rpad * D.d_model;  // partials of one K split: [Rpad][d]
@@ -1009,7 +1009,7 @@ dynamo_status dynamo_moe_forward_host(dynamo_ctx* ctx, const void* x_host, const
     const float* lm = xm ? (const float*)mapped_address(logits_host, lbytes) : nullptr;
     void* ym = ybytes <= DIRECT_BYTES ? mapped_address(y_host, ybytes) : nullptr;
     if (lm) {
-        CUDA_TRY(launch_upload(xm, xd, (long long)xbytes, lm, ld, (long long)T * D.n_experts, st));
+        CUDA_TRY(launch_upload(xm, xd, (long long)xbytes, lm, ld, (long long)T * D.n_experts, ctx->n_sms, st));
         ctx->launches += 1;
     } else {
         CUDA_TRY(cudaMemcpyAsync(xd, x_host, xbytes, cudaMemcpyHostToDevice, st));

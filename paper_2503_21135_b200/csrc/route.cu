@@ -803,11 +803,11 @@ cudaError_t launch_scan(const WsDev& ws, int E, int Es, int k, cudaStream_t st) 
     // from 2048 pairs on eight CTAs of 32 warps
     return launch_pdl(scan_kernel, dim3(batches >= 64 ? 8u : 1u), dim3((unsigned)(warps * 32)), 0, st, ws, E, Es, k);
 }
-cudaError_t launch_gather(const LayerDev* L, const WsDev& ws, const void* x, int d, cudaStream_t st) {
+cudaError_t launch_gather(const LayerDev* L, const WsDev& ws, const void* x, int d, int n_sms, cudaStream_t st) {
     if (ws.fold || ws.tc_min != 0x7fffffff) {
         // A group's chunks are cut over as many CTAs as it takes to have five per SM (at most one chunk a warp): 43
         // groups of 4096 15.6 -> 11.3 us, 258 21 -> 14.8; 2114 groups of 2048 cut in two 39 -> 45.
-        const int groups = (ws.Rpad + 7) / 8, ny = std::max(1, std::min(d / KC / 8, (148 * 5 + groups - 1) / groups));
+        const int groups = (ws.Rpad + 7) / 8, ny = std::max(1, std::min(d / KC / 8, (n_sms * 5 + groups - 1) / groups));
         return launch_pdl(gather_group_kernel, dim3((unsigned)groups, (unsigned)ny), dim3(256), 0, st, L, ws,
                           (const __nv_bfloat16*)x);
     }
@@ -823,9 +823,9 @@ cudaError_t launch_front(const LayerDev* L, const WsDev& ws, const void* x, cons
                       Es, k, renorm);
 }
 cudaError_t launch_upload(const void* xh, void* xd, long long x_bytes, const float* lh, float* ld, long long n_logits,
-                          cudaStream_t st) {
+                          int n_sms, cudaStream_t st) {
     const long long nx = x_bytes / 16;
-    const unsigned ctas = (unsigned)std::max(1ll, std::min(592ll, (nx + 255) / 256));
+    const unsigned ctas = (unsigned)std::max(1ll, std::min(4ll * n_sms, (nx + 255) / 256));
     upload_kernel<<<ctas, 256, 0, st>>>((const uint4*)xh, (uint4*)xd, nx, lh, ld, n_logits);
     return cudaGetLastError();
 }
