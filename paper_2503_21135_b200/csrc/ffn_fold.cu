@@ -10,7 +10,7 @@
 // before they work on the current one, and the MMAs of a stage are issued as one run behind one elect (an elect per
 // MMA costs 34 to 60 cycles each).  About 1150 cycles a stage at 64 tokens, 1340 at 139 (4096 x 14336 layer).
 //
-// Work item = (expert, 256-row weight block, tile of <= NT tokens, K split of the down GEMM), dealt round-robin over
+// Work item = (expert, 256-row weight block, tile of <= FF_NT tokens, K split of the down GEMM), dealt round-robin over
 // one persistent CTA per SM; ring, A buffers and accumulators live across items.  18 warps:
 //   warps 0-7 expand  : two groups of four (one warp per lane quarter), a group takes every other stage: the codes of
 //                       four atoms (16 rows x 128 k) -> A buffer in tensor memory.
@@ -22,7 +22,7 @@
 //                       byte-granular ring (up to 16 stages in flight).  The offsets follow from the sizes alone, so
 //                       every role computes them itself.
 //   warp 17 MMA       : sixteen MMAs and one commit per stage.
-// Tensor memory: NA A buffers of 128 columns, then NB accumulator buffers of 2 x NT columns.
+// Tensor memory: FF_NA A buffers of 128 columns, then FF_NB accumulator buffers of 2 x FF_NT columns.
 // Every wait is bounded; after an expired wait a role leaves its loops and the CTA meets at the final barrier.
 #include <cstddef>
 #include <type_traits>
@@ -39,10 +39,13 @@ constexpr int FF_FOLD_WARPS = 8;
 constexpr int FF_W_PROD = FF_EXP_WARPS + FF_FOLD_WARPS, FF_W_MMA = FF_W_PROD + 1;
 constexpr int FF_THREADS = (FF_W_MMA + 1) * 32;
 constexpr int FF_Q = 16;                  // most stages in flight
+constexpr int FF_NT = 64;                   // rows of an expert per pass
+constexpr int FF_NA = 2, FF_NB = 2;       // A buffers of 128 columns, accumulator buffers of 2 * FF_NT, in tensor memory
 constexpr int FF_HDR = 1024;              // barriers and ring bookkeeping
 constexpr int FF_HPITCH = 272;            // bytes per token row of the h tile (128 hidden units fp16 + pad)
 constexpr int FF_SMEM = 226 * 1024;
 constexpr uint32_t FF_TMEM_COLS = 512;
+static_assert(128 * FF_NA + 2 * FF_NT * FF_NB <= (int)FF_TMEM_COLS, "tensor memory");
 constexpr int FF_RG = 8 * XROW;   // operand tile of eight rows with its group sums behind it
 
 struct FfParams {
@@ -66,8 +69,8 @@ struct FfShared {
     uint64_t full[FF_Q];      // block and operand tile landed
     uint64_t empty[FF_Q];     // 8 fold warps are done with the stage (they follow the MMAs, which follow the expand warps)
     uint64_t done[FF_Q];      // the stage's MMAs are complete (commit)
-    uint64_t a_full[4];       // the 4 expand warps of the stage stored A buffer b
-    uint64_t acc_empty[8];    // 8 fold warps have read accumulator buffer i
+    uint64_t a_full[FF_NA];      // the 4 expand warps of the stage stored A buffer b
+    uint64_t acc_empty[FF_NB];   // 8 fold warps have read accumulator buffer i
     uint64_t hready, hfree;   // the item's h tile is written / read by the 8 fold warps
     int size[FF_Q];           // producer only: ring bytes of the stage in slot q
     uint32_t tmem_base;
@@ -357,7 +360,7 @@ __device__ __forceinline__ void ff_store_atom(const Codes<BITS> (&cd)[2], uint32
 }
 
 // One item on a warp that owns lane quarter q (two atoms) of both row tiles in the stages of parity kh.
-template <int BITS, int NA>
+template <int BITS>
 __device__ __forceinline__ bool ff_expand_item(const FfItem& im, FfShared* S, uint32_t sb, uint32_t ring, int cap,
                                                uint32_t a_lanes, int q, int kh, int lane, FfPos& pos, uint32_t& ready,
                                                int32_t* status) {
@@ -367,13 +370,13 @@ __device__ __forceinline__ bool ff_expand_item(const FfItem& im, FfShared* S, ui
         const uint32_t st = ring + pos.place(it < im.n_main ? need : need_pool, cap);
         const uint32_t si = pos.si;
         if ((si & 1) != (uint32_t)kh) continue;
-        const uint32_t b = si % NA, u = si - NA;
+        const uint32_t b = si % FF_NA, u = si - FF_NA;
         if (!__any_sync(0xffffffffu, ready) &&
             !ff_wait(FF_BAR(full, si % FF_Q), (si / FF_Q) & 1, &S->poison, status, 1, si))
             return false;
         // the MMAs that read this A buffer last must be complete before it is written
         uint32_t a_free = 1;
-        if (si >= NA) a_free = ff_test(FF_BAR(done, u % FF_Q), (u / FF_Q) & 1);
+        if (si >= FF_NA) a_free = ff_test(FF_BAR(done, u % FF_Q), (u / FF_Q) & 1);
         ready = ff_test(FF_BAR(full, (si + 2) % FF_Q), ((si + 2) / FF_Q) & 1);
         const uint32_t a_cols = a_lanes + 128 * b;
         if (it < im.n_main) {
@@ -432,7 +435,6 @@ struct FfRole {
 
 // The expand and fold roles are functions of their own: with everything inlined the compiler of the gate/up variant no
 // longer saw that the operands of the MMA role are warp-uniform.
-template <int NA>
 __device__ __noinline__ void ff_expand_role(const FfParams& p, FfRole R, int warp, int lane) {
     const int q = warp & 3, kh = warp >> 2;
     const uint32_t a_lanes = R.tbase + ((uint32_t)(32 * q) << 16);
@@ -445,20 +447,20 @@ __device__ __noinline__ void ff_expand_role(const FfParams& p, FfRole R, int war
     for (int g = blockIdx.x; g < R.total && ok; g += gridDim.x) {
         const FfItem im = ff_item_uni(p.ksplit, R.tab, g, cur, R.n_kc);
         switch (im.bits) {
-            case 2: ok = ff_expand_item<2, NA>(im, R.S, R.sb, R.ring, cap, a_lanes, q, kh, lane, pos, ready, status); break;
-            case 3: ok = ff_expand_item<3, NA>(im, R.S, R.sb, R.ring, cap, a_lanes, q, kh, lane, pos, ready, status); break;
-            case 4: ok = ff_expand_item<4, NA>(im, R.S, R.sb, R.ring, cap, a_lanes, q, kh, lane, pos, ready, status); break;
-            case 6: ok = ff_expand_item<6, NA>(im, R.S, R.sb, R.ring, cap, a_lanes, q, kh, lane, pos, ready, status); break;
-            default: ok = ff_expand_item<8, NA>(im, R.S, R.sb, R.ring, cap, a_lanes, q, kh, lane, pos, ready, status); break;
+            case 2: ok = ff_expand_item<2>(im, R.S, R.sb, R.ring, cap, a_lanes, q, kh, lane, pos, ready, status); break;
+            case 3: ok = ff_expand_item<3>(im, R.S, R.sb, R.ring, cap, a_lanes, q, kh, lane, pos, ready, status); break;
+            case 4: ok = ff_expand_item<4>(im, R.S, R.sb, R.ring, cap, a_lanes, q, kh, lane, pos, ready, status); break;
+            case 6: ok = ff_expand_item<6>(im, R.S, R.sb, R.ring, cap, a_lanes, q, kh, lane, pos, ready, status); break;
+            default: ok = ff_expand_item<8>(im, R.S, R.sb, R.ring, cap, a_lanes, q, kh, lane, pos, ready, status); break;
         }
     }
 }
 
 // ---- fold: one item on one (lane quarter, row tile) warp, NC columns (n_mma rounded up to an instantiated width) ----
-template <bool GATEUP, int NC, int NT, int NB, int G>
+template <bool GATEUP, int NC, int G>
 __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im, FfShared* S, uint32_t sb, uint32_t ring,
                                              uint8_t* htile, uint32_t acc_lanes, int q, int mt, int fw, int lane,
-                                             int ic, FfPos& pos, FfCycle<NB>& acb, uint32_t& ready, bool& clamped) {
+                                             int ic, FfPos& pos, FfCycle<FF_NB>& acb, uint32_t& ready, bool& clamped) {
     constexpr int NG = KC / G;
     volatile int* poison = &S->poison;
     int32_t* status = p.ws.status;
@@ -497,7 +499,7 @@ __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im
         tc_fence_after();
 #pragma unroll
         for (int g = 0; g < NG; ++g, acb.next()) {
-            const uint32_t acc = acc_lanes + acb.i * (2 * NT);
+            const uint32_t acc = acc_lanes + acb.i * (2 * FF_NT);
             uint32_t r[2][16];
             ff_ld16(acc, r[0]);
 #pragma unroll
@@ -532,7 +534,7 @@ __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im
             }
             ready = 0;
             tc_fence_after();
-            const uint32_t acc = acc_lanes + acb.i * (2 * NT);
+            const uint32_t acc = acc_lanes + acb.i * (2 * FF_NT);
             const uint64_t one2 = pack2(1.f, 1.f);
 #pragma unroll
             for (int c0 = 0; c0 < NC; c0 += 16) {
@@ -620,31 +622,31 @@ __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im
     return true;
 }
 
-template <bool GATEUP, int NT, int NA, int NB, int G>
+template <bool GATEUP, int G>
 __device__ __noinline__ void ff_fold_role(const FfParams& p, FfRole R, uint8_t* htile, int fw, int lane) {
     const int q = fw & 3, mt = fw >> 2;
-    const uint32_t acc_lanes = R.tbase + 128 * NA + mt * NT + ((uint32_t)(32 * q) << 16);
+    const uint32_t acc_lanes = R.tbase + 128 * FF_NA + mt * FF_NT + ((uint32_t)(32 * q) << 16);
     bool ok = true, clamped = false;
-    FfCycle<NB> acb;
+    FfCycle<FF_NB> acb;
     uint32_t ready = 0;
     int ic = 0, cur = 0;
     FfPos pos;
     for (int g = blockIdx.x; g < R.total && ok; g += gridDim.x, ++ic) {
         const FfItem im = ff_item_uni(p.ksplit, R.tab, g, cur, R.n_kc);
         if (im.n_mma <= 16)
-            ok = ff_fold_item<GATEUP, 16, NT, NB, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
+            ok = ff_fold_item<GATEUP, 16, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
         else if (im.n_mma <= 32)
-            ok = ff_fold_item<GATEUP, 32, NT, NB, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
+            ok = ff_fold_item<GATEUP, 32, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
         else if (im.n_mma <= 48)
-            ok = ff_fold_item<GATEUP, 48, NT, NB, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
+            ok = ff_fold_item<GATEUP, 48, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
         else
-            ok = ff_fold_item<GATEUP, NT, NT, NB, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
+            ok = ff_fold_item<GATEUP, FF_NT, G>(p, im, R.S, R.sb, R.ring, htile, acc_lanes, q, mt, fw, lane, ic, pos, acb, ready, clamped);
     }
     if (clamped) atomicOr(p.ws.status, STATUS_RANGE);
 }
 
 // ---- MMA issuer (a function of its own, see ff_expand_role) ---------------------------------------------------------
-template <int NT, int NA, int NB, int G>
+template <int G>
 __device__ __noinline__ void ff_mma_role(const FfParams& p, FfRole R) {
     FfShared* S = R.S;
     const FfExpert* tab = R.tab;
@@ -657,10 +659,10 @@ __device__ __noinline__ void ff_mma_role(const FfParams& p, FfRole R) {
     // ---------------- MMA issuer: warp-uniform, one elected lane issues ----------------
     // (A stored A buffer vouches for the stage's operand tile: the expand warps waited for it.)
     bool ok = true;
-    FfCycle<NA> ab;
-    FfCycle<NB> acb;
+    FfCycle<FF_NA> ab;
+    FfCycle<FF_NB> acb;
     uint32_t ready = 0;   // the next stage's barriers, asked for before this stage's MMAs are issued
-    const uint32_t acc0 = tbase + 128 * NA;
+    const uint32_t acc0 = tbase + 128 * FF_NA;
     for (int g = blockIdx.x; g < total && ok; g += gridDim.x) {
         const FfItem im = ff_item_uni(p.ksplit, tab, g, cur, n_kc);
         const uint32_t idesc = (1u << 4) | ((uint32_t)(im.n_mma >> 3) << 17) | ((128u >> 4) << 24);
@@ -670,7 +672,7 @@ __device__ __noinline__ void ff_mma_role(const FfParams& p, FfRole R) {
             const bool pool = it >= im.n_main;
             const uint32_t xt = ring_a + (pool ? pos.place(need_pool, cap) + POOL_GROUP * POOL_TILE_PITCH
                                                : pos.place(need, cap) + im.blk_bytes);
-            FfCycle<NB> acb1 = acb;
+            FfCycle<FF_NB> acb1 = acb;
             if (G == 64 && !pool) acb1.next();
             if (!__any_sync(0xffffffffu, ready)) {
                 ok = ff_wait(FF_BAR(acc_empty, acb1.i), acb1.par ^ 1, poison, status, 8, pos.si) &&
@@ -679,8 +681,8 @@ __device__ __noinline__ void ff_mma_role(const FfParams& p, FfRole R) {
             }
             tc_fence_after();
             // (the shuffles tell the compiler that the operands are warp-uniform)
-            const uint32_t d0 = __shfl_sync(0xffffffffu, acc0 + acb.i * (2 * NT), 0);
-            const uint32_t d1 = G == 64 ? __shfl_sync(0xffffffffu, acc0 + acb1.i * (2 * NT), 0) : d0;
+            const uint32_t d0 = __shfl_sync(0xffffffffu, acc0 + acb.i * (2 * FF_NT), 0);
+            const uint32_t d1 = G == 64 ? __shfl_sync(0xffffffffu, acc0 + acb1.i * (2 * FF_NT), 0) : d0;
             const uint32_t a0 = __shfl_sync(0xffffffffu, tbase + 128 * ab.i, 0);
             const uint32_t xu = __shfl_sync(0xffffffffu, xt, 0);
             const uint32_t done_bar = FF_BAR(done, pos.si % FF_Q);
@@ -689,11 +691,11 @@ __device__ __noinline__ void ff_mma_role(const FfParams& p, FfRole R) {
             if (!pool || it == n_st - 1) acb.next();
             ab.next();
             // main and cached-channel stages alike: an upper bound of what the next stage waits for
-            FfCycle<NB> nx = acb;
+            FfCycle<FF_NB> nx = acb;
             if (G == 64) nx.next();
             ready = ff_test(FF_BAR(acc_empty, nx.i), nx.par ^ 1) & ff_test(FF_BAR(a_full, ab.i), ab.par);
             // operand tile: main [row group][k octet 16][8][8] + sums, cached channels [row group][k octet 4][8][8]
-            ff_mma_stage<G>(d0, d1, a0, NT, tc_desc(xu, 128, pool ? 512 : FF_RG),
+            ff_mma_stage<G>(d0, d1, a0, FF_NT, tc_desc(xu, 128, pool ? 512 : FF_RG),
                             __shfl_sync(0xffffffffu, idesc, 0), acc_flag, pool ? 0u : 1u);
             asm volatile(
                 "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
@@ -704,10 +706,8 @@ __device__ __noinline__ void ff_mma_role(const FfParams& p, FfRole R) {
     if (!ok) *poison = 1;
 }
 
-template <bool GATEUP, int NT, int G>
+template <bool GATEUP, int G>
 __global__ void __launch_bounds__(FF_THREADS, 1) ffn_fold_kernel(const __grid_constant__ FfParams p) {
-    constexpr int NA = 2, NB = 2;
-    static_assert(128 * NA + 2 * NT * NB <= (int)FF_TMEM_COLS, "tensor memory");
     extern __shared__ __align__(1024) uint8_t smem[];
     FfShared* S = reinterpret_cast<FfShared*>(smem);
     FfExpert* tab = reinterpret_cast<FfExpert*>(smem + FF_HDR);
@@ -721,10 +721,10 @@ __global__ void __launch_bounds__(FF_THREADS, 1) ffn_fold_kernel(const __grid_co
             mbar_init(&S->empty[i], FF_FOLD_WARPS);
             mbar_init(&S->done[i], 1);
         }
-        for (int i = 0; i < NA; ++i) {
+        for (int i = 0; i < FF_NA; ++i) {
             mbar_init(&S->a_full[i], FF_EXP_WARPS / 2);
         }
-        for (int i = 0; i < NB; ++i) mbar_init(&S->acc_empty[i], FF_FOLD_WARPS);
+        for (int i = 0; i < FF_NB; ++i) mbar_init(&S->acc_empty[i], FF_FOLD_WARPS);
         mbar_init(&S->hready, FF_FOLD_WARPS);
         mbar_init(&S->hfree, FF_FOLD_WARPS);
         S->poison = 0;
@@ -750,7 +750,7 @@ __global__ void __launch_bounds__(FF_THREADS, 1) ffn_fold_kernel(const __grid_co
         FfExpert t;
         t.cnt = off ? 0 : p.ws.counts[e];
         if (t.cnt > p.ws.tc_min) t.cnt = 0;
-        t.n_tt = (t.cnt + NT - 1) / NT;
+        t.n_tt = (t.cnt + FF_NT - 1) / FF_NT;
         t.tile_rows = t.n_tt > 0 ? ((t.cnt + t.n_tt - 1) / t.n_tt + 7) & ~7 : 8;   // even tiles
         t.row0 = p.ws.off_pad[e];
         t.bits = ex.bits;
@@ -792,9 +792,9 @@ __global__ void __launch_bounds__(FF_THREADS, 1) ffn_fold_kernel(const __grid_co
     FfRole R;
     R.S = S; R.tab = tab; R.sb = sb; R.ring = ring_a; R.tbase = tbase; R.total = total; R.n_kc = n_kc;
     if (warp < FF_EXP_WARPS) {
-        ff_expand_role<NA>(p, R, warp, lane);
+        ff_expand_role(p, R, warp, lane);
     } else if (warp < FF_W_PROD) {
-        ff_fold_role<GATEUP, NT, NA, NB, G>(p, R, htile, warp - FF_EXP_WARPS, lane);
+        ff_fold_role<GATEUP, G>(p, R, htile, warp - FF_EXP_WARPS, lane);
     } else {
         if (warp == FF_W_PROD) {
             // ---------------- producer: one thread ----------------
@@ -855,7 +855,7 @@ __global__ void __launch_bounds__(FF_THREADS, 1) ffn_fold_kernel(const __grid_co
             }
             __syncwarp();
         } else if (warp == FF_W_MMA) {
-            ff_mma_role<NT, NA, NB, G>(p, R);
+            ff_mma_role<G>(p, R);
         }
         __syncwarp();
     }
@@ -867,21 +867,16 @@ __global__ void __launch_bounds__(FF_THREADS, 1) ffn_fold_kernel(const __grid_co
     }
 }
 
-template <bool GATEUP, int NT, int G>
+template <bool GATEUP, int G>
 static cudaError_t ff_launch(const FfParams& p, int n_ctas, cudaStream_t st) {
     cudaError_t err =
-        cudaFuncSetAttribute(ffn_fold_kernel<GATEUP, NT, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, FF_SMEM);
+        cudaFuncSetAttribute(ffn_fold_kernel<GATEUP, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, FF_SMEM);
     if (err != cudaSuccess) return err;
-    return launch_pdl(ffn_fold_kernel<GATEUP, NT, G>, dim3((unsigned)n_ctas), dim3(FF_THREADS), (size_t)FF_SMEM, st, p);
-}
-template <int NT, int G>
-static cudaError_t ff_launch_mat(const FfParams& p, int gateup, int n_ctas, cudaStream_t st) {
-    return gateup ? ff_launch<true, NT, G>(p, n_ctas, st) : ff_launch<false, NT, G>(p, n_ctas, st);
+    return launch_pdl(ffn_fold_kernel<GATEUP, G>, dim3((unsigned)n_ctas), dim3(FF_THREADS), (size_t)FF_SMEM, st, p);
 }
 
 cudaError_t launch_ffn_fold(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
                             long long split_stride, int n_sms, int G, cudaStream_t st) {
-    constexpr int NT = 64;   // rows of an expert per pass
     FfParams p;
     p.L = L;
     p.ws = ws;
@@ -891,9 +886,10 @@ cudaError_t launch_ffn_fold(const LayerDev* L, const WsDev& ws, int gateup, int 
     p.split_stride = split_stride;
     auto up = [](int v, int a) { return (v + a - 1) / a * a; };
     p.off_h = up(FF_HDR + (n_experts + 1) * (int)sizeof(FfExpert), 128);
-    p.off_ring = up(p.off_h + (gateup ? NT * FF_HPITCH : 0), 1024);
+    p.off_ring = up(p.off_h + (gateup ? FF_NT * FF_HPITCH : 0), 1024);
     p.ring_bytes = FF_SMEM - p.off_ring;
-    return G == 64 ? ff_launch_mat<NT, 64>(p, gateup, n_sms, st) : ff_launch_mat<NT, 128>(p, gateup, n_sms, st);
+    if (gateup) return G == 64 ? ff_launch<true, 64>(p, n_sms, st) : ff_launch<true, 128>(p, n_sms, st);
+    return G == 64 ? ff_launch<false, 64>(p, n_sms, st) : ff_launch<false, 128>(p, n_sms, st);
 }
 
 }  // namespace dyn
