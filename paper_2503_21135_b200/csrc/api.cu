@@ -47,9 +47,9 @@ cudaError_t launch_ffn_stream(const LayerDev* L, const WsDev& ws, int gateup, in
                               bool leads, int n_sms, int G, cudaStream_t st);
 cudaError_t launch_ffn_fold(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int ksplit, int n_experts,
                             long long split_stride, int n_sms, int G, cudaStream_t st);
-cudaError_t setup_ffn_tc2(int n_sms, int* clusters_out);
+cudaError_t setup_ffn_tc2(int n_sms, int G, int* clusters_out);
 cudaError_t launch_ffn_tc2(const LayerDev* L, const WsDev& ws, int gateup, int n_rb, int n_experts, int n_clusters,
-                           int fills, cudaStream_t st);
+                           int fills, int G, cudaStream_t st);
 cudaError_t launch_stats(const LayerDev* L, const WsDev& ws, const void* x, float* stats, float* part, int32_t* ctr, int E,
                          int n_slices, int beside, cudaStream_t st);
 cudaError_t launch_select(const LayerDev* L, float* stats, int E, int P, int n_sel, int reset, int32_t* chosen,
@@ -730,7 +730,7 @@ dynamo_status dynamo_pack_experts(dynamo_ctx* ctx, const void* w_gate, const voi
         if (cudaGetDevice(&dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
             ctx->n_sms = sms;
-        CUDA_TRY(setup_ffn_tc2(ctx->n_sms, ctx->tc2_clusters));
+        CUDA_TRY(setup_ffn_tc2(ctx->n_sms, G, ctx->tc2_clusters));
     }
     ctx->packed = true;
     // install the empty significant sets (sig_pool -> zero tile, sig_chan -> -1)
@@ -890,12 +890,12 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         // The fold kernel goes first: a launch of the pair kernel in front of it cost 3.5 us even where it had no expert to
         // work on (139 tokens, two launches: 306 us a pass, 299 so), behind it the clusters start where its CTAs have ended.
         CUDA_TRY(launch_ffn_fold(L, ws, 1, ctx->host_layer.n_rb13, 1, n, split_stride, ctx->n_sms, D.group_size, st));
-        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, ctx->host_layer.n_rb13, n, ctx->tc2_clusters[1], 1, st));
+        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, ctx->host_layer.n_rb13, n, ctx->tc2_clusters[1], 1, D.group_size, st));
         if (stats_beside)
             if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
         if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
         CUDA_TRY(launch_ffn_fold(L, ws, 0, ctx->host_layer.n_rb2, ws.ksplit, n, split_stride, ctx->n_sms, D.group_size, st));
-        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, ctx->host_layer.n_rb2, n, ctx->tc2_clusters[0], 1, st));
+        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, ctx->host_layer.n_rb2, n, ctx->tc2_clusters[0], 1, D.group_size, st));
     } else {
         const int n_rb13 = ctx->host_layer.n_rb13, n_rb2 = ctx->host_layer.n_rb2;
         const int tiles = use_tc ? 3 : stream_tiles(D, T, n_rb13, ctx->n_sms);
@@ -905,7 +905,7 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         // The pair kernel goes first where there is one: its clusters walk a fixed list and leave the last round uneven,
         // and the streaming kernel's queue fills the SMs as they come free (fine-grained layer, 300 tokens: 244 us a pass
         // with the streaming kernel first and a launch waiting for the other, 229 so; 2048: 499, 483).
-        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, n_rb13, n, ctx->tc2_clusters[1], 0, st));
+        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 1, n_rb13, n, ctx->tc2_clusters[1], 0, D.group_size, st));
         CUDA_TRY(launch_ffn_stream(L, ws, 1, n_rb13, 1, n, split_stride, tiles, passes * n_rb13, long_rows, few, use_tc,
                                    stats_beside || few, ctx->n_sms, D.group_size, st));
         if (few)
@@ -914,7 +914,7 @@ static dynamo_status forward_impl(dynamo_ctx* ctx, const void* x, const float* r
         if (stats_beside)
             if (const dynamo_status e = collect_stats(); e != DYNAMO_OK) return e;
         if (ctx->prof_ev[1]) CUDA_TRY(cudaEventRecord(ctx->prof_ev[1], st));
-        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, n_rb2, n, ctx->tc2_clusters[0], 0, st));
+        if (use_tc) CUDA_TRY(launch_ffn_tc2(L, ws, 0, n_rb2, n, ctx->tc2_clusters[0], 0, D.group_size, st));
         CUDA_TRY(launch_ffn_stream(L, ws, 0, n_rb2, ws.ksplit, n, split_stride, tiles, passes * n_rb2 * ws.ksplit,
                                    long_rows, few, use_tc, ctx->down_active || few, ctx->n_sms, D.group_size, st));
         if (few)

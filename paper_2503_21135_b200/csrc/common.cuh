@@ -190,18 +190,6 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
-// Arrive on the barrier at the same shared-memory offset in CTA `cta` of the cluster.  Default semantics on
-// purpose: what these arrivals hand over is the COMPLETION of asynchronous work (tensor-memory stores and loads
-// waited for with tcgen05.wait, bulk copies observed on their own barrier), not generic-proxy data, so no
-// cluster-scope fence is needed; an explicit .release.cluster here (and .acquire.cluster on the waiting side) cost
-// the pair kernel a fifth of its time.
-__device__ __forceinline__ void mbar_arrive_remote(uint64_t* bar, uint32_t cta) {
-    asm volatile(
-        "{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, %1;\n\t"
-        "mbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}" ::"r"(smem_u32(bar)),
-        "r"(cta)
-        : "memory");
-}
 // A word of the leader's shared memory (CTA 0 of the cluster, same offset), behind a cluster barrier.
 __device__ __forceinline__ int ld_leader(const int* p) {
     int v;
@@ -210,17 +198,6 @@ __device__ __forceinline__ int ld_leader(const int* p) {
                  : "r"(smem_u32(p))
                  : "memory");
     return v;
-}
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
 }
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
@@ -291,26 +268,94 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     }
 }
 
-// The same wait for barriers that threads of the peer CTA arrive on (default acquire: see mbar_arrive_remote).
-__device__ __forceinline__ bool mbar_wait_bounded_cluster(uint64_t* bar, uint32_t parity, volatile int* poison,
-                                                          int32_t* status) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
+// Shared memory by 32-bit address: barriers, ring and tables are addressed by offset from the CTA's base (a generic
+// pointer would be converted again at every use).
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 lds64(uint32_t a) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t lds32(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// A role's place in a byte-granular ring of stages: the offsets follow from the sizes alone, so every role computes them
+// itself.
+struct RingPos {
+    uint32_t si = 0;   // running stage number
+    int head = 0;
+    __device__ __forceinline__ int place(int need, int cap) {   // ring offset of a stage of `need` bytes
+        const int off = head + need > cap ? 0 : head;
+        head = off + need;
+        return off;
+    }
+};
+
+// ---- barriers by 32-bit shared-memory address, waited for by whole warps ----------------------------------------------
+__device__ __forceinline__ void bar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// The same on the barrier at that offset in the leader (CTA 0) of the cluster.  Default semantics on purpose: what these
+// arrivals hand over is the COMPLETION of asynchronous work (tensor-memory stores and loads waited for with tcgen05.wait,
+// bulk copies observed on their own barrier), not generic-proxy data, so no cluster-scope fence is needed; an explicit
+// .release.cluster here (and .acquire.cluster on the waiting side) cost the pair kernel a fifth of its time.
+__device__ __forceinline__ void bar_arrive_leader(uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, 0;\n\tmbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}" ::"r"(bar)
+        : "memory");
+}
+// Bounded wait of a whole warp on one barrier; false after an expired wait (here or elsewhere in the CTA).  All lanes
+// poll together and the loop is left by vote: the compiler then knows that the warp is converged behind it and keeps
+// the operands of tcgen05 instructions in uniform registers (16 MMAs issue in 165 cycles, in 1100 otherwise).
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* poison, int32_t* status, int where,
+                                        uint32_t aux) {
+    uint32_t n = 0;
     unsigned long long t0 = 0;
-    uint32_t spins = 0;
     while (true) {
-        if (mbar_try_wait_cluster(bar, parity)) return true;
-        if ((++spins & 0x3ff) == 0) {
-            if (*poison) return false;
-            const unsigned long long now = globaltimer_ns();
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 20000;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (__any_sync(0xffffffffu, ok)) return true;
+        if ((++n & 0x3ff) == 0) {
+            if (__any_sync(0xffffffffu, *poison)) return false;
+            const unsigned long long now = __shfl_sync(0xffffffffu, globaltimer_ns(), 0);
             if (t0 == 0) {
                 t0 = now;
             } else if (now - t0 > WAIT_LIMIT_NS) {
-                *poison = 1;
-                atomicOr(status, STATUS_TIMEOUT);
+                if ((threadIdx.x & 31) == 0) {
+                    *poison = 1;
+                    if (atomicCAS(status + 8, 0, where | 0x1000) == 0) {
+                        status[9] = (int)blockIdx.x;
+                        status[10] = (int)threadIdx.x;
+                        status[11] = (int)aux;
+                    }
+                    atomicOr(status, STATUS_TIMEOUT);
+                }
+                __syncwarp();
                 return false;
             }
         }
     }
+}
+// One poll whose answer is used later: a poll takes hundreds of cycles beside tensor-memory traffic, so the roles ask
+// for their next stage before they work on the current one.
+__device__ __forceinline__ uint32_t bar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok)
+                 : "r"(bar), "r"(parity)
+                 : "memory");
+    return ok;
 }
 
 // 1-D bulk async copy global -> shared, completion counted on an mbarrier (bytes % 16 == 0,

@@ -126,6 +126,58 @@ __device__ __forceinline__ void expand(const Codes<BITS>& c, uint32_t (&a)[4]) {
     }
 }
 
+// The packed words of one atom that a lane owns (both half chunks), as they lie in shared memory: 4, 6, 8, 12 or 16.
+template <int BITS>
+__device__ __forceinline__ void load_raw(uint32_t (&w)[16], uint32_t atom, int lane) {
+    auto put = [&](int i, uint4 v) {
+        w[i] = v.x; w[i + 1] = v.y; w[i + 2] = v.z; w[i + 3] = v.w;
+    };
+    put(0, lds128(atom + lane * 16));
+    if constexpr (BITS == 3) {
+        const uint2 hb = lds64(atom + 512 + lane * 8);
+        w[4] = hb.x; w[5] = hb.y;
+    }
+    if constexpr (BITS >= 4) put(4, lds128(atom + 512 + lane * 16));
+    if constexpr (BITS >= 6) put(8, lds128(atom + 1024 + lane * 16));
+    if constexpr (BITS == 8) put(12, lds128(atom + 1536 + lane * 16));
+}
+template <int BITS, int HALF>
+__device__ __forceinline__ void codes_of(Codes<BITS>& c, const uint32_t (&w)[16]) {
+    if constexpr (BITS == 2 || BITS == 3) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            c.w[i] = w[2 * HALF + i];
+            c.ws[i] = c.w[i] >> (BITS == 2 ? 10 : 8);
+        }
+        if constexpr (BITS == 3) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                c.t0[i] = rotr32(w[4 + i], HALF * 8);
+                c.t1[i] = rotr32(w[4 + i], HALF * 8 + 1);
+            }
+        }
+    } else if constexpr (BITS == 8) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) c.w[i] = w[8 * HALF + i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            c.w[i] = w[4 * HALF + i];
+            c.ws[i] = c.w[i] >> 8;
+        }
+        if constexpr (BITS == 6) {
+#pragma unroll
+            for (int rh = 0; rh < 2; ++rh) {
+                const uint32_t hw = w[8 + 2 * HALF + rh], sw = prmt(hw, 0u, 0x2301u);   // bytes of each half swapped
+                c.t[rh][0] = hw;
+                c.t[rh][1] = hw >> 2;
+                c.t[rh][2] = sw;
+                c.t[rh][3] = sw >> 2;
+            }
+        }
+    }
+}
+
 // In-place bit offset o of the code of (MMA step S4 of a half chunk, k pair h): see layout.cuh.
 template <int BITS>
 __host__ __device__ constexpr int code_offset(int s4, int h) {

@@ -142,17 +142,6 @@ struct FfCycle {
         }
     }
 };
-// A role's place in the stage sequence: ring slot and write offset.
-struct FfPos {
-    uint32_t si = 0;   // running stage number: slot si % FF_Q, parity (si / FF_Q) & 1
-    int head = 0;
-    __device__ __forceinline__ int place(int need, int cap) {   // ring offset of a stage of `need` bytes
-        const int off = head + need > cap ? 0 : head;
-        head = off + need;
-        return off;
-    }
-};
-
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
     uint64_t r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
@@ -166,96 +155,11 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
-// Shared memory by 32-bit address: barriers, ring and tables are addressed by offset from the CTA's base (a generic
-// pointer would be converted again at every use).
-__device__ __forceinline__ uint4 lds128(uint32_t a) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint2 lds64(uint32_t a) {
-    uint2 v;
-    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint32_t lds32(uint32_t a) {
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-    return v;
-}
 __device__ __forceinline__ void lds_sums(uint32_t a, uint64_t& x, uint64_t& y) {   // four fp32 as two pairs
     asm volatile("ld.shared.v2.b64 {%0,%1}, [%2];" : "=l"(x), "=l"(y) : "r"(a) : "memory");
 }
-__device__ __forceinline__ void ff_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool ff_try(uint32_t bar, uint32_t parity, uint32_t hint_ns) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(hint_ns)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait of a whole warp on one barrier; false after an expired wait (here or elsewhere in the CTA).  All lanes
-// poll together and the loop is left by vote: the compiler then knows that the warp is converged behind it and keeps
-// the operands of tcgen05 instructions in uniform registers (16 MMAs issue in 165 cycles, in 1100 otherwise).
-__device__ __forceinline__ bool ff_wait(uint32_t bar, uint32_t parity, volatile int* poison, int32_t* status, int where,
-                                        uint32_t aux) {
-    uint32_t n = 0;
-    unsigned long long t0 = 0;
-    while (true) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 20000;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (__any_sync(0xffffffffu, ok)) return true;
-        if ((++n & 0x3ff) == 0) {
-            if (__any_sync(0xffffffffu, *poison)) return false;
-            const unsigned long long now = __shfl_sync(0xffffffffu, globaltimer_ns(), 0);
-            if (t0 == 0) {
-                t0 = now;
-            } else if (now - t0 > WAIT_LIMIT_NS) {
-                if ((threadIdx.x & 31) == 0) {
-                    *poison = 1;
-                    if (atomicCAS(status + 8, 0, where | 0x1000) == 0) {
-                        status[9] = (int)blockIdx.x;
-                        status[10] = (int)threadIdx.x;
-                        status[11] = (int)aux;
-                    }
-                    atomicOr(status, STATUS_TIMEOUT);
-                }
-                __syncwarp();
-                return false;
-            }
-        }
-    }
-}
-// One poll whose answer is used later: a poll takes hundreds of cycles beside tensor-memory traffic, so the roles ask
-// for their next stage before they work on the current one.
-__device__ __forceinline__ uint32_t ff_test(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok)
-                 : "r"(bar), "r"(parity)
-                 : "memory");
-    return ok;
-}
 // barrier offsets from the CTA's shared-memory base
 #define FF_BAR(field, i) (sb + (uint32_t)offsetof(FfShared, field) + 8u * (uint32_t)(i))
-// one weight row per lane, 16 consecutive accumulator columns
-__device__ __forceinline__ void ff_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
-
 // ---- MMA issue: runs of instructions behind one elect, operands warp-uniform ------------------------------------
 #define FF_MMA(pred, d, a, k, acc)                                \
     "add.s64 bd, %4, " #k "*16;\n\tadd.s32 aa, " a ", " #k "*8;\n\t" \
@@ -362,7 +266,7 @@ __device__ __forceinline__ void ff_store_atom(const Codes<BITS> (&cd)[2], uint32
 // One item on a warp that owns lane quarter q (two atoms) of both row tiles in the stages of parity kh.
 template <int BITS>
 __device__ __forceinline__ bool ff_expand_item(const FfItem& im, FfShared* S, uint32_t sb, uint32_t ring, int cap,
-                                               uint32_t a_lanes, int q, int kh, int lane, FfPos& pos, uint32_t& ready,
+                                               uint32_t a_lanes, int q, int kh, int lane, RingPos& pos, uint32_t& ready,
                                                int32_t* status) {
     const int n_st = im.n_main + im.n_pool;
     const int need = im.need(), need_pool = im.need_pool();
@@ -372,12 +276,12 @@ __device__ __forceinline__ bool ff_expand_item(const FfItem& im, FfShared* S, ui
         if ((si & 1) != (uint32_t)kh) continue;
         const uint32_t b = si % FF_NA, u = si - FF_NA;
         if (!__any_sync(0xffffffffu, ready) &&
-            !ff_wait(FF_BAR(full, si % FF_Q), (si / FF_Q) & 1, &S->poison, status, 1, si))
+            !warp_wait(FF_BAR(full, si % FF_Q), (si / FF_Q) & 1, &S->poison, status, 1, si))
             return false;
         // the MMAs that read this A buffer last must be complete before it is written
         uint32_t a_free = 1;
-        if (si >= FF_NA) a_free = ff_test(FF_BAR(done, u % FF_Q), (u / FF_Q) & 1);
-        ready = ff_test(FF_BAR(full, (si + 2) % FF_Q), ((si + 2) / FF_Q) & 1);
+        if (si >= FF_NA) a_free = bar_test(FF_BAR(done, u % FF_Q), (u / FF_Q) & 1);
+        ready = bar_test(FF_BAR(full, (si + 2) % FF_Q), ((si + 2) / FF_Q) & 1);
         const uint32_t a_cols = a_lanes + 128 * b;
         if (it < im.n_main) {
             constexpr int GRP = BITS >= 6 ? 2 : 4;   // atoms whose codes are in registers at a time
@@ -389,7 +293,7 @@ __device__ __forceinline__ bool ff_expand_item(const FfItem& im, FfShared* S, ui
                     ff_load_codes<BITS>(cd[a], st + (8 * ((a0 + a) >> 1) + 2 * q + (a & 1)) * (256 * BITS), lane);
                 if (a0 == 0) {
                     if (!__any_sync(0xffffffffu, a_free) &&
-                        !ff_wait(FF_BAR(done, u % FF_Q), (u / FF_Q) & 1, &S->poison, status, 2, si))
+                        !warp_wait(FF_BAR(done, u % FF_Q), (u / FF_Q) & 1, &S->poison, status, 2, si))
                         return false;
                     tc_fence_after();
                 }
@@ -400,7 +304,7 @@ __device__ __forceinline__ bool ff_expand_item(const FfItem& im, FfShared* S, ui
         } else {
             // cached-channel stage: fp16 tiles [pool column][256 rows] -> A fragments
             if (!__any_sync(0xffffffffu, a_free) &&
-                !ff_wait(FF_BAR(done, u % FF_Q), (u / FF_Q) & 1, &S->poison, status, 2, si))
+                !warp_wait(FF_BAR(done, u % FF_Q), (u / FF_Q) & 1, &S->poison, status, 2, si))
                 return false;
             tc_fence_after();
             const int mi = lane >> 3, r = lane & 7;
@@ -420,7 +324,7 @@ __device__ __forceinline__ bool ff_expand_item(const FfItem& im, FfShared* S, ui
         tc_wait_st();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) ff_arrive(FF_BAR(a_full, b));
+        if (lane == 0) bar_arrive(FF_BAR(a_full, b));
     }
     return true;
 }
@@ -443,7 +347,7 @@ __device__ __noinline__ void ff_expand_role(const FfParams& p, FfRole R, int war
     bool ok = true;
     uint32_t ready = 0;
     int cur = 0;
-    FfPos pos;
+    RingPos pos;
     for (int g = blockIdx.x; g < R.total && ok; g += gridDim.x) {
         const FfItem im = ff_item_uni(p.ksplit, R.tab, g, cur, R.n_kc);
         switch (im.bits) {
@@ -460,7 +364,7 @@ __device__ __noinline__ void ff_expand_role(const FfParams& p, FfRole R, int war
 template <bool GATEUP, int NC, int G>
 __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im, FfShared* S, uint32_t sb, uint32_t ring,
                                              uint8_t* htile, uint32_t acc_lanes, int q, int mt, int fw, int lane,
-                                             int ic, FfPos& pos, FfCycle<FF_NB>& acb, uint32_t& ready, bool& clamped) {
+                                             int ic, RingPos& pos, FfCycle<FF_NB>& acb, uint32_t& ready, bool& clamped) {
     constexpr int NG = KC / G;
     volatile int* poison = &S->poison;
     int32_t* status = p.ws.status;
@@ -476,9 +380,9 @@ __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im
         const uint32_t st = ring + pos.place(need, p.ring_bytes);
         const uint32_t slot = pos.si % FF_Q, par = (pos.si / FF_Q) & 1;
         // zero-point times the group sums, as soon as the copies have landed
-        if (!__any_sync(0xffffffffu, ready) && !ff_wait(FF_BAR(full, slot), par, poison, status, 3, pos.si)) return false;
-        const uint32_t done = ff_test(FF_BAR(done, slot), par);
-        ready = ff_test(FF_BAR(full, (pos.si + 1) % FF_Q), ((pos.si + 1) / FF_Q) & 1);
+        if (!__any_sync(0xffffffffu, ready) && !warp_wait(FF_BAR(full, slot), par, poison, status, 3, pos.si)) return false;
+        const uint32_t done = bar_test(FF_BAR(done, slot), par);
+        ready = bar_test(FF_BAR(full, (pos.si + 1) % FF_Q), ((pos.si + 1) / FF_Q) & 1);
         uint64_t s2[NG];
 #pragma unroll
         for (int g = 0; g < NG; ++g) {
@@ -495,25 +399,25 @@ __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im
                 total[c / 2 + 1] = fma2(m2, xb, total[c / 2 + 1]);
             }
         }
-        if (!__any_sync(0xffffffffu, done) && !ff_wait(FF_BAR(done, slot), par, poison, status, 4, pos.si)) return false;
+        if (!__any_sync(0xffffffffu, done) && !warp_wait(FF_BAR(done, slot), par, poison, status, 4, pos.si)) return false;
         tc_fence_after();
 #pragma unroll
         for (int g = 0; g < NG; ++g, acb.next()) {
             const uint32_t acc = acc_lanes + acb.i * (2 * FF_NT);
             uint32_t r[2][16];
-            ff_ld16(acc, r[0]);
+            tc_ld_rows16(acc, r[0]);
 #pragma unroll
             for (int c0 = 0; c0 < NC; c0 += 16) {
                 tc_wait_ld();
                 const uint32_t (&rr)[16] = r[(c0 / 16) & 1];
                 if (c0 + 16 < NC) {
-                    ff_ld16(acc + c0 + 16, r[(c0 / 16 + 1) & 1]);
+                    tc_ld_rows16(acc + c0 + 16, r[(c0 / 16 + 1) & 1]);
                 } else {   // the buffer is read: hand it back to the MMA warp, and the stage to the producer
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) {
-                        ff_arrive(FF_BAR(acc_empty, acb.i));
-                        if (g == NG - 1) ff_arrive(FF_BAR(empty, slot));
+                        bar_arrive(FF_BAR(acc_empty, acb.i));
+                        if (g == NG - 1) bar_arrive(FF_BAR(empty, slot));
                     }
                 }
 #pragma unroll
@@ -529,8 +433,8 @@ __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im
             for (int it = 0; it < im.n_pool; ++it, ++pos.si) {
                 const uint32_t slot = pos.si % FF_Q;
                 pos.place(im.need_pool(), p.ring_bytes);
-                if (!ff_wait(FF_BAR(done, slot), (pos.si / FF_Q) & 1, poison, status, 4, pos.si)) return false;
-                if (lane == 0) ff_arrive(FF_BAR(empty, slot));
+                if (!warp_wait(FF_BAR(done, slot), (pos.si / FF_Q) & 1, poison, status, 4, pos.si)) return false;
+                if (lane == 0) bar_arrive(FF_BAR(empty, slot));
             }
             ready = 0;
             tc_fence_after();
@@ -539,7 +443,7 @@ __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im
 #pragma unroll
             for (int c0 = 0; c0 < NC; c0 += 16) {
                 uint32_t r[16];
-                ff_ld16(acc + c0, r);
+                tc_ld_rows16(acc + c0, r);
                 tc_wait_ld();
 #pragma unroll
                 for (int c = 0; c < 16; c += 2)
@@ -548,12 +452,12 @@ __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) ff_arrive(FF_BAR(acc_empty, acb.i));
+            if (lane == 0) bar_arrive(FF_BAR(acc_empty, acb.i));
             acb.next();
         }
         // SwiGLU.  Lanes l (gate row) and l ^ 8 (the matching up row) split the columns between them: the gate lane
         // takes the first half, the up lane the second, one value each crosses per column.
-        if (ic && !ff_wait(FF_BAR(hfree, 0), (ic - 1) & 1, poison, status, 5, ic)) return false;
+        if (ic && !warp_wait(FF_BAR(hfree, 0), (ic - 1) & 1, poison, status, 5, ic)) return false;
         const bool up = (lane & 8) != 0;
         const int hid = 64 * mt + 8 * (2 * q + (lane >> 4)) + (lane & 7);   // hidden unit within the block's 128
 #pragma unroll
@@ -573,8 +477,8 @@ __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im
             }
         }
         __syncwarp();
-        if (lane == 0) ff_arrive(FF_BAR(hready, 0));
-        if (!ff_wait(FF_BAR(hready, 0), ic & 1, poison, status, 6, ic)) return false;
+        if (lane == 0) bar_arrive(FF_BAR(hready, 0));
+        if (!warp_wait(FF_BAR(hready, 0), ic & 1, poison, status, 6, ic)) return false;
         // h of eight hidden units of one token per thread: operand tile of the down GEMM, scaled for its codes
         const int t = 32 * fw + lane;
         const int oct = t & 15;
@@ -606,7 +510,7 @@ __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im
             }
         }
         __syncwarp();
-        if (lane == 0) ff_arrive(FF_BAR(hfree, 0));
+        if (lane == 0) bar_arrive(FF_BAR(hfree, 0));
     } else {
         float* yb = p.ws.ypart + (size_t)im.split * p.split_stride + (size_t)im.row0 * p.L->d + im.rb * RB + row;
         const size_t d = p.L->d;
@@ -630,7 +534,7 @@ __device__ __noinline__ void ff_fold_role(const FfParams& p, FfRole R, uint8_t* 
     FfCycle<FF_NB> acb;
     uint32_t ready = 0;
     int ic = 0, cur = 0;
-    FfPos pos;
+    RingPos pos;
     for (int g = blockIdx.x; g < R.total && ok; g += gridDim.x, ++ic) {
         const FfItem im = ff_item_uni(p.ksplit, R.tab, g, cur, R.n_kc);
         if (im.n_mma <= 16)
@@ -655,7 +559,7 @@ __device__ __noinline__ void ff_mma_role(const FfParams& p, FfRole R) {
     int32_t* status = p.ws.status;
     volatile int* poison = &S->poison;
     int cur = 0;
-    FfPos pos;
+    RingPos pos;
     // ---------------- MMA issuer: warp-uniform, one elected lane issues ----------------
     // (A stored A buffer vouches for the stage's operand tile: the expand warps waited for it.)
     bool ok = true;
@@ -675,8 +579,8 @@ __device__ __noinline__ void ff_mma_role(const FfParams& p, FfRole R) {
             FfCycle<FF_NB> acb1 = acb;
             if (G == 64 && !pool) acb1.next();
             if (!__any_sync(0xffffffffu, ready)) {
-                ok = ff_wait(FF_BAR(acc_empty, acb1.i), acb1.par ^ 1, poison, status, 8, pos.si) &&
-                     ff_wait(FF_BAR(a_full, ab.i), ab.par, poison, status, 9, pos.si);
+                ok = warp_wait(FF_BAR(acc_empty, acb1.i), acb1.par ^ 1, poison, status, 8, pos.si) &&
+                     warp_wait(FF_BAR(a_full, ab.i), ab.par, poison, status, 9, pos.si);
                 if (!ok) break;
             }
             tc_fence_after();
@@ -693,7 +597,7 @@ __device__ __noinline__ void ff_mma_role(const FfParams& p, FfRole R) {
             // main and cached-channel stages alike: an upper bound of what the next stage waits for
             FfCycle<FF_NB> nx = acb;
             if (G == 64) nx.next();
-            ready = ff_test(FF_BAR(acc_empty, nx.i), nx.par ^ 1) & ff_test(FF_BAR(a_full, ab.i), ab.par);
+            ready = bar_test(FF_BAR(acc_empty, nx.i), nx.par ^ 1) & bar_test(FF_BAR(a_full, ab.i), ab.par);
             // operand tile: main [row group][k octet 16][8][8] + sums, cached channels [row group][k octet 4][8][8]
             ff_mma_stage<G>(d0, d1, a0, FF_NT, tc_desc(xu, 128, pool ? 512 : FF_RG),
                             __shfl_sync(0xffffffffu, idesc, 0), acc_flag, pool ? 0u : 1u);
@@ -787,7 +691,7 @@ __global__ void __launch_bounds__(FF_THREADS, 1) ffn_fold_kernel(const __grid_co
     const int cap = p.ring_bytes;
     const uint32_t sb = smem_u32(smem), ring_a = sb + p.off_ring;
     int cur = 0;
-    FfPos pos;
+    RingPos pos;
 
     FfRole R;
     R.S = S; R.tab = tab; R.sb = sb; R.ring = ring_a; R.tbase = tbase; R.total = total; R.n_kc = n_kc;

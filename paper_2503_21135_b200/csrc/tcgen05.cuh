@@ -81,18 +81,11 @@ __device__ __forceinline__ void tc_commit_elect(uint64_t* bar) {
 // Two-CTA forms (cta_group::2): one MMA spans the tensor cores of both CTAs of a cluster, M = 256 (each CTA
 // holds 128 rows of A in its tensor memory and gets 128 rows of D), each CTA's shared memory holds N/2 rows
 // of B at the same offset; a commit can signal the barrier at one offset in both CTAs.
-__device__ __forceinline__ void tc2_mma_ts_elect(uint32_t d, uint32_t a, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\telect.sync _|q, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
-        "r"(a), "l"(bdesc), "r"(idesc), "r"(acc)
-        : "memory");
-}
-__device__ __forceinline__ void tc2_commit_both_elect(uint64_t* bar) {
+__device__ __forceinline__ void tc2_commit_both_elect(uint32_t bar) {
     asm volatile(
         "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
         "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(
-            smem_u32(bar)),
+            bar),
         "h"((uint16_t)3)
         : "memory");
 }
@@ -101,6 +94,16 @@ __device__ __forceinline__ void tc_ld_x2(uint32_t taddr, uint32_t (&r)[8]) {
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(taddr)
                  : "memory");
+}
+
+// One tensor-memory lane (weight row) per lane, 16 consecutive accumulator columns
+__device__ __forceinline__ void tc_ld_rows16(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
 }
 
 }  // namespace dyn
