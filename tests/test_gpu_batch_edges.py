@@ -288,3 +288,20 @@ def test_either_streaming_variant_of_a_small_batch(group_size):
         assert gpu.kernel_launches() - before == 8   # front, two of either FFN launch, statistics, correction, combine
         ends = [t for i in range(3) if counts[i] for t in np.flatnonzero(e == i)[[0, -1]]]
         _check(cfg, gpu, ora, x, lg, np.unique(np.array(ends, np.int32)))
+
+
+@pytest.mark.parametrize("d_model,group_size", [(256, 128), (512, 64), (768, 128)])
+def test_token_tiles_of_the_pair_kernel(d_model, group_size):
+    """Rows around its tiles (even ones of at most 256 rows, an MMA of 32 at a time) and around 128, up to where two items
+    have accumulators of their own; several items a pair of SMs, narrow and wide ones in turn; an item of two stages and one
+    of four are wholly dequantized ahead of the epilogue before them."""
+    counts = [33, 128, 129, 256, 257, 513, 160, 96]
+    T = sum(counts)
+    cfg, gpu, ora = _layer(T, n_experts=8, top_k=1, group_size=group_size, d_model=d_model, d_ff=4096)
+    e = np.concatenate([np.full(c, i) for i, c in enumerate(counts)])[np.random.default_rng(7).permutation(T)]
+    lg = torch.zeros((T, 8))
+    lg[torch.arange(T), torch.from_numpy(e)] = 4.0
+    rows = [np.flatnonzero(e == i) for i in range(8)]   # token-ascending inside an expert
+    toks = np.concatenate([r[sorted({0, 31, 32, len(r) // 2, 127 % len(r), 128 % len(r), 159 % len(r), 160 % len(r), 255 % len(r),
+                                     256 % len(r), len(r) - 1})] for r in rows])
+    _check(cfg, gpu, ora, wl.activations(cfg, T, step=36), lg, toks)
