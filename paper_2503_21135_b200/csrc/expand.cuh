@@ -14,7 +14,7 @@ struct Codes;
 template <>
 struct Codes<2> { uint32_t w[2], ws[2]; };
 template <>
-struct Codes<3> { uint32_t w[2], ws[2], t0[2], t1[2]; };
+struct Codes<3> { uint32_t w[2], ws[2], t0[2], t1[2]; };  // W of the half and its >> 9; fields 5, 6; field 7
 template <>
 struct Codes<4> { uint32_t w[4], ws[4]; };
 template <>
@@ -28,7 +28,13 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     return r;
 }
 
-__device__ __forceinline__ uint32_t rotr32(uint32_t v, int n) { return __funnelshift_r(v, v, n); }
+// 3-bit words of one row half: the half chunk's own word, then the fields in W2 and the spread one.
+__device__ __forceinline__ void codes3(Codes<3>& c, int half, int rh, uint32_t w0, uint32_t w1, uint32_t w2) {
+    c.w[rh] = half ? w1 : w0;
+    c.ws[rh] = c.w[rh] >> 9;
+    c.t0[rh] = half ? w2 >> 9 : w2;
+    c.t1[rh] = half ? (c.ws[rh] & 0x00400040u) | ((w0 >> 8) & 0x00800080u) | ((w2 >> 7) & 0x01000100u) : w2;
+}
 
 template <int BITS>
 __device__ __forceinline__ void load_codes(Codes<BITS>& c, const uint8_t* atom, int lane, int half) {
@@ -62,12 +68,10 @@ __device__ __forceinline__ void load_codes(Codes<BITS>& c, const uint8_t* atom, 
         c.w[0] = v.x; c.w[1] = v.y;
         c.ws[0] = v.x >> 10; c.ws[1] = v.y >> 10;
     } else {
-        const uint2 v = *reinterpret_cast<const uint2*>(atom + lane * 16 + half * 8);
-        const uint2 hb = *reinterpret_cast<const uint2*>(atom + 512 + lane * 8);
-        c.w[0] = v.x; c.w[1] = v.y;
-        c.ws[0] = v.x >> 8; c.ws[1] = v.y >> 8;
-        c.t0[0] = rotr32(hb.x, half * 8); c.t0[1] = rotr32(hb.y, half * 8);
-        c.t1[0] = rotr32(hb.x, half * 8 + 1); c.t1[1] = rotr32(hb.y, half * 8 + 1);
+        const uint4 v = *reinterpret_cast<const uint4*>(atom + lane * 16);
+        const uint2 x = *reinterpret_cast<const uint2*>(atom + 512 + lane * 8);
+        codes3(c, half, 0, v.x, v.z, x.x);
+        codes3(c, half, 1, v.y, v.w, x.y);
     }
 }
 
@@ -115,12 +119,11 @@ __device__ __forceinline__ void expand(const Codes<BITS>& c, uint32_t (&a)[4]) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int phi = 2 * S4 + h;
-            const int i = phi & 3;
+            const int o = phi <= 4 ? 3 * (phi % 3) : 3 * (phi - 5);
 #pragma unroll
             for (int rh = 0; rh < 2; ++rh) {
-                const uint32_t lo = (phi < 4) ? c.w[rh] : c.ws[rh];
-                const uint32_t hi = (phi < 4) ? c.t0[rh] : c.t1[rh];
-                a[rh + 2 * h] = (lo & (0x00030003u << (2 * i))) | ((hi & (0x00040004u << (2 * i))) | MAGIC);
+                const uint32_t src = phi <= 2 ? c.w[rh] : phi <= 4 ? c.ws[rh] : phi <= 6 ? c.t0[rh] : c.t1[rh];
+                a[rh + 2 * h] = (src & (0x00070007u << o)) | MAGIC;
             }
         }
     }
@@ -143,19 +146,15 @@ __device__ __forceinline__ void load_raw(uint32_t (&w)[16], uint32_t atom, int l
 }
 template <int BITS, int HALF>
 __device__ __forceinline__ void codes_of(Codes<BITS>& c, const uint32_t (&w)[16]) {
-    if constexpr (BITS == 2 || BITS == 3) {
+    if constexpr (BITS == 2) {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             c.w[i] = w[2 * HALF + i];
-            c.ws[i] = c.w[i] >> (BITS == 2 ? 10 : 8);
+            c.ws[i] = c.w[i] >> 10;
         }
-        if constexpr (BITS == 3) {
+    } else if constexpr (BITS == 3) {
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                c.t0[i] = rotr32(w[4 + i], HALF * 8);
-                c.t1[i] = rotr32(w[4 + i], HALF * 8 + 1);
-            }
-        }
+        for (int i = 0; i < 2; ++i) codes3(c, HALF, i, w[i], w[2 + i], w[4 + i]);
     } else if constexpr (BITS == 8) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) c.w[i] = w[8 * HALF + i];
@@ -182,7 +181,7 @@ __device__ __forceinline__ void codes_of(Codes<BITS>& c, const uint32_t (&w)[16]
 template <int BITS>
 __host__ __device__ constexpr int code_offset(int s4, int h) {
     const int phi = 2 * s4 + h;
-    return BITS == 2 ? (phi <= 4 ? 2 * phi : 2 * phi - 10) : BITS == 3 ? 2 * (phi & 3) : (BITS == 4 || BITS == 6) ? 4 * h : 0;
+    return BITS == 2 ? (phi <= 4 ? 2 * phi : 2 * phi - 10) : BITS == 3 ? (phi <= 4 ? 3 * (phi % 3) : 3 * (phi - 5)) : (BITS == 4 || BITS == 6) ? 4 * h : 0;
 }
 
 }  // namespace dyn

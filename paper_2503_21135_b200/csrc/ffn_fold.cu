@@ -192,51 +192,10 @@ __device__ __forceinline__ void ff_mma_stage(uint32_t d0, uint32_t d1, uint32_t 
 // ---- expand: codes of two atoms of every other stage -> A buffer ---------------------------------------------------
 template <int BITS>
 __device__ __forceinline__ void ff_load_codes(Codes<BITS> (&c)[2], uint32_t atom, int lane) {   // both half chunks
-    if constexpr (BITS == 2 || BITS == 3) {
-        const uint4 v = lds128(atom + lane * 16);
-        c[0].w[0] = v.x; c[0].w[1] = v.y; c[1].w[0] = v.z; c[1].w[1] = v.w;
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int i = 0; i < 2; ++i) c[h].ws[i] = c[h].w[i] >> (BITS == 2 ? 10 : 8);
-        if constexpr (BITS == 3) {
-            const uint2 hb = lds64(atom + 512 + lane * 8);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                c[h].t0[0] = rotr32(hb.x, h * 8); c[h].t0[1] = rotr32(hb.y, h * 8);
-                c[h].t1[0] = rotr32(hb.x, h * 8 + 1); c[h].t1[1] = rotr32(hb.y, h * 8 + 1);
-            }
-        }
-    } else if constexpr (BITS == 4 || BITS == 6) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint4 v = lds128(atom + h * 512 + lane * 16);
-            c[h].w[0] = v.x; c[h].w[1] = v.y; c[h].w[2] = v.z; c[h].w[3] = v.w;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) c[h].ws[i] = c[h].w[i] >> 8;
-        }
-        if constexpr (BITS == 6) {
-            const uint4 hb = lds128(atom + 1024 + lane * 16);
-            const uint32_t hw[2][2] = {{hb.x, hb.y}, {hb.z, hb.w}};
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                for (int rh = 0; rh < 2; ++rh) {
-                    const uint32_t sw = prmt(hw[h][rh], 0u, 0x2301u);   // bytes of each 16-bit half swapped
-                    c[h].t[rh][0] = hw[h][rh];
-                    c[h].t[rh][1] = hw[h][rh] >> 2;
-                    c[h].t[rh][2] = sw;
-                    c[h].t[rh][3] = sw >> 2;
-                }
-        }
-    } else {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint4 v0 = lds128(atom + (2 * h) * 512 + lane * 16), v1 = lds128(atom + (2 * h + 1) * 512 + lane * 16);
-            c[h].w[0] = v0.x; c[h].w[1] = v0.y; c[h].w[2] = v0.z; c[h].w[3] = v0.w;
-            c[h].w[4] = v1.x; c[h].w[5] = v1.y; c[h].w[6] = v1.z; c[h].w[7] = v1.w;
-        }
-    }
+    uint32_t raw[16];
+    load_raw<BITS>(raw, atom, lane);
+    codes_of<BITS, 0>(c[0], raw);
+    codes_of<BITS, 1>(c[1], raw);
 }
 
 template <int BITS>
