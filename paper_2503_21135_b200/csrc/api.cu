@@ -97,8 +97,9 @@ inline bool decode_sized(const dynamo_layer_desc& D, int T) {
 }
 // Batches that take the fold kernel: more tokens than the streaming kernel serves alone, and few enough that most
 // experts have one 64-row tile (the codes are expanded once per tile).  Layer of eight experts, top-2, 4096 x 14336:
-// 65 tokens 249 us (streaming kernel 255), 100 tokens 269 (streaming and pair kernel 357), 139: 311 (523),
-// 200: 344 (465), 256 (64 rows an expert): 462 (468), 500: 671 (541).  Not with shared experts, whose rows are all the
+// 70 tokens 242 us (streaming and pair kernel 264), 100: 248 (332), 139: 300 (444), 200: 324 (380), 240: 391 (382),
+// 248 (62 rows an expert): 420 (384); the last batches stay for their exact products (the pair kernel rounds the weights).
+// Not with shared experts, whose rows are all the
 // tokens: the fine-grained layer at 128 tokens 240 us (176), at 300 260 (212).
 // Small experts keep a CTA for 16 stages at a time, and its start and its end weigh: where there are many of them, only
 // between a mean of 20 rows (the streaming kernel's second pass begins at 25) and 40 (an expert's second tile at 65).
