@@ -367,17 +367,6 @@ __global__ void __launch_bounds__(1024) scan_kernel(WsDev ws, int E, int Es, int
 // multiplied by 2^x_scale_exp(bits of the row's expert, k) so that the FFN kernels can use packed codes
 // in place; the per-group sums are of the unscaled fp16 values.
 enum : int { LAY_ROWS, LAY_TILES };   // which kernel reads the row: streaming, pair
-// A cached channel's activation, zero where it is not significant (ch < 0: no channel).  Mask word and activation are loaded
-// side by side.
-__device__ __forceinline__ float pool_value(const __nv_bfloat16* xr, const uint32_t* mask, int ch, bool& clamped) {
-    if (ch < 0) return 0.f;
-    const float xv = __bfloat162float(xr[ch]);
-    const bool sig = (mask[ch >> 5] >> (ch & 31)) & 1u;
-    bool hit = false;
-    const float v = clamp_act(xv, hit);
-    clamped |= hit && sig;
-    return sig ? v : 0.f;
-}
 __device__ __forceinline__ void gather_row(const LayerDev* __restrict__ L, const WsDev& ws,
                                            const __nv_bfloat16* __restrict__ x, int row, int t, int e, int seg0, int lay, int part, int n_parts) {
     const bool tc = lay != LAY_ROWS;
@@ -393,18 +382,6 @@ __device__ __forceinline__ void gather_row(const LayerDev* __restrict__ L, const
     const float sc1 = __uint_as_float((uint32_t)(127 + x_scale_exp(bits, 4 * lane + 2)) << 23);
     const int rg = row >> 3, rr = row & 7;
     bool clamped = false;
-    // The cached channel of column j (see below; -1: none).  The first one is asked for ahead of the row, and mask bit and
-    // activation of a channel are then loaded together: three latencies one behind the other stood at the end before (1 token of
-    // 4096 64.2 -> 63.6 us a pass, 64 of 512 26.3 -> 25.8).
-    const int P = L->P, P_pad = sw ? L->P_pad : 0;
-    const int32_t* ci = L->cache_idx + (long long)e * P;
-    auto channel = [&](int j) -> int {
-        // operand position kp of a 16-column step holds pool column 16*step + sigma(kp): the A tile reaches TMEM through an
-        // ldmatrix fragment whose k pairs (2t, 2t+1 | 2t+8, 2t+9) land on TMEM k 4t .. 4t+3.
-        const int kp = j & 15, pj = tc ? (j & ~15) + 2 * (kp >> 2) + (kp & 1) + ((kp & 2) ? 8 : 0) : j;
-        return t >= 0 && j < P_pad && pj < P ? ci[pj] : -1;
-    };
-    int ch_next = channel(32 * part + lane);
     // four chunks at a time, their loads in flight together: a chunk's load, mask and sum are a chain of latencies
     for (int c0 = part; c0 < n_kc; c0 += 4 * n_parts) {
         uint2 raw[4];
@@ -460,15 +437,32 @@ __device__ __forceinline__ void gather_row(const LayerDev* __restrict__ L, const
     // currently significant: the FFN kernels multiply them with the contiguous 8-bit-valued tiles of the
     // whole cache pool, so a switch only has to flip mask bits.
     if (!sw) return;
+    const int P = L->P, P_pad = L->P_pad;
+    const int32_t* ci = L->cache_idx + (long long)e * P;
     uint8_t* xp = reinterpret_cast<uint8_t*>(ws.xsig);
     for (int j = 32 * part + lane; j < P_pad; j += 32 * n_parts) {
-        const int pq = j >> 5, col = j & 31, ch = ch_next;
-        ch_next = channel(j + 32 * n_parts);
-        const float v = pool_value(xr, mask, ch, clamped);
-        // streaming path [row][32 columns]; else an 8-row operand tile of group pq: [k-octet 4][row 8][8 k] fp16 = 512 B
-        uint8_t* dst = tc ? xp + xpool_off(pq, 8 * rg, ws.Rcap) + (col >> 3) * 128 + rr * 16 + (col & 7) * 2
-                          : xp + xpool_off(pq, row, ws.Rcap) + col * 2;
-        *reinterpret_cast<__half*>(dst) = __float2half_rn(v);
+        const int pq = j >> 5, col = j & 31;
+        if (!tc) {
+            float v = 0.f;
+            if (j < P) {
+                const int ch = ci[j];
+                if ((mask[ch >> 5] >> (ch & 31)) & 1u) v = clamp_act(__bfloat162float(xr[ch]), clamped);
+            }
+            *reinterpret_cast<__half*>(xp + xpool_off(pq, row, ws.Rcap) + col * 2) = __float2half_rn(v);
+        } else {
+            // operand position kp of a 16-column step holds pool column 16*step + sigma(kp): the A tile reaches
+            // TMEM through an ldmatrix fragment whose k pairs (2t, 2t+1 | 2t+8, 2t+9) land on TMEM k 4t .. 4t+3.
+            const int step = col >> 4, kp = col & 15;
+            const int pj = pq * 32 + step * 16 + 2 * (kp >> 2) + (kp & 1) + ((kp & 2) ? 8 : 0);
+            float v = 0.f;
+            if (t >= 0 && pj < P) {
+                const int ch = ci[pj];
+                if ((mask[ch >> 5] >> (ch & 31)) & 1u) v = clamp_act(__bfloat162float(xr[ch]), clamped);
+            }
+            // 8-row operand tile of group pq: [k-octet 4][row 8][8 k] fp16 = 512 B
+            *reinterpret_cast<__half*>(xp + xpool_off(pq, 8 * rg, ws.Rcap) + (col >> 3) * 128 + rr * 16 + (col & 7) * 2) =
+                __float2half_rn(v);
+        }
     }
 }
 
@@ -486,9 +480,8 @@ __global__ void __launch_bounds__(256) gather_kernel(const LayerDev* __restrict_
 // tile, so that four lanes read 64 consecutive bytes of a row and a warp writes 512 consecutive bytes; the chain of
 // loads that finds a row's expert and token is paid once per group.  One CTA per row wrote every 128-byte line of a
 // tile from eight CTAs and took 59 us at 2048 fine-grained tokens (16.9 k rows of 2048), this 36.3.  grid.y cuts the chunks of a
-// group where there are few groups.  Four CTAs an SM: with the 98 registers that the compiler takes otherwise two, and 2048
-// fine-grained tokens 438 us a pass for 421.
-__global__ void __launch_bounds__(256, 4) gather_group_kernel(const LayerDev* __restrict__ L, WsDev ws,
+// group where there are few groups.
+__global__ void __launch_bounds__(256) gather_group_kernel(const LayerDev* __restrict__ L, WsDev ws,
                                                            const __nv_bfloat16* __restrict__ x) {
     pdl_prologue();
     const int row0 = 8 * blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
