@@ -14,7 +14,7 @@ struct Codes;
 template <>
 struct Codes<2> { uint32_t w[2], ws[2]; };
 template <>
-struct Codes<3> { uint32_t w[2], ws[2], t0[2], t1[2]; };  // W of the half and its >> 9; fields 5, 6; field 7
+struct Codes<3> { uint32_t w[2], ws[2], t0[2], t1[2]; };  // W(jh), its >> 6; W2 or its >> 8; the spread fields
 template <>
 struct Codes<4> { uint32_t w[4], ws[4]; };
 template <>
@@ -28,12 +28,14 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     return r;
 }
 
-// 3-bit words of one row half: the half chunk's own word, then the fields in W2 and the spread one.
-__device__ __forceinline__ void codes3(Codes<3>& c, int half, int rh, uint32_t w0, uint32_t w1, uint32_t w2) {
-    c.w[rh] = half ? w1 : w0;
-    c.ws[rh] = c.w[rh] >> 9;
-    c.t0[rh] = half ? w2 >> 9 : w2;
-    c.t1[rh] = half ? (c.ws[rh] & 0x00400040u) | ((w0 >> 8) & 0x00800080u) | ((w2 >> 7) & 0x01000100u) : w2;
+// 3-bit words of one row half, that of the half chunk and the shared one -> the two views of each; two of the eight fields
+// are spread over both words.
+__device__ __forceinline__ uint32_t bits_of(uint32_t mask, uint32_t a, uint32_t b) { return (a & mask) | (b & ~mask); }
+__device__ __forceinline__ void codes3(Codes<3>& c, int half, int rh, uint32_t w, uint32_t x) {
+    c.w[rh] = w;
+    c.ws[rh] = w >> 6;
+    c.t0[rh] = half ? x >> 8 : x;
+    c.t1[rh] = bits_of(0x00880088u, w, bits_of(0x00440044u, w >> 9, half ? x >> 7 : x << 1));
 }
 
 template <int BITS>
@@ -68,10 +70,10 @@ __device__ __forceinline__ void load_codes(Codes<BITS>& c, const uint8_t* atom, 
         c.w[0] = v.x; c.w[1] = v.y;
         c.ws[0] = v.x >> 10; c.ws[1] = v.y >> 10;
     } else {
-        const uint4 v = *reinterpret_cast<const uint4*>(atom + lane * 16);
+        const uint2 v = *reinterpret_cast<const uint2*>(atom + lane * 16 + half * 8);
         const uint2 x = *reinterpret_cast<const uint2*>(atom + 512 + lane * 8);
-        codes3(c, half, 0, v.x, v.z, x.x);
-        codes3(c, half, 1, v.y, v.w, x.y);
+        codes3(c, half, 0, v.x, x.x);
+        codes3(c, half, 1, v.y, x.y);
     }
 }
 
@@ -119,11 +121,10 @@ __device__ __forceinline__ void expand(const Codes<BITS>& c, uint32_t (&a)[4]) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int phi = 2 * S4 + h;
-            const int o = phi <= 4 ? 3 * (phi % 3) : 3 * (phi - 5);
 #pragma unroll
             for (int rh = 0; rh < 2; ++rh) {
-                const uint32_t src = phi <= 2 ? c.w[rh] : phi <= 4 ? c.ws[rh] : phi <= 6 ? c.t0[rh] : c.t1[rh];
-                a[rh + 2 * h] = (src & (0x00070007u << o)) | MAGIC;
+                const uint32_t src = phi < 4 ? (h ? c.ws[rh] : c.w[rh]) : (h ? c.t1[rh] : c.t0[rh]);
+                a[rh + 2 * h] = (src & (0x00070007u << (2 * (phi & 3)))) | MAGIC;
             }
         }
     }
@@ -154,7 +155,7 @@ __device__ __forceinline__ void codes_of(Codes<BITS>& c, const uint32_t (&w)[16]
         }
     } else if constexpr (BITS == 3) {
 #pragma unroll
-        for (int i = 0; i < 2; ++i) codes3(c, HALF, i, w[i], w[2 + i], w[4 + i]);
+        for (int i = 0; i < 2; ++i) codes3(c, HALF, i, w[2 * HALF + i], w[4 + i]);
     } else if constexpr (BITS == 8) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) c.w[i] = w[8 * HALF + i];
@@ -181,7 +182,7 @@ __device__ __forceinline__ void codes_of(Codes<BITS>& c, const uint32_t (&w)[16]
 template <int BITS>
 __host__ __device__ constexpr int code_offset(int s4, int h) {
     const int phi = 2 * s4 + h;
-    return BITS == 2 ? (phi <= 4 ? 2 * phi : 2 * phi - 10) : BITS == 3 ? (phi <= 4 ? 3 * (phi % 3) : 3 * (phi - 5)) : (BITS == 4 || BITS == 6) ? 4 * h : 0;
+    return BITS == 2 ? (phi <= 4 ? 2 * phi : 2 * phi - 10) : BITS == 3 ? 2 * (phi & 3) : (BITS == 4 || BITS == 6) ? 4 * h : 0;
 }
 
 }  // namespace dyn

@@ -131,8 +131,8 @@ __device__ __forceinline__ T2Item t2_item(const T2Expert* tab, int g, int& curso
 template <int BITS, int HALF>
 __device__ __forceinline__ void t2_dequant_half(const uint32_t (&raw)[16], uint32_t prm0, uint32_t prm1, uint32_t (&regs)[16]) {
     constexpr int BIAS = BITS == 2 ? 4 : (BITS == 3 ? 3 : ((BITS == 4 || BITS == 6) ? 2 : 0));
-    constexpr int NOFF = BITS == 2 ? 5 : (BITS == 3 ? 3 : ((BITS == 4 || BITS == 6) ? 2 : 1));  // distinct offsets 0, step, 2*step, ...
-    constexpr int OSTEP = (BITS == 4 || BITS == 6) ? 4 : (BITS == 3 ? 3 : 2);
+    constexpr int NOFF = BITS == 2 ? 5 : (BITS == 3 ? 4 : ((BITS == 4 || BITS == 6) ? 2 : 1));  // distinct offsets 0, step, 2*step, ...
+    constexpr int OSTEP = (BITS == 4 || BITS == 6) ? 4 : 2;
     const __half2 k1024 = __float2half2_rn(1024.f);
     __half2 S2[2], M2[2][NOFF];
 #pragma unroll

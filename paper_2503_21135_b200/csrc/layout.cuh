@@ -16,15 +16,19 @@
 //   2-bit: atom = [32 lanes x 16 B]; word jh*2 + rowhalf (jh = s/4, the 64-k half chunk);
 //          field phi = 2*(s%4) + h at bits [2phi, 2phi+2) (even k) and +16 (odd k);
 //          phi <= 4 used in place (o = 2phi), phi >= 5 after >> 10 (o = 2phi - 10).
-//   3-bit: three words per row half hold the sixteen fields of a lane (five to a 16-bit half, and bit 15 of each word):
-//          W0 and W1 (jh = 0, 1; [32 lanes x 16 B], word jh*2 + rowhalf) fields phi = 0..4 of their half chunk at bits 3phi:
-//          phi <= 2 in place (o = 3phi), 3 and 4 after >> 9 (o = 3phi - 9); W2 ([32 lanes x 8 B], word = rowhalf)
-//          phi = 5..7 of jh = 0 at bits 3(phi-5), in place, and phi = 5, 6 of jh = 1 at bits 9 + 3(phi-5), after >> 9.
-//          phi = 7 of jh = 1 is spread over the three bits 15: bit 0 of the code in W1 (on bit 6 after >> 9), bit 1 in W0
-//          (on 7 after >> 8), bit 2 in W2 (on 8 after >> 7), so o = 6 as for phi = 7 of jh = 0.  46 logical
-//          instructions an atom and lane (32 of them the masks that every width has); a 2-bit and a 1-bit plane took 76.
-//          Layers with two 3-bit experts of eight (4096 x 14336), us a pass: 1 token 72 -> 65, 8: 155 -> 150, 4 x 16:
-//          688 -> 665, 139: 302 -> 293.
+//   3-bit: three words per row half hold the sixteen fields of a lane: W0 and W1 (jh = 0, 1; [32 lanes x 16 B], word
+//          jh*2 + rowhalf) and W2 ([32 lanes x 8 B], word = rowhalf), each with four whole fields at bits 0, 4, 8 and 12 of its
+//          16-bit halves and single bits at 3, 7, 11 and 15.  o = 2(phi % 4).
+//          phi = 0, 2 at bits 0, 4 of W(jh), in place; phi = 1, 3 at bits 8, 12 after >> 6; phi = 4, 6 of jh = 0 at bits 0, 4
+//          of W2, in place, of jh = 1 at bits 8, 12 after >> 8.  phi = 5, 7 (o = 2, 6) are spread over single bits that lie
+//          four apart as the fields do, so one shift of a word serves both: bit 0 of the code at bits 11, 15 of W(jh) (>> 9),
+//          bit 1 at 3, 7 of W(jh), in place, bit 2 in W2 at 3, 7 (jh = 0, << 1) or 11, 15 (jh = 1, >> 7).  54 logical
+//          instructions an atom and lane (32 of them the masks that every width has); a 2-bit and a 1-bit plane take 76:
+//          1, 4, 12, 32, 64 tokens of a layer with two 3-bit experts of eight (4096 x 14336, mean of eight routers) 65, 124,
+//          169, 201, 244 us a pass, as planes 68, 128, 170, 205, 244.  Fields packed three bits apart (o = 0, 3, 6; 46
+//          instructions) take 63, 123, 166, 199, 242, but the tensor cores align the products of an MMA by the operands'
+//          exponents, and with o = 0 in three steps of four instead of two a sum over 14336 hidden activations from 0.02 to 2
+//          is twice as far from its value in 64 bits (2-norm 2.7e-5 -> 5.0e-5).
 //   4-bit: atom = 2 planes (= half chunks) x [32 lanes x 16 B]; word rowhalf*2 + (s%4)/2;
 //          nibble phi = 2*(s%2) + h at bits [4phi, 4phi+4) (even k) and +16 (odd k);
 //          phi <= 1 in place (o = 4phi), phi >= 2 after >> 8 (o = 4phi - 8): o = 4h.
@@ -50,7 +54,7 @@ struct CodeLoc {
 
 // Number of parts that the code of input index kk lies in.
 __host__ __device__ inline int code_parts(int bits, int kk) {
-    return bits == 6 ? 2 : (bits == 3 && (kk & 0x72) == 0x72 ? 3 : 1);
+    return bits == 6 ? 2 : (bits == 3 && (kk & 0x22) == 0x22 ? 3 : 1);
 }
 
 // r: row in atom (0..15), kk: k in chunk (0..127).  For 6-bit, part 0 = low four bits, part 1 = high two bits; for 3-bit,
@@ -85,12 +89,13 @@ __host__ __device__ inline CodeLoc code_loc(int bits, int r, int kk, int part) {
         L.width = 2;
     } else {  // 3-bit
         const int phi = 2 * s4 + h;
-        const bool split = jh == 1 && phi == 7;
-        const int w = split ? (part == 0 ? 1 : part == 1 ? 0 : 2) : (phi <= 4 ? jh : 2);
+        const bool spread = (phi & 5) == 5;
+        const int w = (spread ? part < 2 : phi < 4) ? jh : 2;
         L.byte_off = (w == 2 ? 512 + lane * 8 : lane * 16 + 8 * w) + rowhalf * 4;
-        L.shift = 16 * odd + (split ? 15 : phi <= 4 ? 3 * phi : 3 * (phi - 5) + 9 * jh);
-        L.width = split ? 1 : 3;
-        L.lo = split ? part : 0;
+        L.shift = 16 * odd + 4 * (phi >> 1 & 1) +
+                  (spread ? 3 + 8 * (part == 2 ? jh : 1 - part) : 8 * (phi < 4 ? phi & 1 : jh));
+        L.width = spread ? 1 : 3;
+        L.lo = spread ? part : 0;
     }
     return L;
 }
@@ -105,7 +110,7 @@ __host__ __device__ inline int x_scale_exp(int bits, int k) {
     const int phi = 2 * s4 + h;
     int o = 0;
     if (bits == 2) o = phi <= 4 ? 2 * phi : 2 * phi - 10;
-    else if (bits == 3) o = phi <= 4 ? 3 * (phi % 3) : 3 * (phi - 5);
+    else if (bits == 3) o = 2 * (phi & 3);
     else if (bits == 4 || bits == 6) o = 4 * h;
     return x_scale_bias(bits) - o;
 }

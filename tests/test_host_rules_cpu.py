@@ -110,3 +110,53 @@ def test_a_buffer_has_to_lie_within_one_registration(covers):
     assert not covers(0, 0, 16 * page, 1) and not covers(*first, 16 * page, 2 ** 64 - 1)
     top = 2 ** 64 - page
     assert covers(top, page - 1, top, page - 1) and not covers(top, page - 1, top + 8, page)
+
+
+@pytest.fixture(scope="module")
+def layout(tmp_path_factory):
+    lib = _compile(tmp_path_factory, "layout", """
+        #define __host__
+        #define __device__
+        #include "layout.cuh"
+        extern "C" int scale_exp(int bits, int k) { return dyn::x_scale_exp(bits, k); }
+        extern "C" int parts(int bits, int k) { return dyn::code_parts(bits, k); }
+        extern "C" void loc(int bits, int r, int k, int part, int* out) {
+            const dyn::CodeLoc l = dyn::code_loc(bits, r, k, part);
+            out[0] = l.byte_off; out[1] = l.shift; out[2] = l.width; out[3] = l.lo;
+        }
+        """)
+
+    def loc(bits, r, k, part):
+        out = (ctypes.c_int * 4)()
+        lib.loc(bits, r, k, part, out)
+        return list(out)
+
+    return lib, loc
+
+
+@pytest.mark.parametrize("bits,bias,offsets", [(2, 4, [0, 2, 4, 6, 8, 0, 2, 4]), (3, 3, [0, 2, 4, 6] * 2), (4, 2, [0, 4] * 4),
+                                               (6, 2, [0, 4] * 4), (8, 0, [0] * 8)])
+def test_codes_lie_at_the_offsets_that_the_sums_are_exact_for(layout, bits, bias, offsets):
+    """The activation of a code at bit offset o carries 2^(bias - o), and the tensor cores align their sums by the operands'
+    exponents: the offsets decide the last bits of a result and how exact it is (3-bit codes at 0, 3 and 6: twice the error)."""
+    lib, _ = layout
+    for k in range(256):
+        phi = 2 * (k >> 4 & 3) + (k >> 1 & 1)
+        assert lib.scale_exp(bits, k) == bias - offsets[phi]
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4, 6, 8])
+def test_every_bit_of_an_atom_belongs_to_one_code(layout, bits):
+    lib, loc = layout
+    taken = np.zeros(256 * bits * 8, np.int32)
+    for r in range(16):
+        for k in range(128):
+            code = 0
+            for part in range(lib.parts(bits, k)):
+                off, shift, width, lo = loc(bits, r, k, part)
+                assert off % 4 == 0 and 0 <= shift and shift + width <= 32
+                taken[off * 8 + shift: off * 8 + shift + width] += 1
+                assert code & (((1 << width) - 1) << lo) == 0
+                code |= ((1 << width) - 1) << lo
+            assert code == (1 << bits) - 1
+    assert np.all(taken == 1)
