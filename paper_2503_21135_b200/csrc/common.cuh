@@ -311,6 +311,13 @@ __device__ __forceinline__ void bar_arrive_leader(uint32_t bar) {
         "{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, 0;\n\tmbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}" ::"r"(bar)
         : "memory");
 }
+// Whether any lane's poll found its phase complete.  A vote does not order memory: the warp barrier behind it makes what the
+// lane that saw the phase has acquired visible to the others, which go on to read the stage.
+__device__ __forceinline__ bool warp_saw(uint32_t ok) {
+    const bool any = __any_sync(0xffffffffu, ok);
+    __syncwarp();
+    return any;
+}
 // Bounded wait of a whole warp on one barrier; false after an expired wait (here or elsewhere in the CTA).  All lanes
 // poll together and the loop is left by vote: the compiler then knows that the warp is converged behind it and keeps
 // the operands of tcgen05 instructions in uniform registers (16 MMAs issue in 165 cycles, in 1100 otherwise).
@@ -325,7 +332,7 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
             : "=r"(ok)
             : "r"(bar), "r"(parity)
             : "memory");
-        if (__any_sync(0xffffffffu, ok)) return true;
+        if (warp_saw(ok)) return true;
         if ((++n & 0x3ff) == 0) {
             if (__any_sync(0xffffffffu, *poison)) return false;
             const unsigned long long now = __shfl_sync(0xffffffffu, globaltimer_ns(), 0);

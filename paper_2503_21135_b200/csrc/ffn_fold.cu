@@ -234,7 +234,7 @@ __device__ __forceinline__ bool ff_expand_item(const FfItem& im, FfShared* S, ui
         const uint32_t si = pos.si;
         if ((si & 1) != (uint32_t)kh) continue;
         const uint32_t b = si % FF_NA, u = si - FF_NA;
-        if (!__any_sync(0xffffffffu, ready) &&
+        if (!warp_saw(ready) &&
             !warp_wait(FF_BAR(full, si % FF_Q), (si / FF_Q) & 1, &S->poison, status, 1, si))
             return false;
         // the MMAs that read this A buffer last must be complete before it is written
@@ -251,7 +251,7 @@ __device__ __forceinline__ bool ff_expand_item(const FfItem& im, FfShared* S, ui
                 for (int a = 0; a < GRP; ++a)
                     ff_load_codes<BITS>(cd[a], st + (8 * ((a0 + a) >> 1) + 2 * q + (a & 1)) * (256 * BITS), lane);
                 if (a0 == 0) {
-                    if (!__any_sync(0xffffffffu, a_free) &&
+                    if (!warp_saw(a_free) &&
                         !warp_wait(FF_BAR(done, u % FF_Q), (u / FF_Q) & 1, &S->poison, status, 2, si))
                         return false;
                     tc_fence_after();
@@ -262,7 +262,7 @@ __device__ __forceinline__ bool ff_expand_item(const FfItem& im, FfShared* S, ui
             }
         } else {
             // cached-channel stage: fp16 tiles [pool column][256 rows] -> A fragments
-            if (!__any_sync(0xffffffffu, a_free) &&
+            if (!warp_saw(a_free) &&
                 !warp_wait(FF_BAR(done, u % FF_Q), (u / FF_Q) & 1, &S->poison, status, 2, si))
                 return false;
             tc_fence_after();
@@ -339,7 +339,7 @@ __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im
         const uint32_t st = ring + pos.place(need, p.ring_bytes);
         const uint32_t slot = pos.si % FF_Q, par = (pos.si / FF_Q) & 1;
         // zero-point times the group sums, as soon as the copies have landed
-        if (!__any_sync(0xffffffffu, ready) && !warp_wait(FF_BAR(full, slot), par, poison, status, 3, pos.si)) return false;
+        if (!warp_saw(ready) && !warp_wait(FF_BAR(full, slot), par, poison, status, 3, pos.si)) return false;
         const uint32_t done = bar_test(FF_BAR(done, slot), par);
         ready = bar_test(FF_BAR(full, (pos.si + 1) % FF_Q), ((pos.si + 1) / FF_Q) & 1);
         uint64_t s2[NG];
@@ -358,7 +358,7 @@ __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im
                 total[c / 2 + 1] = fma2(m2, xb, total[c / 2 + 1]);
             }
         }
-        if (!__any_sync(0xffffffffu, done) && !warp_wait(FF_BAR(done, slot), par, poison, status, 4, pos.si)) return false;
+        if (!warp_saw(done) && !warp_wait(FF_BAR(done, slot), par, poison, status, 4, pos.si)) return false;
         tc_fence_after();
 #pragma unroll
         for (int g = 0; g < NG; ++g, acb.next()) {
@@ -537,7 +537,7 @@ __device__ __noinline__ void ff_mma_role(const FfParams& p, FfRole R) {
                                                : pos.place(need, cap) + im.blk_bytes);
             FfCycle<FF_NB> acb1 = acb;
             if (G == 64 && !pool) acb1.next();
-            if (!__any_sync(0xffffffffu, ready)) {
+            if (!warp_saw(ready)) {
                 ok = warp_wait(FF_BAR(acc_empty, acb1.i), acb1.par ^ 1, poison, status, 8, pos.si) &&
                      warp_wait(FF_BAR(a_full, ab.i), ab.par, poison, status, 9, pos.si);
                 if (!ok) break;

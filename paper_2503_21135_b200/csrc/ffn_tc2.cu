@@ -196,7 +196,7 @@ __device__ __forceinline__ T2Deq t2_deq(uint8_t* smem, uint32_t tbase, int rank,
 __device__ __forceinline__ bool t2_hand_over(const T2Deq& c, uint32_t gis, uint32_t xready) {
     const uint32_t sb = c.sb, b = gis % T2_NA;
     tc_wait_st();
-    if (!__any_sync(0xffffffffu, xready) && !warp_wait(T2_BAR(fullx, b), (gis / T2_NX) & 1, c.poison, c.status, 15, gis))
+    if (!warp_saw(xready) && !warp_wait(T2_BAR(fullx, b), (gis / T2_NX) & 1, c.poison, c.status, 15, gis))
         return false;
     tc_fence_before();
     __syncwarp();
@@ -228,7 +228,7 @@ __device__ __forceinline__ int t2_dequant_run(const T2Deq& c, int n, uint32_t gi
 #pragma unroll 1
     for (; gi < end; gi += 2) {
         const uint32_t b = gi % T2_NA, dpar = ((gi / T2_NA) & 1) ^ 1;
-        if (!__any_sync(0xffffffffu, ready) &&
+        if (!warp_saw(ready) &&
             !warp_wait(T2_BAR(full, gi % T2_NW), (gi / T2_NW) & 1, c.poison, c.status, 13, gi))
             return -1;
         const uint32_t st = sb + T2_OFF_STAGE + pos.place(NEED, T2_WRING);
@@ -248,7 +248,7 @@ __device__ __forceinline__ int t2_dequant_run(const T2Deq& c, int n, uint32_t gi
         const uint32_t a_free = bar_test(T2_BAR(done, b), dpar);
         ready = bar_test(T2_BAR(full, (gi + 2) % T2_NW), ((gi + 2) / T2_NW) & 1);
         t2_dequant_half<BITS, 0>(raw, prm[0][0], prm[1][0], regs);
-        if (!__any_sync(0xffffffffu, a_free) && !warp_wait(T2_BAR(done, b), dpar, c.poison, c.status, 14, gi)) return -1;
+        if (!warp_saw(a_free) && !warp_wait(T2_BAR(done, b), dpar, c.poison, c.status, 14, gi)) return -1;
         tc_fence_after();
         tc_st_x4(c.a_lanes + 64 * b, regs);
         t2_dequant_half<BITS, 1>(raw, prm[0][NG - 1], prm[1][NG - 1], regs);
@@ -346,7 +346,7 @@ __device__ __noinline__ void t2_mma_role(const T2Params& p, const T2Expert* tab,
             const uint32_t b = gi % T2_NA;
             // A buffer b stored by the 16 dequant warps of the pair that own the stage; each also waited for its CTA's
             // operand tile before it arrived
-            if (!__any_sync(0xffffffffu, ready)) {
+            if (!warp_saw(ready)) {
                 ok = warp_wait(T2_BAR(a_full, b), (gi / T2_NA) & 1, poison, status, 12, gi);
                 if (!ok) break;
             }
