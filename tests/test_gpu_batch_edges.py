@@ -290,14 +290,10 @@ def test_either_streaming_variant_of_a_small_batch(group_size):
         _check(cfg, gpu, ora, x, lg, np.unique(np.array(ends, np.int32)))
 
 
-@pytest.mark.parametrize("d_model,group_size", [(256, 128), (512, 64), (768, 128)])
-def test_token_tiles_of_the_pair_kernel(d_model, group_size):
-    """Rows around its tiles (even ones of at most 256 rows, an MMA of 32 at a time) and around 128, up to where two items
-    have accumulators of their own; several items a pair of SMs, narrow and wide ones in turn; an item of two stages and one
-    of four are wholly dequantized ahead of the epilogue before them."""
+def _check_pair_tiles(**kw):
     counts = [33, 128, 129, 256, 257, 513, 160, 96]
     T = sum(counts)
-    cfg, gpu, ora = _layer(T, n_experts=8, top_k=1, group_size=group_size, d_model=d_model, d_ff=4096)
+    cfg, gpu, ora = _layer(T, n_experts=8, top_k=1, **kw)
     e = np.concatenate([np.full(c, i) for i, c in enumerate(counts)])[np.random.default_rng(7).permutation(T)]
     lg = torch.zeros((T, 8))
     lg[torch.arange(T), torch.from_numpy(e)] = 4.0
@@ -305,3 +301,20 @@ def test_token_tiles_of_the_pair_kernel(d_model, group_size):
     toks = np.concatenate([r[sorted({0, 31, 32, len(r) // 2, 127 % len(r), 128 % len(r), 159 % len(r), 160 % len(r), 255 % len(r),
                                      256 % len(r), len(r) - 1})] for r in rows])
     _check(cfg, gpu, ora, wl.activations(cfg, T, step=36), lg, toks)
+
+
+@pytest.mark.parametrize("d_model,group_size", [(256, 128), (512, 64), (768, 128)])
+def test_token_tiles_of_the_pair_kernel(d_model, group_size):
+    """Rows around its tiles (of at most 256 rows, an MMA of 32 at a time) and around 128, up to where two items have
+    accumulators of their own; 352 gate/up items for at most 74 pairs of SMs, narrow and wide ones in turn."""
+    _check_pair_tiles(d_model=d_model, d_ff=4096, group_size=group_size)
+
+
+@pytest.mark.parametrize("d_model,d_ff,group_size,cache", [(256, 4096, 64, 0), (256, 4096, 128, 0), (4096, 128, 128, 64),
+                                                           (4096, 256, 64, 64), (4096, 384, 128, 0), (4096, 384, 64, 64),
+                                                           (4096, 512, 128, 64)])
+def test_short_items_of_the_pair_kernel(d_model, d_ff, group_size, cache):
+    """Items of one, two, three and four stages, two to five of them a pair of SMs (352 gate/up items without cached channels,
+    or 176 down items): an item is wholly dequantized ahead of the epilogue before it, and stage numbers, ring offsets and
+    barrier phases run on over items that are shorter than that lead."""
+    _check_pair_tiles(d_model=d_model, d_ff=d_ff, group_size=group_size, max_sig=cache // 2, cache_size=cache)
