@@ -10,11 +10,9 @@ namespace dyn {
 
 constexpr int RB = 256;          // weight rows per packed block
 constexpr int KC = 128;          // input indices (k) per packed block
-constexpr int ATOM_ROWS = 16;    // rows of one MMA fragment tile; a block has 16 atoms
 constexpr int XROW = 288;        // bytes per (token row, k-chunk) in activation buffers:
                                  // 128 fp16 + two fp32 sums (k 0..63, 64..127) + pad; 288/4 = 72 = 8 (mod 32) banks
 constexpr int XROW_SUM_OFF = 256;
-constexpr int POOL_TILE_BYTES = 512;   // one cached channel's 8-bit-valued fp16 column for the 256 rows of a block
 constexpr int MAX_EXPERTS = 264;
 constexpr int HI_BITS = 8;
 
@@ -175,9 +173,6 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 __device__ __forceinline__ void fence_barrier_init() {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
-__device__ __forceinline__ void fence_proxy_async() {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -289,7 +284,6 @@ __device__ __forceinline__ uint32_t lds32(uint32_t a) {
 // A role's place in a byte-granular ring of stages: the offsets follow from the sizes alone, so every role computes them
 // itself.
 struct RingPos {
-    uint32_t si = 0;   // running stage number
     int head = 0;
     __device__ __forceinline__ int place(int need, int cap) {   // ring offset of a stage of `need` bytes
         const int off = head + need > cap ? 0 : head;
@@ -373,10 +367,6 @@ __device__ __forceinline__ void bulk_g2s(void* smem_dst, const void* gsrc, uint3
             smem_u32(smem_dst)),
         "l"(gsrc), "r"(bytes), "r"(smem_u32(bar))
         : "memory");
-}
-
-__device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
 // m16n8k16 fp16 x fp16 -> fp32

@@ -142,6 +142,10 @@ struct FfCycle {
         }
     }
 };
+// A role's place in the stage sequence: running stage number (slot si % FF_Q, parity (si / FF_Q) & 1) and ring offset.
+struct FfPos : RingPos {
+    uint32_t si = 0;
+};
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
     uint64_t r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
@@ -225,7 +229,7 @@ __device__ __forceinline__ void ff_store_atom(const Codes<BITS> (&cd)[2], uint32
 // One item on a warp that owns lane quarter q (two atoms) of both row tiles in the stages of parity kh.
 template <int BITS>
 __device__ __forceinline__ bool ff_expand_item(const FfItem& im, FfShared* S, uint32_t sb, uint32_t ring, int cap,
-                                               uint32_t a_lanes, int q, int kh, int lane, RingPos& pos, uint32_t& ready,
+                                               uint32_t a_lanes, int q, int kh, int lane, FfPos& pos, uint32_t& ready,
                                                int32_t* status) {
     const int n_st = im.n_main + im.n_pool;
     const int need = im.need(), need_pool = im.need_pool();
@@ -306,7 +310,7 @@ __device__ __noinline__ void ff_expand_role(const FfParams& p, FfRole R, int war
     bool ok = true;
     uint32_t ready = 0;
     int cur = 0;
-    RingPos pos;
+    FfPos pos;
     for (int g = blockIdx.x; g < R.total && ok; g += gridDim.x) {
         const FfItem im = ff_item_uni(p.ksplit, R.tab, g, cur, R.n_kc);
         switch (im.bits) {
@@ -323,7 +327,7 @@ __device__ __noinline__ void ff_expand_role(const FfParams& p, FfRole R, int war
 template <bool GATEUP, int NC, int G>
 __device__ __forceinline__ bool ff_fold_item(const FfParams& p, const FfItem& im, FfShared* S, uint32_t sb, uint32_t ring,
                                              uint8_t* htile, uint32_t acc_lanes, int q, int mt, int fw, int lane,
-                                             int ic, RingPos& pos, FfCycle<FF_NB>& acb, uint32_t& ready, bool& clamped) {
+                                             int ic, FfPos& pos, FfCycle<FF_NB>& acb, uint32_t& ready, bool& clamped) {
     constexpr int NG = KC / G;
     volatile int* poison = &S->poison;
     int32_t* status = p.ws.status;
@@ -493,7 +497,7 @@ __device__ __noinline__ void ff_fold_role(const FfParams& p, FfRole R, uint8_t* 
     FfCycle<FF_NB> acb;
     uint32_t ready = 0;
     int ic = 0, cur = 0;
-    RingPos pos;
+    FfPos pos;
     for (int g = blockIdx.x; g < R.total && ok; g += gridDim.x, ++ic) {
         const FfItem im = ff_item_uni(p.ksplit, R.tab, g, cur, R.n_kc);
         if (im.n_mma <= 16)
@@ -518,7 +522,7 @@ __device__ __noinline__ void ff_mma_role(const FfParams& p, FfRole R) {
     int32_t* status = p.ws.status;
     volatile int* poison = &S->poison;
     int cur = 0;
-    RingPos pos;
+    FfPos pos;
     // ---------------- MMA issuer: warp-uniform, one elected lane issues ----------------
     // (A stored A buffer vouches for the stage's operand tile: the expand warps waited for it.)
     bool ok = true;
@@ -650,7 +654,7 @@ __global__ void __launch_bounds__(FF_THREADS, 1) ffn_fold_kernel(const __grid_co
     const int cap = p.ring_bytes;
     const uint32_t sb = smem_u32(smem), ring_a = sb + p.off_ring;
     int cur = 0;
-    RingPos pos;
+    FfPos pos;
 
     FfRole R;
     R.S = S; R.tab = tab; R.sb = sb; R.ring = ring_a; R.tbase = tbase; R.total = total; R.n_kc = n_kc;

@@ -1,6 +1,6 @@
 // Thin inline-PTX wrappers around the 5th-generation tensor-core instructions (tcgen05) used by the
-// two tensor-core FFN kernels: fences, commit, shared-memory operand descriptors, MMA with the A operand
-// in tensor memory, and the 16x256b tensor-memory load/store shapes.
+// two tensor-core FFN kernels: fences, the pair's commit, shared-memory operand descriptors and the
+// tensor-memory load/store shapes (the MMAs themselves are issued in runs, beside their kernels).
 //
 // 16x256b register layout (lane = 4 * gid + tid4 of the issuing warp): register 4j + 0 holds (TMEM lane
 // gid, 32-bit column 8j + 2*tid4), 4j + 1 (gid, 8j + 2*tid4 + 1), 4j + 2 (gid + 8, 8j + 2*tid4),
@@ -15,21 +15,10 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
 // K-major, no swizzle: lbo = bytes between core matrices adjacent in K, sbo = between 8-row groups.
 __device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
     return (uint64_t)((addr >> 4) & 0x3fff) | ((uint64_t)((lbo >> 4) & 0x3fff) << 16) |
            ((uint64_t)((sbo >> 4) & 0x3fff) << 32) | (1ull << 46);
-}
-__device__ __forceinline__ void tc_mma_ts(uint32_t d, uint32_t a, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %5, %5, %5}, p;\n\t}" ::"r"(d),
-        "r"(a), "l"(bdesc), "r"(idesc), "r"(acc), "r"(0)
-        : "memory");
 }
 __device__ __forceinline__ void tc_st_x4(uint32_t taddr, const uint32_t (&r)[16]) {
     asm volatile(
@@ -63,24 +52,10 @@ __device__ __forceinline__ void tc_ld_x4(uint32_t taddr, uint32_t (&r)[16]) {
         : "memory");
 }
 
-// Warp-uniform forms: every lane executes them, one elected lane issues.  Operands computed in
-// warp-uniform code can then stay in uniform registers.
-__device__ __forceinline__ void tc_mma_ts_elect(uint32_t d, uint32_t a, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\telect.sync _|q, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
-        "r"(a), "l"(bdesc), "r"(idesc), "r"(acc)
-        : "memory");
-}
-__device__ __forceinline__ void tc_commit_elect(uint64_t* bar) {
-    asm volatile(
-        "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
-        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar))
-        : "memory");
-}
-// Two-CTA forms (cta_group::2): one MMA spans the tensor cores of both CTAs of a cluster, M = 256 (each CTA
-// holds 128 rows of A in its tensor memory and gets 128 rows of D), each CTA's shared memory holds N/2 rows
-// of B at the same offset; a commit can signal the barrier at one offset in both CTAs.
+// Commit of a pair of CTAs (cta_group::2), executed by a whole warp, issued by one elected lane.  One MMA of the pair spans
+// the tensor cores of both CTAs of a cluster, M = 256 (each CTA holds 128 rows of A in its tensor memory and gets 128 rows
+// of D), each CTA's shared memory holds N/2 rows of B at the same offset; the commit signals the barrier at one offset in
+// both CTAs.
 __device__ __forceinline__ void tc2_commit_both_elect(uint32_t bar) {
     asm volatile(
         "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
@@ -88,12 +63,6 @@ __device__ __forceinline__ void tc2_commit_both_elect(uint32_t bar) {
             bar),
         "h"((uint16_t)3)
         : "memory");
-}
-__device__ __forceinline__ void tc_ld_x2(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
 }
 
 // One tensor-memory lane (weight row) per lane, 16 consecutive accumulator columns
