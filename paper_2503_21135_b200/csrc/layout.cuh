@@ -22,11 +22,11 @@
 //          phi = 0, 2 at bits 0, 4 of W(jh), in place; phi = 1, 3 at bits 8, 12 after >> 6; phi = 4, 6 of jh = 0 at bits 0, 4
 //          of W2, in place, of jh = 1 at bits 8, 12 after >> 8.  phi = 5, 7 (o = 2, 6) are spread over single bits that lie
 //          four apart as the fields do, so one shift of a word serves both: bit 0 of the code at bits 11, 15 of W(jh) (>> 9),
-//          bit 1 at 3, 7 of W(jh), in place, bit 2 in W2 at 3, 7 (jh = 0, << 1) or 11, 15 (jh = 1, >> 7).  54 logical
+//          bit 1 at 3, 7 of W(jh), in place, bit 2 in W2 at 3, 7 (jh = 0) or, after >> 8, 11, 15 (jh = 1), << 1.  54 logical
 //          instructions an atom and lane (32 of them the masks that every width has); a 2-bit and a 1-bit plane take 76:
-//          1, 4, 12, 32, 64 tokens of a layer with two 3-bit experts of eight (4096 x 14336, mean of eight routers) 65, 124,
-//          169, 201, 244 us a pass, as planes 68, 128, 170, 205, 244.  Fields packed three bits apart (o = 0, 3, 6; 46
-//          instructions) take 63, 123, 166, 199, 242, but the tensor cores align the products of an MMA by the operands'
+//          1, 12, 24, 32 and 100 tokens of a layer with two 3-bit experts of eight (4096 x 14336, mean of eight routers) 65,
+//          167, 187, 201 and 261 us a pass, as planes 68, 170, 188, 206 and 269.  Fields packed three bits apart (o = 0, 3, 6;
+//          46 instructions) take 63, 165, 184, 199 and 255, but the tensor cores align the products of an MMA by the operands'
 //          exponents, and with o = 0 in three steps of four instead of two a sum over 14336 hidden activations from 0.02 to 2
 //          is twice as far from its value in 64 bits (2-norm 2.7e-5 -> 5.0e-5).
 //   4-bit: atom = 2 planes (= half chunks) x [32 lanes x 16 B]; word rowhalf*2 + (s%4)/2;
