@@ -7,12 +7,13 @@
 // tensor memory, for a tile of 256 tokens: half the dequant work per flop of the one-CTA kernel at twice
 // the tokens per MMA, so the tensor pipe, not the dequant warps, sets the pace.
 //
-// Work item of a cluster = (expert, 256-row weight block, tile of <= 256 tokens; an expert's tiles are even), K over the whole
+// Work item of a cluster = (expert, 256-row weight block, tile of <= 256 tokens; an expert's tiles are equal up to the rounding
+// to 32 rows, from eight on they are 256 and a rest), K over the whole
 // input axis; items are dealt round-robin over the clusters; rings, A buffers, accumulators live across items.
 // Per CTA (rank r = 0 leader, 1 peer), 19 warps:
 //   warp 16 weights  : ONE thread; bulk copies of the CTA's half block (codes of atoms 8r..8r+7, params of rows 128r..) into a
-//                      byte-granular ring of up to eight stages; a place comes free as soon as the stage's warps have used
-//                      its codes.
+//                      byte-granular ring of up to eight stages; a place comes free once the stage's warps have expanded
+//                      its codes (the first half of them into an A buffer, so that one has to be free).
 //   warp 18 operands : bulk copy of ITS half of the token tile (N/2 tokens: the B operand is split across the
 //                      pair) into a ring of four 32 KB slots, freed by the MMAs' commit.
 //   warps 0-15 dequant: a whole atom (16 rows x 128 k) of every OTHER stage each (eight warps per stage): packed
@@ -29,8 +30,10 @@
 // the MMA warp spent 700 on issuing with an elect per MMA and 290 on a poll; then the gap between two items, 7 to 17 thousand
 // cycles, in which every role found its next item by a chain of global loads and the epilogue stored 4-byte words over eight
 // lines.  With the issue as one run, polls asked for early, the experts' table in shared memory and 128-byte stores a stage
-// takes 865 cycles and the gap 6 thousand: 500 tokens 492 -> 416 us a pass, 1000 (skewed) 802 -> 711, 4096 2467 -> 2348,
-// 2048 fine-grained 465 -> 435.  What is left is the epilogue (5 thousand cycles an item) and the dequant warps' latencies.
+// takes 865 cycles and the gap 6 to 7 thousand.  us a pass of the whole layer, passes back to back under the power cap, before
+// and now: 500 tokens 548 -> 487, 1000 (skewed) 924 -> 842, 4096 2766 -> 2630, 2048 fine-grained 486 -> 461; short bursts at full
+// clock, in which the variants below were compared: 500 tokens 492 -> 416, 4096 2467 -> 2348.  What is left is the epilogue (5
+// thousand cycles an item) and the dequant warps' latencies.
 // Every wait is bounded; after an expired wait a CTA leaves its loops and meets its peer at the final
 // cluster barrier (the peer's own waits expire within the same bound).
 #include <cstddef>
@@ -54,7 +57,7 @@ constexpr int T2_POOL_XG = 16 * 512;                              // ... and the
 static_assert(T2_POOL_TILES <= T2_WHALF_MAX && T2_POOL_XG <= T2_XTILE, "cached-channel stage does not fit its slots");
 // Two rings.  The operand tiles (32 KB slots, read by the MMAs) are freed by the MMAs' commit; the packed weights (read
 // only by the dequant warps) lie in a byte-granular ring, up to eight stages of it (four of 8-bit codes), whose places
-// come free as soon as the codes are in registers.
+// come free once the codes are expanded, behind the wait for the stage's A buffer.
 constexpr int T2_NW = 8;
 constexpr int T2_NX = 4;
 constexpr int T2_WRING = 4 * T2_WHALF_MAX;
@@ -78,7 +81,7 @@ struct T2Params {
 };
 
 struct T2Bars {
-    uint64_t full[T2_NW], empty[T2_NW];    // per CTA: weight bytes landed / the stage's 8 dequant warps hold the codes
+    uint64_t full[T2_NW], empty[T2_NW];    // per CTA: weight bytes landed / the stage's 8 dequant warps have expanded the codes
     uint64_t fullx[T2_NX];               // per CTA: operand bytes landed
     uint64_t a_full[T2_NA];              // leader only: the 16 dequant warps of the pair that own the stage stored A buffer b
     uint64_t done[T2_NA];                // per CTA: the stage's MMAs are complete (commit): A buffer and operand slot are free
@@ -458,8 +461,8 @@ __device__ __noinline__ void t2_dequant_role(const T2Params& p, uint8_t* smem, u
     int head = 0;
     // The first stages of the NEXT item are dequantized before this item's epilogue: their A buffers come free while the last
     // MMAs of this item run.  Where both items have accumulators of their own all four buffers are filled, and the MMAs run on
-    // through the epilogue; otherwise three, since the fourth comes free only with the last MMA (4096 tokens: 2405 us a pass
-    // with two, 2348 with three, 2372 with four).
+    // through the epilogue; otherwise three, since the fourth comes free only with the last MMA (4096 tokens, short bursts: 2405 us
+    // a pass with two, 2348 with three, 2372 with four).
     int lead_done = 0;                       // stages of the item already dequantized (as the previous item's lead)
     for (int g = cluster_id; g < total && ok; g += n_clusters, ++ic) {
         int bits, from = lead_done, to, bits_nx = 0;
@@ -541,7 +544,7 @@ __device__ __forceinline__ void tc2_cta(const T2Params& p, uint8_t* smem, bool f
         t.cnt = p.ws.counts[e];
         if (t.cnt <= p.ws.tc_min) t.cnt = 0;
         t.n_tt = (t.cnt + T2_N - 1) / T2_N;
-        t.rows = t.n_tt > 0 ? ((t.cnt + t.n_tt - 1) / t.n_tt + 31) & ~31 : 0;   // even tiles: a narrow one costs its dequantization all the same
+        t.rows = t.n_tt > 0 ? ((t.cnt + t.n_tt - 1) / t.n_tt + 31) & ~31 : 0;   // equal tiles: a narrow one costs its dequantization all the same
         t.first = t.n_tt * p.n_rb;
         t.row0 = p.ws.off_pad[e];
         t.bits = ex.bits;
