@@ -31,7 +31,7 @@
 // cycles, in which every role found its next item by a chain of global loads and the epilogue stored 4-byte words over eight
 // lines.  With the issue as one run, polls asked for early, the experts' table in shared memory and 128-byte stores a stage
 // takes 865 cycles and the gap 6 to 7 thousand.  us a pass of the whole layer, passes back to back under the power cap, before
-// and now: 500 tokens 548 -> 487, 1000 (skewed) 924 -> 842, 4096 2766 -> 2630, 2048 fine-grained 486 -> 461; short bursts at full
+// and now: 500 tokens 542 -> 479, 1000 (skewed) 904 -> 834, 4096 2719 -> 2590, 2048 fine-grained 476 -> 451; short bursts at full
 // clock, in which the variants below were compared: 500 tokens 492 -> 416, 4096 2467 -> 2348.  What is left is the epilogue (5
 // thousand cycles an item) and the dequant warps' latencies.
 // Every wait is bounded; after an expired wait a CTA leaves its loops and meets its peer at the final
